@@ -114,8 +114,11 @@ enum {
   ISING_ENGINE_PERSISTENT = 2, /* one cooperative launch per anneal call, bounded grid barrier;
                                   deterministic anneals of a graph with int8 weights and at most
                                   4095 vertices (at most 1024 colours and 4M CSR entries) run in
-                                  one block instead: block barriers between classes, the packed
-                                  adjacency streamed by bulk copies */
+                                  one block or one cluster of blocks instead, each with a map of
+                                  every spin in shared memory. What AUTO runs as PERSISTENT takes
+                                  that spin-map form too (on every SM where a class has enough
+                                  work) for deterministic anneals of graphs of up to 204,800
+                                  vertices and 4096 neighbours a vertex */
   ISING_ENGINE_DATAFLOW = 3,   /* one cooperative launch per anneal call without barriers: each
                                   neighbour read waits (bounded) until the neighbour carries the
                                   update the colour order requires; racy mode runs as PERSISTENT */
@@ -125,7 +128,9 @@ enum {
                                   rows' neighbours to finish the sweep the colour order requires
                                   (per-item counters, release/acquire); for graphs whose rows
                                   are not sliced across warps, deterministic linear schedule;
-                                  otherwise runs as PERSISTENT_GRID */
+                                  otherwise runs as PERSISTENT_GRID. Such graphs of up to 204,800
+                                  vertices run in the spin-map form instead (a lattice larger
+                                  than 100,000 vertices does not) */
   ISING_ENGINE_HALO = 7,       /* one cooperative launch per anneal call, one block per SM: the
                                   graph is cut into one part per block (recursive breadth-first
                                   bisection); a block keeps every vertex within D = S * K hops of
@@ -558,7 +563,8 @@ int ising_engine_used(ising_graph* g, int32_t* out);
  * latches it in the handle (create a new handle to continue; the CUDA
  * context stays usable). Kinds:
  *   ISING_FAULT_SKIP_ARRIVAL  persistent grid engine: block 0 skips its first
- *                             grid-barrier arrival, so every block's wait runs out;
+ *                             grid-barrier arrival, so every block's wait runs out
+ *                             (spin-map form: block 0 publishes no spins);
  *   ISING_FAULT_SHORT_COPY    block engine: the first chunk's barrier expects 16
  *                             bytes that never arrive, so its wait runs out.
  * wait_budget_ns bounds every wait of later anneal calls (0: the default; at

@@ -18,7 +18,8 @@
 // f_i = sum_j w_ij s_j of its rows (Eq. 2), then the update rule and the
 // random flip of Algorithm 2. The engines differ in how a colour class waits
 // for the previous one: a launch per class, a grid barrier, per-neighbour or
-// per-item dataflow waits, or block barriers for small graphs.
+// per-item dataflow waits, block barriers for small graphs, or the spin maps of
+// map.cuh.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -38,6 +39,7 @@
 #include "graph_handle.h"
 #include "halo.cuh"
 #include "hub.cuh"
+#include "map.cuh"
 
 using isingx::HostGraph;
 using isingx::PhiloxKey;
@@ -234,111 +236,6 @@ __global__ void __launch_bounds__(kPersistBlock, 2)
   }
 }
 
-// Small graphs whose whole packed CSR fits in one block's shared memory (the
-// 800-vertex workload: 38k entries, 160 KB): one block of 1024 threads holds
-// the row offsets, the entries, every state byte and the sweep's flips, for
-// the whole anneal call. A class is one pass in which 16 lanes share a row
-// (its entries strided over them, four in flight per lane, four shuffles to
-// combine) and the row's
-// first lane decides it at once, then one block barrier. The state bytes go
-// back to global memory at the end of the call. Deterministic linear
-// schedule (flip bias allowed); the spins equal one grid phase per class.
-constexpr int kCsrBlockThreads = 1024;
-constexpr int kCsrRowLanes = 16;
-
-struct CsrBlockLayout {
-  int rp, adj, cls, state, flip, total;
-};
-
-__host__ __device__ inline CsrBlockLayout csr_block_layout(int n, long long nnz, int ncls) {
-  CsrBlockLayout L{};
-  long long o = 0;
-  L.rp = 0;
-  o += 4LL * (n + 1);
-  L.adj = static_cast<int>((o + 15) & ~15LL);
-  o = L.adj + 4LL * nnz;
-  L.cls = static_cast<int>(o);
-  o += 4LL * (ncls + 1);
-  L.state = static_cast<int>(o);
-  o += n + 1;  // one spare state byte (spin +1) for a padding column
-  L.flip = static_cast<int>(o);
-  o += n;
-  o = (o + 15) & ~15LL;
-  L.total = o > 0x7fffffffLL ? 0x7fffffff : static_cast<int>(o);
-  return L;
-}
-
-__global__ void __launch_bounds__(kCsrBlockThreads, 1)
-    csr_block_kernel(DevGraph d, int n, int nnz, int ncls, const int32_t* __restrict__ class_pos,
-                     uint64_t t_begin, uint32_t sweeps, uint64_t T, uint64_t T0, uint32_t replica,
-                     isingx::PhiloxRounds rk) {
-  extern __shared__ __align__(16) unsigned char csr_mem[];
-  const CsrBlockLayout L = csr_block_layout(n, nnz, ncls);
-  int32_t* rp = reinterpret_cast<int32_t*>(csr_mem + L.rp);
-  int32_t* adj = reinterpret_cast<int32_t*>(csr_mem + L.adj);
-  int32_t* cls = reinterpret_cast<int32_t*>(csr_mem + L.cls);
-  uint8_t* state = csr_mem + L.state;
-  uint8_t* flip = csr_mem + L.flip;
-  const int tid = threadIdx.x;
-  for (int i = tid; i <= n; i += kCsrBlockThreads) rp[i] = __ldg(d.row_ptr + i);
-  for (int i = tid; i < nnz; i += kCsrBlockThreads) adj[i] = __ldg(d.adj + i);
-  for (int i = tid; i <= ncls; i += kCsrBlockThreads) cls[i] = __ldg(class_pos + i);
-  for (int i = tid; i < n; i += kCsrBlockThreads) state[i] = static_cast<uint8_t>(d.spins[i]);
-  if (tid == 0) state[n] = 0;
-  const int q = tid % kCsrRowLanes;                  // lane within the row's group
-  const int grp = tid / kCsrRowLanes;                // row group
-  const int ngrp = kCsrBlockThreads / kCsrRowLanes;
-  __syncthreads();
-  for (uint32_t k = 0; k < sweeps; ++k) {
-    const SweepArgs a = sweep_args(t_begin + k, T, T0, replica);
-    for (int i = tid; i < n; i += kCsrBlockThreads)
-      flip[i] = flip_drawn(d, i, static_cast<uint32_t>(__ldg(d.orig + i)), a, rk) ? 1 : 0;
-    __syncthreads();
-    for (int c = 0; c < ncls; ++c) {
-      const int ce = cls[c + 1];
-      for (int r0 = cls[c]; r0 < ce; r0 += ngrp) {
-        const int r = r0 + grp;
-        int f = 0;
-        if (r < ce) {
-          const int e1 = rp[r + 1];
-          int e = rp[r] + q;
-          for (; e + 3 * kCsrRowLanes < e1; e += 4 * kCsrRowLanes) {
-            uint32_t x[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = static_cast<uint32_t>(adj[e + u * kCsrRowLanes]);
-            int sp[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) sp[u] = state[x[u] >> 8];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-              f += static_cast<int>(static_cast<int8_t>(static_cast<uint8_t>(x[u] & 0xffu))) * isingx::spin_of(sp[u]);
-          }
-          for (; e < e1; e += kCsrRowLanes) {
-            const uint32_t x = static_cast<uint32_t>(adj[e]);
-            const int w = static_cast<int>(static_cast<int8_t>(static_cast<uint8_t>(x & 0xffu)));
-            f += w * isingx::spin_of(state[x >> 8]);
-          }
-        }
-        // every lane of the warp reaches the shuffles (r0 is uniform)
-#pragma unroll
-        for (int o = 1; o < kCsrRowLanes; o <<= 1) f += __shfl_xor_sync(isingx::kFullMask, f, o, kCsrRowLanes);
-        if (r < ce && q == 0) {
-          const int bt = state[r];
-          int sv = isingx::spin_of(bt);
-          if (f > 0)
-            sv = -1;
-          else if (f < 0)
-            sv = 1;
-          if (flip[r]) sv = -sv;
-          state[r] = static_cast<uint8_t>(isingx::state_byte(sv, ((bt >> 1) & 1) ^ 1));
-        }
-      }
-      __syncthreads();
-    }
-  }
-  for (int i = tid; i < n; i += kCsrBlockThreads) d.spins[i] = static_cast<int8_t>(state[i]);
-}
-
 // Block engine (block.cuh): a graph of at most 4095 vertices, every sweep of
 // an anneal call in one block; deterministic pass, with Algorithm 1's flips
 // after each sweep when nflip0 > 0.
@@ -353,10 +250,7 @@ __global__ void __launch_bounds__(isingx::kBlockThreads)
   unsigned seq = 0;
   for (uint32_t k = 0; k < sweeps; ++k) {
     const SweepArgs a = sweep_args(t_begin + k, T, T0, replica);
-    if (ba.resident_words > 0)
-      isingx::block_sweep_resident(d, ba, a, rk, sh);
-    else if (!isingx::block_sweep(d, ba, a, rk, sh, seq))
-      return;
+    if (!isingx::block_sweep(d, ba, a, rk, sh, seq)) return;
     if (nflip0 != 0u) {
       // the sweep's updates are in global memory; warp 0 flips N_t spins
       const uint32_t N = isingx::nflip_count(nflip0, T, t_begin + k);
@@ -551,7 +445,10 @@ void free_device(ising_graph* g) {
                   g->d_halo_imports, g->d_halo_nbrs, g->d_halo_exports, g->d_halo_quads, g->d_halo_flags,
                   g->d_spins2, g->d_hub_split, g->d_hub_end, g->d_hub_sums, g->d_hub_acc,
                   g->d_hub_flips, g->d_hub_bits, g->d_hub_pflips, g->d_hub_blk,
-                  g->d_gnn_hchunk, g->d_gnn_chunk_row};
+                  g->d_gnn_hchunk, g->d_gnn_chunk_row, g->d_map_blocks, g->d_map_task,
+                  g->d_map_words, g->d_map_weights, g->d_map_row_pos, g->d_map_row_orig,
+                  g->d_map_class, g->d_map_steps, g->d_map_msg, g->d_map_index, g->d_map_mail,
+                  g->d_pick_count, g->d_picks};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }
@@ -718,31 +615,7 @@ cudaError_t launch_block(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint
   ba.class_pos = g->d_class_begin;
   ba.wait_ns = static_cast<long long>(g->wait_budget_ns);
   ba.short_copy = g->fault_kind == ISING_FAULT_SHORT_COPY ? 1 : 0;
-  int optin = 0;
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device);
-  // the whole packed CSR in shared memory (linear schedule; not under the
-  // short-copy test, which needs the copies)
-  if (g->packed && nflip0 == 0u && !ba.short_copy && g->nnz < (1LL << 30)) {
-    const int csr_smem = csr_block_layout(g->n, g->nnz, g->num_colours).total;
-    if (csr_smem <= optin) {
-      cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(csr_block_kernel),
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, csr_smem);
-      if (e != cudaSuccess) return e;
-      g->launches++;
-      csr_block_kernel<<<1, kCsrBlockThreads, csr_smem, g->stream>>>(
-          g->dev(), g->n, static_cast<int>(g->nnz), g->num_colours, g->d_class_begin, t_begin, sweeps, T, T0,
-          replica, rk);
-      return cudaGetLastError();
-    }
-  }
-  // every word resident in shared memory when it fits (not under the
-  // short-copy test, which needs the copies)
-  const int words = g->block_num_words;
-  ba.resident_words = 0;
-  if (!ba.short_copy && words > 0 &&
-      isingx::block_layout(ba.n, ba.num_chunks, ba.num_classes, words).total <= optin)
-    ba.resident_words = words;
-  const int smem = isingx::block_layout(ba.n, ba.num_chunks, ba.num_classes, ba.resident_words).total;
+  const int smem = isingx::block_layout(ba.n, ba.num_chunks, ba.num_classes).total;
   cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(block_kernel),
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
@@ -1019,6 +892,236 @@ cudaError_t launch_hub(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint64
                : launch_hub_t<false, false>(g, t_begin, sweeps, T, T0, replica, rk);
 }
 
+// The spin-map engine (map.cuh) on the handle's plan.
+template <int MODE>
+const void* map_kernel_of(bool wide, int stage) {
+  using isingx::map_kernel;
+  if (wide) return stage <= 2 ? reinterpret_cast<const void*>(map_kernel<MODE, true, 2>)
+                              : reinterpret_cast<const void*>(map_kernel<MODE, true, 4>);
+  if (stage <= 1) return reinterpret_cast<const void*>(map_kernel<MODE, false, 1>);
+  if (stage <= 2) return reinterpret_cast<const void*>(map_kernel<MODE, false, 2>);
+  if (stage <= 4) return reinterpret_cast<const void*>(map_kernel<MODE, false, 4>);
+  return reinterpret_cast<const void*>(map_kernel<MODE, false, 8>);
+}
+
+const void* map_kernel_for(int mode, bool wide, int stage) {
+  if (mode == isingx::kMapBlock) return map_kernel_of<isingx::kMapBlock>(wide, stage);
+  if (mode == isingx::kMapBlockStream) return map_kernel_of<isingx::kMapBlockStream>(wide, stage);
+  if (mode == isingx::kMapCluster) return map_kernel_of<isingx::kMapCluster>(wide, stage);
+  return map_kernel_of<isingx::kMapGrid>(wide, stage);
+}
+
+void map_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int mode, int K, int warps, int smem, cudaStream_t s) {
+  *cfg = cudaLaunchConfig_t{};
+  cfg->gridDim = dim3(K);
+  cfg->blockDim = dim3(32 * warps);
+  cfg->dynamicSmemBytes = static_cast<size_t>(smem);
+  cfg->stream = s;
+  if (mode <= isingx::kMapBlockStream) return;
+  if (mode == isingx::kMapCluster) {
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = K;
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  } else {
+    attr->id = cudaLaunchAttributeCooperative;
+    attr->val.cooperative = 1;
+  }
+  cfg->attrs = attr;
+  cfg->numAttrs = 1;
+}
+
+// Whether the device can run a plan: shared memory, a cluster of that size, or
+// K co-resident blocks.
+bool map_fits(const isingx::MapPlan& mp, bool wide) {
+  const void* kernel = map_kernel_for(mp.mode, wide, mp.stage);
+  bool fits = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, mp.smem_bytes) == cudaSuccess;
+  if (fits && mp.mode == isingx::kMapCluster) {
+    fits = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    map_config(&cfg, &attr, mp.mode, mp.K, mp.warps, mp.smem_bytes, nullptr);
+    int clusters = 0;
+    fits = fits && cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters >= 1;
+  } else if (fits && mp.mode == isingx::kMapGrid) {
+    int per_sm = 0, sms = 0, dev = 0, coop = 0;
+    fits = cudaGetDevice(&dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop != 0 &&
+           cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * mp.warps,
+                                                         static_cast<size_t>(mp.smem_bytes)) == cudaSuccess &&
+           per_sm * sms >= mp.K;
+  }
+  cudaGetLastError();
+  return fits;
+}
+
+// The plan a graph gets, by the work of a class: its entries, and eight for
+// each of its rows (decision, draw, publication). Up to 4,000 one block is
+// fastest: no exchange (a 1000-vertex, 10,000-edge graph takes 4.1 us a sweep
+// on one block and 5.6 on the cluster; 2000 vertices and 20,000 edges, 5,600
+// a class, 5.8 and 5.0). Up to 300,000 a class the 16 blocks of a cluster, whose
+// exchange costs 0.3 us (70,000 vertices and 2.1M edges, 227,000 a class: 39 us
+// against 42 on the grid); beyond that, every SM and its 1.3 us exchange
+// (100,000 vertices and 5M edges, 360,000 a class: 84 against 62 us). Lattices
+// wait for a halo plan: until then the cluster up to 100,000 vertices (9.8
+// against 11.6 us by item dataflow at 90,300, 14.3 against 13.3 at 160,000).
+void choose_map_plan(const HostGraph& hg, int num_sms, int device, bool wide, bool lattice,
+                     isingx::MapPlan* mp) {
+  int optin = 0;
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+  const int64_t work = hg.nnz + 8 * static_cast<int64_t>(hg.n), classes = std::max(1, hg.num_colours);
+  auto build = [&](int mode, int K) {
+    isingx::build_map_plan(hg, mode, K, wide, optin, mp);
+    return mp->ok && map_fits(*mp, wide);
+  };
+  if (work <= 4000 * classes && (build(isingx::kMapBlock, 1) || build(isingx::kMapBlockStream, 1))) return;
+  if ((lattice ? hg.n <= 100000 : work <= 300000 * classes) &&
+      (build(isingx::kMapCluster, 16) || build(isingx::kMapCluster, 8)))
+    return;
+  if (!lattice && build(isingx::kMapGrid, std::min(num_sms, std::max(1, hg.n / 32)))) return;
+  mp->ok = false;
+}
+
+cudaError_t upload_map_plan(ising_graph* g, const isingx::MapPlan& mp) {
+  cudaError_t e;
+  if ((e = alloc_copy(&g->d_map_blocks, mp.blocks.data(), mp.blocks.size(), g->stream)) != cudaSuccess) return e;
+  if ((e = alloc_copy(&g->d_map_task, mp.tasks.data(), mp.tasks.size(), g->stream)) != cudaSuccess) return e;
+  const size_t entry_bytes = std::max<size_t>(16, static_cast<size_t>(mp.total_groups) * 512);
+  if ((e = cudaMalloc(reinterpret_cast<void**>(&g->d_map_words), entry_bytes)) != cudaSuccess) return e;
+  if (!g->packed && (e = cudaMalloc(reinterpret_cast<void**>(&g->d_map_weights), entry_bytes)) != cudaSuccess) return e;
+  if ((e = alloc_copy(&g->d_map_row_pos, mp.row_pos.data(), mp.row_pos.size(), g->stream)) != cudaSuccess) return e;
+  if ((e = alloc_copy(&g->d_map_row_orig, mp.row_orig.data(), mp.row_orig.size(), g->stream)) != cudaSuccess) return e;
+  const size_t KC = mp.class_row.size(), C1 = mp.class_bytes.size();
+  if ((e = alloc_copy<int32_t>(&g->d_map_class, nullptr, 3 * KC, g->stream)) != cudaSuccess) return e;
+  const std::vector<int32_t>* tables[3] = {&mp.class_row, &mp.class_seg, &mp.block_msg};
+  for (int i = 0; i < 3; ++i)
+    if ((e = cudaMemcpyAsync(g->d_map_class + i * KC, tables[i]->data(), KC * sizeof(int32_t),
+                             cudaMemcpyHostToDevice, g->stream)) != cudaSuccess)
+      return e;
+  if ((e = alloc_copy<int32_t>(&g->d_map_steps, nullptr, 2 * C1, g->stream)) != cudaSuccess) return e;
+  if ((e = cudaMemcpyAsync(g->d_map_steps, mp.class_bytes.data(), C1 * sizeof(int32_t), cudaMemcpyHostToDevice,
+                           g->stream)) != cudaSuccess)
+    return e;
+  if ((e = cudaMemcpyAsync(g->d_map_steps + C1, mp.class_msg.data(), C1 * sizeof(int32_t), cudaMemcpyHostToDevice,
+                           g->stream)) != cudaSuccess)
+    return e;
+  if ((e = alloc_copy(&g->d_map_msg, mp.msg.data(), mp.msg.size(), g->stream)) != cudaSuccess) return e;
+  if ((e = alloc_copy(&g->d_map_index, mp.map_index.data(), mp.map_index.size(), g->stream)) != cudaSuccess) return e;
+  if ((e = alloc_copy<unsigned long long>(&g->d_map_mail, nullptr,
+                                           2 * static_cast<size_t>(mp.K) * static_cast<size_t>(mp.mail_stride), g->stream)) != cudaSuccess)
+    return e;
+  const dim3 grid(static_cast<unsigned>(mp.K), mp.mode == isingx::kMapGrid ? 4u : 32u);
+  if (g->packed)
+    isingx::map_fill_kernel<true><<<grid, 256, 0, g->stream>>>(
+        g->dev(), g->d_map_blocks, reinterpret_cast<const int4*>(g->d_map_task), mp.warps, g->d_map_row_pos,
+        g->d_map_index, reinterpret_cast<int4*>(g->d_map_words), nullptr);
+  else
+    isingx::map_fill_kernel<false><<<grid, 256, 0, g->stream>>>(
+        g->dev(), g->d_map_blocks, reinterpret_cast<const int4*>(g->d_map_task), mp.warps, g->d_map_row_pos,
+        g->d_map_index, reinterpret_cast<int4*>(g->d_map_words), reinterpret_cast<int4*>(g->d_map_weights));
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  g->map_mode = mp.mode;
+  g->map_K = mp.K;
+  g->map_smem = mp.smem_bytes;
+  g->map_bytes = mp.map_bytes;
+  g->map_warps = mp.warps;
+  g->map_tasks = mp.max_tasks;
+  g->map_rows = mp.max_rows;
+  g->map_groups = mp.max_groups;
+  g->map_stage = mp.stage;
+  g->map_stride = mp.mail_stride;
+  g->map_ok = true;
+  return cudaSuccess;
+}
+
+cudaError_t launch_map(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint64_t T, uint64_t T0,
+                       uint32_t replica, const isingx::PhiloxRounds& rk, uint32_t n0, int par0) {
+  const bool wide = !g->packed;
+  const void* kernel = map_kernel_for(g->map_mode, wide, g->map_stage);
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, g->map_smem);
+  if (e != cudaSuccess) return e;
+  if (g->map_mode == isingx::kMapCluster &&
+      (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
+    return e;
+  const size_t KC = static_cast<size_t>(g->map_K) * (static_cast<size_t>(g->num_colours) + 1);
+  isingx::MapArgs a{};
+  a.blocks = g->d_map_blocks;
+  a.tasks = reinterpret_cast<const int4*>(g->d_map_task);
+  a.words = reinterpret_cast<const int4*>(g->d_map_words);
+  a.weights = reinterpret_cast<const int4*>(g->d_map_weights);
+  a.row_pos = g->d_map_row_pos;
+  a.row_orig = g->d_map_row_orig;
+  a.class_row = g->d_map_class;
+  a.class_seg = g->d_map_class + KC;
+  a.block_msg = g->d_map_class + 2 * KC;
+  a.class_bytes = g->d_map_steps;
+  a.class_msg = g->d_map_steps + g->num_colours + 1;
+  a.msg = g->d_map_msg;
+  a.map_index = g->d_map_index;
+  a.mail = g->d_map_mail;
+  a.mail_stride = g->map_stride;
+  a.n = g->n;
+  a.classes = g->num_colours;
+  a.map_bytes = g->map_bytes;
+  a.tasks_max = g->map_tasks;
+  a.rows_max = g->map_rows;
+  a.groups_max = g->map_groups;
+  a.budget = g->wait_budget_ns > 0 ? static_cast<long long>(g->wait_budget_ns) : isingx::kBarrierBudgetNs;
+  a.error = &g->d_barrier->error;
+  a.skip_block = g->fault_kind == ISING_FAULT_SKIP_ARRIVAL ? 1 : 0;
+  // Algorithm 1: the picks of as many sweeps as kPickInts holds, then those
+  // sweeps, and so on
+  constexpr size_t kPickInts = size_t(1) << 22;
+  size_t chunk = sweeps;
+  if (n0 != 0u) {
+    chunk = std::min<size_t>(sweeps, std::max<size_t>(1, kPickInts / n0));
+    if (chunk > g->pick_sweeps || chunk * n0 > g->pick_cap) {
+      cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+      if ((e = cudaStreamIsCapturing(g->stream, &capture)) != cudaSuccess) return e;
+      if (capture != cudaStreamCaptureStatusNone) return cudaErrorMemoryAllocation;
+      if ((e = cudaStreamSynchronize(g->stream)) != cudaSuccess) return e;
+      cudaFree(g->d_pick_count);
+      cudaFree(g->d_picks);
+      g->d_pick_count = nullptr;
+      g->d_picks = nullptr;
+      g->pick_sweeps = g->pick_cap = 0;
+      if ((e = cudaMalloc(reinterpret_cast<void**>(&g->d_pick_count), chunk * sizeof(uint32_t))) != cudaSuccess) return e;
+      if ((e = cudaMalloc(reinterpret_cast<void**>(&g->d_picks), chunk * n0 * sizeof(int32_t))) != cudaSuccess) return e;
+      g->pick_sweeps = chunk;
+      g->pick_cap = chunk * n0;
+    }
+    a.pick_count = g->d_pick_count;
+    a.picks = g->d_picks;
+    a.pick_stride = static_cast<int32_t>(n0);
+  }
+  DevGraph d = g->dev();
+  isingx::PhiloxRounds rounds = rk;
+  for (uint64_t done = 0; done < sweeps; done += chunk) {
+    uint32_t now = static_cast<uint32_t>(std::min<uint64_t>(chunk, sweeps - done));
+    uint64_t t = t_begin + done;
+    a.par_end = par0 ^ static_cast<int>((done + now) & 1u);
+    if (n0 != 0u) {
+      g->launches++;
+      isingx::map_picks_kernel<<<now, 32, static_cast<size_t>(g->n + 31) / 32 * 4, g->stream>>>(
+          g->n, t, T, n0, replica, rk, g->d_pos, g->d_map_index, g->d_pick_count, g->d_picks, a.pick_stride);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    if (g->map_mode == isingx::kMapGrid &&
+        (e = cudaMemsetAsync(g->d_map_mail, 0,
+                             2 * sizeof(unsigned long long) * static_cast<size_t>(g->map_K) *
+                                 static_cast<size_t>(g->map_stride),
+                             g->stream)) != cudaSuccess)
+      return e;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    map_config(&cfg, &attr, g->map_mode, g->map_K, g->map_warps, g->map_smem, g->stream);
+    void* args[] = {&d, &a, &t, &now, &T, &T0, &replica, &rounds};
+    g->launches++;
+    if ((e = cudaLaunchKernelExC(&cfg, kernel, args)) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 // The non-hub classes' work split for G blocks (block 0 runs the hub
 // classes): per class, G item offsets; worker block b takes items
 // [blk[b], blk[b + 1]) of the class, a contiguous range of about equal
@@ -1200,19 +1303,23 @@ int ising_create(int32_t n, int64_t m, const int32_t* src, const int32_t* dst, c
     }
   }
   isingx::BlockPlan block;
+  isingx::MapPlan map_plan;
   std::vector<int32_t> dep_ptr, deps;  // item dependencies (before the columns are packed)
   bool have_deps = false;
   std::vector<int32_t> packed_words;  // graphs kept for the halo plan pack into a copy
+  bool keep_host = false;
   try {
     if (g->packed) isingx::build_block_plan(hg, &block);
-    have_deps = isingx::build_item_deps(hg, plan, &dep_ptr, &deps);
+    // graphs the halo engine may take keep their host graph for its plan
+    keep_host = g->packed && !block.ok && hg.num_colours <= isingx::kHaloMaxClasses &&
+                hg.max_degree <= isingx::kHaloMaxWidth && hg.n >= 64 * g->num_sms;
+    // small graphs and graphs without hubs: the spin-map engine
+    if (block.ok || hub_end.empty()) choose_map_plan(hg, g->num_sms, g->device, !g->packed, keep_host, &map_plan);
+    if (!map_plan.ok) have_deps = isingx::build_item_deps(hg, plan, &dep_ptr, &deps);
   } catch (const std::bad_alloc&) {
     delete g;
     return ISING_ENOMEM;
   }
-  // graphs the halo engine may take keep their host graph for its plan
-  const bool keep_host = g->packed && !block.ok && hg.num_colours <= isingx::kHaloMaxClasses &&
-                         hg.max_degree <= isingx::kHaloMaxWidth && hg.n >= 64 * g->num_sms;
 
   cudaError_t e = cudaSuccess;
   const size_t N = static_cast<size_t>(hg.n);
@@ -1293,8 +1400,8 @@ int ising_create(int32_t n, int64_t m, const int32_t* src, const int32_t* dst, c
                           g->stream)) != cudaSuccess) break;
       g->block_ok = true;
       g->block_num_chunks = static_cast<int32_t>(block.chunk_off.size());
-      g->block_num_words = static_cast<int32_t>(block.words.size());
     }
+    if (map_plan.ok && (e = upload_map_plan(g, map_plan)) != cudaSuccess) break;
     if (!hub_end.empty()) {
       const size_t X = hub_end.size();
       if ((e = alloc_copy(&g->d_hub_split, hub_split.data(), X, g->stream)) != cudaSuccess) break;
@@ -1455,6 +1562,7 @@ static int anneal_impl(ising_graph* g, const ising_schedule* sched, uint32_t swe
   const isingx::PhiloxRounds rk = isingx::philox_rounds(isingx::philox_key(seed, 0u));
   // AUTO: the persistent engine when the device supports cooperative launches.
   int engine = g->engine;
+  const bool unsliced = g->num_slots == 0;
   if (engine == ISING_ENGINE_AUTO) {
     int coop = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, g->device);
@@ -1473,7 +1581,7 @@ static int anneal_impl(ising_graph* g, const ising_schedule* sched, uint32_t swe
       if (g->halo_state == 1 && g->halo_ratio <= kHaloAutoRatio)
         engine = ISING_ENGINE_HALO;
       else
-        engine = g->itemflow_ok ? ISING_ENGINE_ITEMFLOW : ISING_ENGINE_PERSISTENT;
+        engine = unsliced ? ISING_ENGINE_ITEMFLOW : ISING_ENGINE_PERSISTENT;
     } else {
       engine = ISING_ENGINE_PERSISTENT;
     }
@@ -1513,6 +1621,20 @@ static int anneal_impl(ising_graph* g, const ising_schedule* sched, uint32_t swe
       }
     }
     engine = ISING_ENGINE_ITEMFLOW;  // racy, N-flip or no plan
+  }
+  // the spin-map form of the block engine, of the item-dataflow engine and of
+  // what AUTO runs as PERSISTENT
+  const bool use_map = g->map_ok && mode == ISING_MODE_DET && g->fault_kind != ISING_FAULT_SHORT_COPY &&
+                       (engine == ISING_ENGINE_ITEMFLOW ||
+                        (engine == ISING_ENGINE_PERSISTENT && (g->block_ok || g->engine == ISING_ENGINE_AUTO)));
+  if (use_map && !(engine == ISING_ENGINE_ITEMFLOW && (nflip || !unsliced))) {
+    g->engine_used = engine == ISING_ENGINE_ITEMFLOW ? ISING_ENGINE_ITEMFLOW
+                     : g->block_ok                   ? ISING_ENGINE_USED_BLOCK
+                                                     : ISING_ENGINE_PERSISTENT_GRID;
+    const cudaError_t e = launch_map(g, sched->t_begin, sweeps, sched->t_total, T0, sched->replica, rk, n0, par0);
+    if (e == cudaSuccess) return ISING_OK;
+    if (e != cudaErrorMemoryAllocation) return cuda_fail(g, e);
+    cudaGetLastError();  // no room for Algorithm 1's picks: an engine that draws them as it goes
   }
   if (engine == ISING_ENGINE_ITEMFLOW) {
     if (mode == ISING_MODE_DET && !nflip && g->itemflow_ok) {

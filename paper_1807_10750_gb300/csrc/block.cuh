@@ -12,10 +12,9 @@
 // class applies Eq. 2 and Algorithm 2's flip exactly as the grid engines do.
 // The spins are identical to a sweep of one grid phase per class.
 //
-// When every packed word fits in shared memory with the tables (the
-// 800-vertex workload's 38k words take 154 KB), the block loads them once per
-// launch instead (resident form): no copies, no waits, and a class costs two
-// block barriers.
+// It runs the small graphs that the spin-map engine (map.cuh) has no plan for:
+// near-cliques of several hundred colours, whose per-class tables exceed a
+// block's shared memory.
 #pragma once
 
 #include <cstdint>
@@ -37,7 +36,6 @@ struct BlockArgs {
   const int32_t* class_pos;     // per class + 1: first position
   long long wait_ns;            // bound of every wait (0: kBlockWaitNs)
   int short_copy;               // failure-detection tests: the first chunk expects 16 more bytes
-  int resident_words;           // > 0: every word is kept in shared memory (that many words)
 };
 
 constexpr int kBlockThreads = 512;
@@ -46,17 +44,16 @@ constexpr int kBlockChunkBytes = kBlockChunkWords * 4;
 constexpr int kBlockWordsPerThread = kBlockChunkWords / kBlockThreads;
 static_assert(kBlockWordsPerThread % 4 == 0, "whole 16-byte loads per thread");
 
-// Dynamic shared memory: kBlockRing mbarriers and chunk buffers (or, in the
-// resident form, every word), an int accumulator per vertex (plus a spare slot
-// for the padding words), the chunk table, the class tables, then per vertex
+// Dynamic shared memory: kBlockRing mbarriers and chunk buffers, an int
+// accumulator per vertex (plus a spare slot for the padding words), the chunk table, the class tables, then per vertex
 // its state byte, its spin (+1/-1) and its flip decision. Offsets in bytes.
 struct BlockLayout {
   int acc, chunk, cls_chunk, cls_pos, state, spin, flip, total;
 };
 
-__host__ __device__ inline BlockLayout block_layout(int n, int nch, int ncls, int resident_words) {
+__host__ __device__ inline BlockLayout block_layout(int n, int nch, int ncls) {
   BlockLayout L{};
-  int o = 128 + (resident_words > 0 ? ((4 * resident_words + 15) & ~15) : kBlockRing * kBlockChunkBytes);
+  int o = 128 + kBlockRing * kBlockChunkBytes;
   L.acc = o;
   o += 4 * (n + 1);
   o = (o + 7) & ~7;
@@ -147,7 +144,7 @@ struct BlockShared {
 };
 
 __device__ __forceinline__ BlockShared block_shared(unsigned char* base, const BlockArgs& ba) {
-  const BlockLayout L = block_layout(ba.n, ba.num_chunks, ba.num_classes, ba.resident_words);
+  const BlockLayout L = block_layout(ba.n, ba.num_chunks, ba.num_classes);
   BlockShared s;
   s.bar = reinterpret_cast<unsigned long long*>(base);
   s.buf = reinterpret_cast<uint32_t*>(base + 128);
@@ -173,9 +170,6 @@ __device__ __forceinline__ void block_setup(const BlockArgs& ba, const BlockShar
     sh.cls_chunk[i] = ba.class_chunk[i];
     sh.cls_pos[i] = ba.class_pos[i];
   }
-  // resident form: every word, once (the word count is a multiple of 4)
-  for (int i = threadIdx.x; i < ba.resident_words / 4; i += blockDim.x)
-    reinterpret_cast<uint4*>(sh.buf)[i] = __ldg(reinterpret_cast<const uint4*>(ba.words) + i);
 }
 
 // Issue chunk q of this sweep, whose launch-wide sequence number is sq.
@@ -271,24 +265,6 @@ __device__ __forceinline__ void block_sweep_start(const DevGraph& d, const Sweep
     sh.flip[i] = flip_drawn(d, i, static_cast<uint32_t>(__ldg(d.orig + i)), a, rk) ? 1 : 0;
   }
   if (tid == 0) sh.acc[n] = 0;
-}
-
-// One sweep in the resident form: every class's words are in shared memory
-// already, so a class is its chunks, a block barrier, its decisions and a
-// block barrier.
-__device__ __forceinline__ void block_sweep_resident(const DevGraph& d, const BlockArgs& ba, const SweepArgs& a,
-                                                     const PhiloxRounds& rk, const BlockShared& sh) {
-  const int tid = threadIdx.x;
-  const int lane = tid & 31;
-  block_sweep_start(d, a, rk, sh, ba.n, tid);
-  __syncthreads();
-  for (int k = 0; k < ba.num_classes; ++k) {
-    for (int q = sh.cls_chunk[k]; q < sh.cls_chunk[k + 1]; ++q)
-      block_chunk(sh, sh.buf + sh.chunk[q].x, sh.chunk[q].y, ba.n, tid, lane);
-    __syncthreads();
-    block_decide(d, sh, k, tid);
-    __syncthreads();
-  }
 }
 
 // One sweep a.t of every class. seq numbers chunks over the whole launch:

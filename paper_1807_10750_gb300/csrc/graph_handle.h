@@ -68,7 +68,6 @@ struct ising_graph {
   // block engine of small graphs (host_graph.h, block.cuh)
   bool block_ok = false;
   int32_t block_num_chunks = 0;
-  int32_t block_num_words = 0;
   int32_t* d_block_words = nullptr;
   int32_t* d_block_chunk_off = nullptr;
   int32_t* d_block_chunk_len = nullptr;
@@ -111,6 +110,24 @@ struct ising_graph {
   uint32_t* d_hub_pflips = nullptr;  // a sweep's flips by position (n / 32 + 2 words)
   int32_t* d_hub_blk = nullptr;      // non-hub classes' work split over the worker blocks
   int32_t hub_grid = 0;              // blocks the split was made for
+  // spin-map engine (map.cuh)
+  bool map_ok = false;
+  int map_mode = 0, map_K = 0, map_warps = 0, map_smem = 0;
+  int32_t map_bytes = 0, map_tasks = 0, map_rows = 0, map_groups = 0, map_stage = 0, map_stride = 0;
+  isingx::MapBlock* d_map_blocks = nullptr;
+  isingx::MapTask* d_map_task = nullptr;
+  int32_t* d_map_words = nullptr;
+  int32_t* d_map_weights = nullptr;
+  int32_t* d_map_row_pos = nullptr;
+  int32_t* d_map_row_orig = nullptr;
+  int32_t* d_map_class = nullptr;      // class_row, class_seg, block_msg: K x (C + 1) each
+  int32_t* d_map_steps = nullptr;      // class_bytes, class_msg: C + 1 each
+  int32_t* d_map_msg = nullptr;
+  int32_t* d_map_index = nullptr;      // position -> map index
+  unsigned long long* d_map_mail = nullptr;
+  uint32_t* d_pick_count = nullptr;    // Algorithm 1's picks of a launch (grown on use)
+  int32_t* d_picks = nullptr;
+  size_t pick_sweeps = 0, pick_cap = 0;
   uint8_t* d_bias = nullptr;         // per-position flip bias (null: none)
   int32_t* d_rowid = nullptr;        // row of every CSR entry (built on first use)
   int32_t* d_gnn_hchunk = nullptr;   // warm-start network: per row, its first entry chunk or -1

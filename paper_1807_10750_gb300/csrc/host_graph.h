@@ -208,6 +208,86 @@ void bisect_parts(const HostGraph& g, int32_t parts, std::vector<int32_t>* part,
 void build_halo_plan(const HostGraph& g, int32_t parts, int32_t sweeps_per_epoch, HaloPlan* hp,
                      const std::atomic<bool>* cancel = nullptr);
 
+// Spin-map engine (map.cuh). K blocks share every colour class: a class's rows
+// are cut into units of one warp -- L lanes a row, 32 / L rows -- which are
+// dealt to the blocks in turn, and every block keeps the spins of the whole
+// graph in shared memory, one byte each. Positions are renumbered for that
+// map: class by class, block by block, a block's units in order.
+//
+// Row r of a unit of R = 32 / L rows belongs to lanes r, r + R, r + 2 R, ... A
+// unit's entries are stored as `groups` groups of 32 int4: entry 4 g + k of
+// lane l is the row's entry L (4 g + k) + l / R, word (map index << 8) |
+// (w & 0xff), padded with weight 0; wide weights sit in a second array of the
+// same layout. L is the smallest power of two that leaves a lane at most
+// kMapSlots entries, twice as many in a class that would otherwise need more
+// than one round of every warp.
+//
+// A block's work of a sweep is a table of rounds of `warps` tasks, class by
+// class; a task is a unit, a word of 32 flip draws for the next sweep, both
+// or neither. The draws go to the warps without a unit where there are any.
+constexpr int32_t kMapSlots = 16;
+constexpr int32_t kMapMaxWarps = 16;
+constexpr int32_t kMapMaxBlocks = 1024;
+constexpr int32_t kMapMaxDegree = 4096;
+constexpr int32_t kMapMaxVertices = 200 * 1024;
+constexpr int32_t kMapFlipShift = 18;  // map indices below 2^18, flip words below 2^14 - 1
+// One block with its entries in shared memory, or read from L2 as in the other
+// two: the blocks of one cluster, and one block per SM.
+enum MapMode { kMapBlock = 0, kMapBlockStream = 1, kMapCluster = 2, kMapGrid = 3 };
+
+struct MapTask {
+  int32_t words;  // first group of the unit within its block's groups
+  int32_t base;   // map index of the unit's first row | (flip word + 1) << kMapFlipShift
+  int32_t row;    // its first row among the block's rows | 1 << 31 on a class's last round
+  int32_t shape;  // rows | log2(L) << 8 | groups << 16; 0: no unit
+};
+
+// Per block, offsets into the flat arrays.
+struct MapBlock {
+  int32_t task0, rounds;   // `tasks`: rounds * warps entries
+  int32_t words0, groups;  // the entries (in groups of 32 int4)
+  int32_t row0, rows;      // `row_pos`, `row_orig` (rows a multiple of 32)
+  int32_t pad0, pad1;
+};
+
+struct MapPlan {
+  bool ok = false;
+  int32_t mode = 0, K = 0, warps = 0;
+  int32_t stage = 0;         // groups of the largest unit
+  int32_t map_bytes = 0;     // bytes of the map (a multiple of 16)
+  int32_t mail_stride = 0;   // messages of the largest class (grid)
+  int32_t max_tasks = 0, max_rows = 0, max_groups = 0;  // over the blocks
+  int32_t smem_bytes = 0;
+  std::vector<MapBlock> blocks;
+  std::vector<MapTask> tasks;
+  int64_t total_groups = 0;  // entry groups of all blocks; map_fill_kernel writes them on the device
+  std::vector<int32_t> row_pos, row_orig;  // per block row: position and caller id, -1 for padding
+  std::vector<int32_t> class_row;   // K x (C + 1): a block's first row of every class
+  std::vector<int32_t> class_seg;   // K x (C + 1): the map index of that row
+  std::vector<int32_t> block_msg;   // K x (C + 1): its first message of every class (grid)
+  std::vector<int32_t> class_bytes; // C + 1: bytes every block receives in a class (cluster)
+  std::vector<int32_t> class_msg;   // C + 1: first message of every class (grid)
+  std::vector<int32_t> msg;         // per message of 32 rows: (map index / 4) << 4 | words it
+                                    // fills; every block has one or more per class
+  std::vector<int32_t> map_index;   // position -> map index
+};
+
+// Fills mp (ok = true) for K blocks of `mode` and `warps` warps when the graph
+// has at most kMapMaxVertices vertices and kMapMaxDegree entries a row and a
+// block's tables fit in smem_limit bytes, its entries among them in mode
+// kMapBlock. wide: 32-bit weights.
+void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int64_t smem_limit, MapPlan* mp);
+
+// Shared memory of a block (map.cuh lays it out in this order): the map, the
+// resident entries (and weights), the tasks, the class tables (rows, map
+// segments, messages or received bytes, class messages), the rows' ids, two
+// sweeps of flip bits, the rows' biases, and 64 bytes for the barriers.
+inline int64_t map_smem_bytes(int32_t map_bytes, int64_t entry_groups, int32_t tasks, int32_t classes,
+                              int32_t rows) {
+  return int64_t(map_bytes) + entry_groups * 512 + int64_t(tasks) * 16 + 4 * ((int64_t(classes) + 4) / 4 * 4) * 4 +
+         int64_t(rows) * 4 + int64_t(rows) / 32 * 8 + int64_t(rows) + 64;
+}
+
 // Returns 0, or a negative ISING_* status.
 int build_host_graph(int32_t n, int64_t m, const int32_t* src, const int32_t* dst,
                      const int32_t* w, HostGraph* out);
