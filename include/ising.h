@@ -344,6 +344,11 @@ int ising_plan_halo(int32_t n, int64_t m, const int32_t* src, const int32_t* dst
  * of (floor(v / 4), 0, r, 1) for
  * ising_batch_init_random -- so each instance/replica reproduces a single-graph
  * anneal keyed by that instance and replica exactly.
+ *
+ * Batches whose rows have at most 63 entries and whose weights are at most 31
+ * in magnitude run with each instance on one block or on the blocks of a
+ * cluster, by its size, unless a tuning is set; others, and batches with a
+ * tuning set, run one block per instance.
  * ------------------------------------------------------------------------ */
 typedef struct ising_batch ising_batch; /* opaque */
 
@@ -379,7 +384,8 @@ int ising_batch_set_spins(ising_batch* b, int32_t graph, uint32_t replica, const
  * threads, one instance per block at a time), the threads that share a row's
  * entries (1, 2 or 4; their partial sums are combined by warp shuffles) and
  * the tail mode (0: every colour class with a block barrier after it; 32:
- * classes of at most 32 vertices decided by one warp with warp barriers).
+ * classes of at most 32 vertices decided by one warp with warp barriers), and
+ * goes on without a tuning where the clustered form is faster than all of them.
  * Results do not depend on the configuration. out_block (may be NULL)
  * receives the chosen block size; ising_batch_tuning reports the rest.
  * Synchronises the batch's stream. */

@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "../../include/ising.h"
+#include "batch_map.cuh"
 #include "batch_view.h"
 #include "host_graph.h"
 #include "philox.cuh"
@@ -419,9 +420,26 @@ uint64_t batch_t0(double p0) {
 constexpr int kBlockChoices[3] = {128, 256, 512};
 constexpr int kSplitChoices[3] = {1, 2, 4};
 constexpr int kTailChoices[2] = {0, 32};
+constexpr int kBatchError = 15;  // d_work: work queue heads, then the clustered form's error flag
+constexpr int kBatchWork = 16;
 constexpr int kTuneConfigs = 18;  // block x split x tail
 
 }  // namespace
+
+// Instances of the clustered form that share a cluster size; all but the
+// first group run on streams of their own beside the first.
+struct BatchMapGroup {
+  int K = 1, clusters = 1, smem = 0, count = 0;
+  bool unit = false;
+  int32_t map_bytes = 0, units_max = 0, classes_max = 0;
+  cudaStream_t stream = nullptr;
+  cudaEvent_t join = nullptr;
+  isingx::BatchMapInst* inst = nullptr;
+  isingx::BatchMapUnit* units = nullptr;
+  int32_t *block_unit = nullptr, *class_unit = nullptr, *class_bytes = nullptr;
+  int32_t *dst = nullptr, *row_sum = nullptr, *map_index = nullptr;
+  int4* words = nullptr;
+};
 
 struct ising_batch {
   int device = 0;
@@ -457,6 +475,11 @@ struct ising_batch {
   int tail = 0;   // classes up to this size decided by one warp
   float probe_ms[kTuneConfigs] = {};  // the autotuner's probe times
   int64_t total_nnz = 0;
+  // the clustered form (batch_map.cuh): one group of instances per cluster
+  // size. A tuning set by the caller selects the one-block kernel instead.
+  std::vector<BatchMapGroup> groups;
+  bool tuned = false;
+  cudaEvent_t fork = nullptr;
   // the instances as one graph, for the warm-start network (batch_union)
   int32_t* d_union_row_ptr = nullptr;
   int32_t* d_union_vbase = nullptr;
@@ -482,7 +505,18 @@ struct ising_batch {
 
 namespace {
 
+void group_free(BatchMapGroup& g) {
+  if (g.stream) cudaStreamDestroy(g.stream);
+  if (g.join) cudaEventDestroy(g.join);
+  void* ptrs[] = {g.inst, g.units, g.block_unit, g.class_unit, g.class_bytes, g.dst, g.row_sum, g.map_index, g.words};
+  for (void* p : ptrs)
+    if (p) cudaFree(p);
+  g = BatchMapGroup();
+}
+
 void batch_free(ising_batch* b) {
+  for (BatchMapGroup& g : b->groups) group_free(g);
+  if (b->fork) cudaEventDestroy(b->fork);
   if (b->graph_exec) cudaGraphExecDestroy(b->graph_exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   void* ptrs[] = {b->d_graphs,       b->d_order,       b->d_row_ptr,    b->d_adj,
@@ -559,11 +593,195 @@ int batch_grid(ising_batch* b, int block, int split, size_t smem) {
   return std::min(per_sm * b->num_sms, std::max(1, b->num_graphs));
 }
 
+// ---------------------------------------------------------------------------
+// The clustered form: host tables, launch.
+// ---------------------------------------------------------------------------
+const void* batch_map_kernel_for(bool cluster, bool unit) {
+  using isingx::batch_map_kernel;
+  if (cluster)
+    return unit ? reinterpret_cast<const void*>(batch_map_kernel<true, true>)
+                : reinterpret_cast<const void*>(batch_map_kernel<true, false>);
+  return unit ? reinterpret_cast<const void*>(batch_map_kernel<false, true>)
+              : reinterpret_cast<const void*>(batch_map_kernel<false, false>);
+}
+
+void batch_map_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int K, int clusters, int smem,
+                      cudaStream_t s) {
+  *cfg = cudaLaunchConfig_t{};
+  cfg->gridDim = dim3(static_cast<unsigned>(K * clusters));
+  cfg->blockDim = dim3(isingx::kBatchMapThreads);
+  cfg->dynamicSmemBytes = static_cast<size_t>(smem);
+  cfg->stream = s;
+  if (K == 1) return;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = static_cast<unsigned>(K);
+  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  cfg->attrs = attr;
+  cfg->numAttrs = 1;
+}
+
+// Uploads a plan that the device can run and lets the device lay out the
+// entries; *runs is false if it cannot.
+cudaError_t group_upload(ising_batch* b, const isingx::BatchMapPlan& p, const int32_t* d_row_base, BatchMapGroup* g,
+                         bool* runs) {
+  const void* kernel = batch_map_kernel_for(p.K > 1, p.unit);
+  int clusters = 0;
+  *runs = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem) == cudaSuccess;
+  if (p.K == 1) {
+    *runs = *runs && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&clusters, kernel, isingx::kBatchMapThreads,
+                                                                   static_cast<size_t>(p.smem)) == cudaSuccess;
+    clusters *= b->num_sms;
+  } else {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    batch_map_config(&cfg, &attr, p.K, 1, p.smem, b->stream);
+    *runs = *runs && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess;
+  }
+  cudaGetLastError();
+  *runs = *runs && clusters >= 1;
+  if (!*runs) return cudaSuccess;
+  static_assert(sizeof(isingx::BatchMapUnit) == sizeof(int4), "a unit is one 16-byte load");
+  g->K = p.K;
+  g->unit = p.unit;
+  g->count = static_cast<int>(p.inst.size());
+  g->clusters = std::min(clusters, g->count);
+  g->smem = p.smem;
+  g->map_bytes = p.map_bytes;
+  g->units_max = p.units_max;
+  g->classes_max = p.classes_max;
+  cudaError_t e;
+  int32_t* d_unit_inst = nullptr;
+  do {
+    if ((e = cudaStreamCreateWithFlags(&g->stream, cudaStreamNonBlocking)) != cudaSuccess) break;
+    if ((e = cudaEventCreateWithFlags(&g->join, cudaEventDisableTiming)) != cudaSuccess) break;
+    if ((e = upload(&g->inst, p.inst, b->stream)) != cudaSuccess) break;
+    if ((e = upload(&g->units, p.units, b->stream)) != cudaSuccess) break;
+    if ((e = upload(&g->block_unit, p.block_unit, b->stream)) != cudaSuccess) break;
+    if ((e = upload(&g->class_unit, p.class_unit, b->stream)) != cudaSuccess) break;
+    if ((e = upload(&g->class_bytes, p.class_bytes, b->stream)) != cudaSuccess) break;
+    if ((e = upload(&g->dst, p.dst, b->stream)) != cudaSuccess) break;
+    if ((e = upload(&g->row_sum, p.row_sum, b->stream)) != cudaSuccess) break;
+    if ((e = upload(&g->map_index, p.map_index, b->stream)) != cudaSuccess) break;
+    if ((e = upload(&d_unit_inst, p.unit_inst, b->stream)) != cudaSuccess) break;
+    if ((e = cudaMalloc(reinterpret_cast<void**>(&g->words),
+                        static_cast<size_t>(std::max<int64_t>(p.groups, 1)) * 512)) != cudaSuccess)
+      break;
+    isingx::batch_map_fill_kernel<<<b->num_sms * 8, 256, 0, b->stream>>>(
+        reinterpret_cast<const int4*>(g->units), d_unit_inst, static_cast<int>(p.units.size()), g->inst, d_row_base,
+        b->d_row_ptr, b->d_adj, g->map_index, g->words);
+    if ((e = cudaGetLastError()) != cudaSuccess) break;
+    e = cudaStreamSynchronize(b->stream);
+  } while (false);
+  cudaFree(d_unit_inst);
+  return e;
+}
+
+// The groups of the clustered form, largest cluster first. Without room for
+// them, or with an instance that does not fit, there are none.
+cudaError_t groups_build(ising_batch* b, const std::vector<isingx::BatchMapRows>& rows,
+                         const std::vector<int32_t>& order, const std::vector<int32_t>& row_base, bool unit, int wmax) {
+  int optin = 0;
+  cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, b->device);
+  if (e != cudaSuccess) return e;
+  int64_t total = 0;
+  for (const isingx::BatchMapRows& r : rows) total += static_cast<int64_t>(r.degree.size());
+  std::vector<const isingx::BatchMapRows*> left;
+  for (int32_t gi : order) left.push_back(&rows[static_cast<size_t>(gi)]);
+  int32_t* d_row_base = nullptr;
+  if ((e = upload(&d_row_base, row_base, b->stream)) != cudaSuccess) return e;
+  bool fits = true;
+  for (int K = 16; K >= 1 && fits && e == cudaSuccess; K /= 2) {
+    std::vector<const isingx::BatchMapRows*> mine, rest;
+    for (const isingx::BatchMapRows* r : left)
+      (K <= isingx::batch_map_blocks(static_cast<int64_t>(r->degree.size()), total, b->num_sms) ? mine : rest).push_back(r);
+    left = rest;
+    if (mine.empty()) continue;
+    isingx::BatchMapPlan plan;
+    b->groups.emplace_back();
+    fits = isingx::build_batch_map(mine, unit, wmax, K, optin, &plan);
+    if (fits) e = group_upload(b, plan, d_row_base, &b->groups.back(), &fits);
+  }
+  cudaFree(d_row_base);
+  if (e == cudaSuccess && fits) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+  if (e != cudaSuccess || !fits) {
+    for (BatchMapGroup& g : b->groups) group_free(g);
+    b->groups.clear();
+  }
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    e = cudaSuccess;
+  }
+  return e;
+}
+
+// Waits for the batch's stream; reports (and latches) a wait of the clustered
+// form that ran out.
+int batch_sync(ising_batch* b) {
+  if (b->groups.empty()) {
+    BATCH_CUDA(b, cudaStreamSynchronize(b->stream));
+    return ISING_OK;
+  }
+  int error = 0;
+  BATCH_CUDA(b, cudaMemcpyAsync(&error, b->d_work + kBatchError, sizeof(error), cudaMemcpyDeviceToHost, b->stream));
+  BATCH_CUDA(b, cudaStreamSynchronize(b->stream));
+  if (error != 0) b->status = ISING_ETIMEOUT;
+  return b->status;
+}
+
+// One launch per group: the first on the batch's stream, the others beside it
+// on their own, forked from and joined to it.
+int groups_launch(ising_batch* b, uint64_t t_begin, uint32_t sweeps, uint64_t T, uint64_t T0, uint64_t seed) {
+  BATCH_CUDA(b, cudaMemsetAsync(b->d_work, 0, sizeof(unsigned) * b->groups.size(), b->stream));
+  if (b->groups.size() > 1) BATCH_CUDA(b, cudaEventRecord(b->fork, b->stream));
+  for (size_t i = 0; i < b->groups.size(); ++i) {
+    BatchMapGroup& g = b->groups[i];
+    const void* kernel = batch_map_kernel_for(g.K > 1, g.unit);
+    BATCH_CUDA(b, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, g.smem));
+    if (g.K > 1) BATCH_CUDA(b, cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    isingx::BatchMapArgs a{};
+    a.inst = g.inst;
+    a.block_unit = g.block_unit;
+    a.units = reinterpret_cast<const int4*>(g.units);
+    a.class_unit = g.class_unit;
+    a.class_bytes = g.class_bytes;
+    a.dst = g.dst;
+    a.row_sum = g.row_sum;
+    a.map_index = g.map_index;
+    a.words = g.words;
+    a.spins = b->d_spins;
+    a.work = b->d_work + i;
+    a.error = reinterpret_cast<int*>(b->d_work + kBatchError);
+    a.num_graphs = g.count;
+    a.K = g.K;
+    a.replicas = b->replicas;
+    a.map_bytes = g.map_bytes;
+    a.units_max = g.units_max;
+    a.classes_max = g.classes_max;
+    a.budget = isingx::kBarrierBudgetNs;
+    uint32_t seed_lo = static_cast<uint32_t>(seed), seed_hi = static_cast<uint32_t>(seed >> 32);
+    const cudaStream_t s = i == 0 ? b->stream : g.stream;
+    if (i > 0) BATCH_CUDA(b, cudaStreamWaitEvent(s, b->fork, 0));
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    batch_map_config(&cfg, &attr, g.K, g.clusters, g.smem, s);
+    void* args[] = {&a, &t_begin, &sweeps, &T, &T0, &seed_lo, &seed_hi};
+    b->launches++;
+    BATCH_CUDA(b, cudaLaunchKernelExC(&cfg, kernel, args));
+    if (i > 0) {
+      BATCH_CUDA(b, cudaEventRecord(g.join, s));
+      BATCH_CUDA(b, cudaStreamWaitEvent(b->stream, g.join, 0));
+    }
+  }
+  return ISING_OK;
+}
+
 // Enqueue one anneal of every instance: reset the work queue, launch the
 // persistent kernel. The pair is captured into a CUDA graph once per block
 // size and replayed with this call's parameters.
 int batch_launch(ising_batch* b, uint64_t t_begin, uint32_t sweeps, uint64_t T, uint64_t T0,
                  uint64_t seed) {
+  if (!b->groups.empty() && !b->tuned) return groups_launch(b, t_begin, sweeps, T, T0, seed);
   const size_t smem = static_cast<size_t>(std::max(b->max_n, 1));
   const void* kernel = batch_kernel_for(b->block, b->split);
   BATCH_CUDA(b, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -626,6 +844,10 @@ int ising_batch_create(int32_t num_graphs, const int32_t* n, const int64_t* m, c
   std::vector<BatchGraph> graphs((size_t)num_graphs);
   std::vector<int32_t> row_ptr, adj, orig, class_pos, class_heavy;
   std::vector<int64_t> size_key((size_t)num_graphs);
+  std::vector<isingx::BatchMapRows> map_rows;
+  std::vector<int32_t> map_row_base;
+  bool map_rows_ok = true, all_unit = true;
+  int64_t map_wmax = 0;
   int64_t edge_off = 0, vtx = 0;
   int rc = ISING_OK;
   try {
@@ -679,6 +901,27 @@ int ising_batch_create(int32_t num_graphs, const int32_t* n, const int64_t* m, c
       for (size_t k = 0; k < (size_t)hg.nnz; ++k)
         adj.push_back(static_cast<int32_t>((static_cast<uint32_t>(hg.col[k]) << 8) |
                                            (static_cast<uint32_t>(hg.w[k]) & 0xffu)));
+      // the clustered form's rows
+      all_unit = all_unit && unit;
+      map_wmax = std::max(map_wmax, wmax);
+      map_rows_ok = map_rows_ok && wmax <= 31 && hg.max_degree <= isingx::kBatchMapDegree;
+      if (map_rows_ok) {
+        isingx::BatchMapRows mr;
+        mr.id = gi;
+        mr.vtx_base = G.vtx_base;
+        mr.class_begin = hg.class_begin;
+        mr.perm = hg.perm;
+        mr.degree.resize((size_t)hg.n);
+        mr.wsum.resize((size_t)hg.n);
+        for (size_t v = 0; v < (size_t)hg.n; ++v) {
+          mr.degree[v] = hg.row_ptr[v + 1] - hg.row_ptr[v];
+          int32_t s = 0;
+          for (int32_t k = hg.row_ptr[v]; k < hg.row_ptr[v + 1]; ++k) s += hg.w[(size_t)k];
+          mr.wsum[v] = s;
+        }
+        map_rows.push_back(std::move(mr));
+        map_row_base.push_back(G.row_base);
+      }
       orig.insert(orig.end(), hg.perm.begin(), hg.perm.end());
       class_pos.insert(class_pos.end(), hg.class_begin.begin(), hg.class_begin.end());
       b->total_weight[(size_t)gi] = hg.total_weight;
@@ -721,10 +964,17 @@ int ising_batch_create(int32_t num_graphs, const int32_t* n, const int64_t* m, c
     if ((e = cudaMalloc(reinterpret_cast<void**>(&b->d_spins), std::max<int64_t>(vtx, 16))) != cudaSuccess) break;
     if ((e = cudaMemsetAsync(b->d_spins, 0, std::max<int64_t>(vtx, 16), b->stream)) != cudaSuccess) break;
     if ((e = cudaMalloc(reinterpret_cast<void**>(&b->d_flips), std::max<int64_t>(vtx, 16))) != cudaSuccess) break;
-    if ((e = cudaMalloc(reinterpret_cast<void**>(&b->d_work), 16)) != cudaSuccess) break;
+    if ((e = cudaMalloc(reinterpret_cast<void**>(&b->d_work), kBatchWork * sizeof(unsigned))) != cudaSuccess) break;
     if ((e = cudaMalloc(reinterpret_cast<void**>(&b->d_energy2),
                         sizeof(long long) * (size_t)num_graphs * replicas)) != cudaSuccess) break;
-    e = cudaStreamSynchronize(b->stream);
+    if ((e = cudaMemsetAsync(b->d_work, 0, kBatchWork * sizeof(unsigned), b->stream)) != cudaSuccess) break;
+    if ((e = cudaStreamSynchronize(b->stream)) != cudaSuccess) break;
+    if (map_rows_ok) try {
+        e = groups_build(b, map_rows, order, map_row_base, all_unit, static_cast<int>(map_wmax));
+      } catch (const std::bad_alloc&) {
+        for (BatchMapGroup& g : b->groups) group_free(g);
+        b->groups.clear();
+      }
   } while (false);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -819,7 +1069,8 @@ int ising_batch_cuts(ising_batch* b, int64_t* out_cuts) {
   std::vector<long long> e2((size_t)b->num_graphs * b->replicas);
   BATCH_CUDA(b, cudaMemcpyAsync(e2.data(), b->d_energy2, e2.size() * sizeof(long long),
                                 cudaMemcpyDeviceToHost, b->stream));
-  BATCH_CUDA(b, cudaStreamSynchronize(b->stream));
+  const int rc2 = batch_sync(b);
+  if (rc2 != ISING_OK) return rc2;
   for (int32_t gi = 0; gi < b->num_graphs; ++gi)
     for (int r = 0; r < b->replicas; ++r) {
       const size_t k = (size_t)gi * b->replicas + r;
@@ -837,7 +1088,8 @@ int ising_batch_get_spins(ising_batch* b, int32_t graph, uint32_t replica, int8_
   std::vector<uint8_t> bytes((size_t)nn);
   BATCH_CUDA(b, cudaMemcpyAsync(bytes.data(), b->d_spins + b->vtx_base[(size_t)graph], (size_t)nn,
                                 cudaMemcpyDeviceToHost, b->stream));
-  BATCH_CUDA(b, cudaStreamSynchronize(b->stream));
+  rc = batch_sync(b);
+  if (rc != ISING_OK) return rc;
   const std::vector<int32_t>& pos = b->pos[(size_t)graph];
   for (int32_t v = 0; v < nn; ++v) out[v] = ((bytes[(size_t)pos[(size_t)v]] >> replica) & 1) ? -1 : 1;
   return ISING_OK;
@@ -880,10 +1132,16 @@ int ising_batch_autotune(ising_batch* b, uint32_t probe_sweeps, int32_t* out_blo
   int best = 0;
   if (e == cudaSuccess) e = cudaEventCreate(&t0);
   if (e == cudaSuccess) e = cudaEventCreate(&t1);
-  for (int cfg = 0; cfg < kTuneConfigs && e == cudaSuccess; ++cfg) {
-    b->block = kBlockChoices[cfg / 6];
-    b->split = kSplitChoices[(cfg / 2) % 3];
-    b->tail = kTailChoices[cfg % 2];
+  // after the configurations, the clustered form where the batch has one
+  const int probes = kTuneConfigs + (b->groups.empty() ? 0 : 1);
+  bool clustered = false;
+  for (int cfg = 0; cfg < probes && e == cudaSuccess; ++cfg) {
+    b->tuned = cfg < kTuneConfigs;
+    if (b->tuned) {
+      b->block = kBlockChoices[cfg / 6];
+      b->split = kSplitChoices[(cfg / 2) % 3];
+      b->tail = kTailChoices[cfg % 2];
+    }
     for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {  // first run warms the captured graph
       e = cudaEventRecord(t0, b->stream);
       if (e == cudaSuccess && batch_launch(b, 0, probe_sweeps, probe_sweeps + 1, batch_t0(0.1), 1) != ISING_OK)
@@ -893,10 +1151,13 @@ int ising_batch_autotune(ising_batch* b, uint32_t probe_sweeps, int32_t* out_blo
     }
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, t0, t1);
-    b->probe_ms[cfg] = ms;
+    if (cfg < kTuneConfigs) b->probe_ms[cfg] = ms;
     if (e == cudaSuccess && ms < best_ms) {
       best_ms = ms;
-      best = cfg;
+      if (cfg < kTuneConfigs)
+        best = cfg;
+      else
+        clustered = true;
     }
   }
   if (e == cudaSuccess)
@@ -913,6 +1174,7 @@ int ising_batch_autotune(ising_batch* b, uint32_t probe_sweeps, int32_t* out_blo
   b->block = kBlockChoices[best / 6];
   b->split = kSplitChoices[(best / 2) % 3];
   b->tail = kTailChoices[best % 2];
+  b->tuned = !clustered;
   if (out_block) *out_block = b->block;
   return ISING_OK;
 }
@@ -921,6 +1183,7 @@ int ising_batch_set_block(ising_batch* b, int32_t block) {
   if (b == nullptr) return ISING_EINVAL;
   if (block != 128 && block != 256 && block != 512) return ISING_EINVAL;
   b->block = block;
+  b->tuned = true;
   return ISING_OK;
 }
 
@@ -932,6 +1195,7 @@ int ising_batch_set_tuning(ising_batch* b, int32_t block, int32_t row_split, int
   b->block = block;
   b->split = row_split;
   b->tail = tail;
+  b->tuned = true;
   return ISING_OK;
 }
 

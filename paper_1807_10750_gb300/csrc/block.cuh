@@ -19,6 +19,7 @@
 
 #include <cstdint>
 
+#include "cluster.cuh"
 #include "host_graph.h"
 #include "philox.cuh"
 #include "sweep.cuh"
@@ -71,10 +72,6 @@ __host__ __device__ inline BlockLayout block_layout(int n, int nch, int ncls) {
   o += n;
   L.total = (o + 15) & ~15;
   return L;
-}
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
 __device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned count) {

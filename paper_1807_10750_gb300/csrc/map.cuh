@@ -47,7 +47,7 @@
 
 #include <cstdint>
 
-#include "block.cuh"
+#include "cluster.cuh"
 #include "host_graph.h"
 #include "philox.cuh"
 #include "sweep.cuh"
@@ -79,41 +79,6 @@ struct MapArgs {
   const int32_t* picks;        // their map indices, pick_stride per sweep
   int32_t pick_stride;
 };
-
-__device__ __forceinline__ uint32_t cluster_addr(uint32_t a, uint32_t rank) {
-  uint32_t r;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-
-__device__ __forceinline__ bool map_try(uint32_t bar, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(done)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return done != 0u;
-}
-
-// The bounded wait for a phase of a local mbarrier whose first tries failed.
-static __device__ __noinline__ bool map_wait(uint32_t bar, uint32_t parity, int* error, long long budget) {
-  const long long t0 = global_ns();
-  for (;;) {
-    for (int it = 0; it < 16; ++it)
-      if (map_try(bar, parity)) return true;
-    if (ld_relaxed_s32(error) != 0) return false;
-    if (global_ns() - t0 > budget) {
-      atomicExch(error, 1);
-      return false;
-    }
-  }
-}
 
 // The bounded wait for a message of sequence number seq.
 static __device__ __noinline__ bool map_poll(const unsigned long long* p, uint32_t seq, unsigned long long* x,

@@ -35,3 +35,13 @@ def test_plan_sweeps_like_the_rows(check, kind, n, m, wmax, mode, K):
         # 2: the tables do not fit (resident entries of a large graph, a map of
         # 200,000 spins beside too many tasks)
         assert r.returncode == 0 or (r.returncode == 2 and n * max(m, n) > 10 ** 6), r.stdout
+
+
+@pytest.mark.parametrize("K", [1, 2, 4, 8, 16])
+def test_batch_tables(tmp_path, K):
+    exe = str(tmp_path / "batch_map_check")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", os.path.join(ROOT, "include"), "-pthread", "-o", exe,
+                    os.path.join(ROOT, "tests", "batch_map_check.cpp"), os.path.join(CSRC, "host_graph.cpp"),
+                    os.path.join(CSRC, "batch_map_plan.cpp")], check=True)
+    r = subprocess.run([exe, str(K), "3"], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
