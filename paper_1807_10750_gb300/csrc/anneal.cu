@@ -99,6 +99,51 @@ __global__ void __launch_bounds__(kBlock, 4)
   }
 }
 
+// What a synchronising call reads after one launch, in pinned host memory.
+struct HostResult {
+  long long twice_energy;
+  int error;  // the barrier state's error flag
+  int bad;    // ising_set_spins: a value other than +1 / -1
+};
+
+// Twice the energy of the current spins, with the barrier state's error flag,
+// straight into pinned host memory: the block that finishes last writes it and
+// clears the accumulators, so a call costs one launch and one wait (a memset,
+// a launch, two copies and two waits before: ising_cut of an 800-vertex graph
+// 24 -> 11 us).
+template <bool PACKED>
+__global__ void __launch_bounds__(kBlock, 4)
+    energy_kernel(DevGraph d, int num_items, unsigned long long* acc, HostResult* out) {
+  const int lane = threadIdx.x & 31;
+  const int nwarps = gridDim.x * kWarpsPerBlock;
+  const SweepArgs a{};
+  const isingx::PhiloxRounds rk{};
+  long long energy = 0;
+  for (int i = (blockIdx.x * kBlock + threadIdx.x) >> 5; i < num_items; i += nwarps) {
+    isingx::Staged<PACKED> st;
+    isingx::stage_item<PACKED>(d, d.items[i], a, rk, lane, st);
+    isingx::finish_item<PACKED, kPassEnergy>(d, st, a, rk, lane, energy);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) energy += __shfl_xor_sync(isingx::kFullMask, energy, o);
+  __shared__ long long part[kWarpsPerBlock];
+  if (lane == 0) part[threadIdx.x >> 5] = energy;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    long long sum = 0;
+    for (int k = 0; k < kWarpsPerBlock; ++k) sum += part[k];
+    atomicAdd(acc, static_cast<unsigned long long>(sum));
+    __threadfence();
+    if (atomicAdd(acc + 1, 1ull) == gridDim.x - 1) {
+      __threadfence();
+      out->twice_energy = static_cast<long long>(atomicExch(acc, 0ull));
+      out->error = isingx::ld_relaxed_s32(d.error);
+      acc[1] = 0ull;
+      __threadfence_system();
+    }
+  }
+}
+
 // First item of colour class cls for this warp. Deterministic passes: item
 // warp of every class (a barrier follows each class). The racy pass walks
 // all classes without a barrier; when the sweep has at least as many items as
@@ -391,9 +436,25 @@ __global__ void gather_spins_kernel(int8_t* out, const int8_t* spins, const int3
     out[o] = static_cast<int8_t>(isingx::spin_of(spins[pos[o]]));
 }
 
-__global__ void check_spins_kernel(const int8_t* in, int n, int32_t* bad) {
+__global__ void check_spins_kernel(const int8_t* in, int n, HostResult* out) {
+  bool bad = false;
   for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < n; o += gridDim.x * blockDim.x)
-    if (in[o] != 1 && in[o] != -1) atomicExch(bad, 1);
+    bad = bad || (in[o] != 1 && in[o] != -1);
+  if (bad) *reinterpret_cast<volatile int*>(&out->bad) = 1;
+}
+
+// Check and scatter in one block: nothing is written if any value is bad.
+constexpr int kOneBlockSpins = 16384;
+__global__ void __launch_bounds__(1024)
+    check_scatter_spins_kernel(int8_t* spins, const int8_t* in, const int32_t* pos, int n, HostResult* out) {
+  bool bad = false;
+  for (int o = threadIdx.x; o < n; o += 1024) bad = bad || (in[o] != 1 && in[o] != -1);
+  if (__syncthreads_or(bad)) {
+    if (threadIdx.x == 0) *reinterpret_cast<volatile int*>(&out->bad) = 1;
+    return;
+  }
+  for (int o = threadIdx.x; o < n; o += 1024)
+    spins[pos[o]] = static_cast<int8_t>(isingx::state_byte(in[o], 0));
 }
 
 __global__ void scatter_spins_kernel(int8_t* spins, const int8_t* in, const int32_t* pos, int n) {
@@ -436,7 +497,7 @@ namespace {
 void free_device(ising_graph* g) {
   void* ptrs[] = {g->d_row_ptr, g->d_adj, g->d_col,  g->d_w,  g->d_ell, g->d_ell_col, g->d_ell_w, g->d_spins,
                   g->d_orig,    g->d_pos,         g->d_items,       g->d_slice_acc,
-                  g->d_slice_parts, g->d_energy,  g->d_flag,
+                  g->d_slice_parts, g->d_energy,
                   g->d_tmp,     g->d_class_items, g->d_all_items, g->d_barrier,
                   g->d_class_begin, g->d_trace, g->d_nflip_bits, g->d_nflip_list,
                   g->d_bias,    g->d_rowid, g->d_block_words, g->d_block_chunk_off,
@@ -451,6 +512,7 @@ void free_device(ising_graph* g) {
                   g->d_pick_count, g->d_picks};
   for (void* p : ptrs)
     if (p) cudaFree(p);
+  if (g->h_result) cudaFreeHost(g->h_result);
 }
 
 // Drop the halo plan (its device arrays); the next anneal that asks for the
@@ -1206,17 +1268,21 @@ int enqueue_energy(ising_graph* g, unsigned long long* slot) {
 }
 
 int compute_energy(ising_graph* g, int64_t* out) {
-  ISING_CUDA(g, cudaMemsetAsync(g->d_energy, 0, sizeof(unsigned long long), g->stream));
-  SweepArgs a{};
-  const isingx::PhiloxRounds rk{};
-  const int32_t all_items[2] = {0, g->num_items};
-  ISING_CUDA(g, launch_items<kPassEnergy>(g, g->d_all_items, all_items, 0, 1, a, rk, g->d_energy));
-  unsigned long long twice = 0;
-  ISING_CUDA(g, cudaMemcpyAsync(&twice, g->d_energy, sizeof(twice), cudaMemcpyDeviceToHost, g->stream));
+  const int grid = grid_for(g->num_items, kWarpsPerBlock, g->num_sms * 64);
+  const DevGraph d = g->dev();
+  HostResult* result = static_cast<HostResult*>(g->h_result);
+  g->launches++;
+  if (g->packed)
+    energy_kernel<true><<<grid, kBlock, 0, g->stream>>>(d, g->num_items, g->d_energy, result);
+  else
+    energy_kernel<false><<<grid, kBlock, 0, g->stream>>>(d, g->num_items, g->d_energy, result);
+  ISING_CUDA(g, cudaGetLastError());
   ISING_CUDA(g, cudaStreamSynchronize(g->stream));
-  const int rc = check_device_error(g);
-  if (rc != ISING_OK) return rc;
-  *out = static_cast<long long>(twice) / 2;
+  if (result->error != 0) {
+    g->status = ISING_ETIMEOUT;
+    return ISING_ETIMEOUT;
+  }
+  *out = result->twice_energy / 2;
   return ISING_OK;
 }
 
@@ -1375,8 +1441,8 @@ int ising_create(int32_t n, int64_t m, const int32_t* src, const int32_t* dst, c
     const size_t slots = plan.split_parts.size();
     if ((e = alloc_copy<unsigned long long>(&g->d_slice_acc, nullptr, 2 * slots, g->stream)) != cudaSuccess) break;
     if ((e = alloc_copy(&g->d_slice_parts, plan.split_parts.data(), slots, g->stream)) != cudaSuccess) break;
-    if ((e = alloc_copy<unsigned long long>(&g->d_energy, nullptr, 1, g->stream)) != cudaSuccess) break;
-    if ((e = alloc_copy<int32_t>(&g->d_flag, nullptr, 1, g->stream)) != cudaSuccess) break;
+    if ((e = alloc_copy<unsigned long long>(&g->d_energy, nullptr, 2, g->stream)) != cudaSuccess) break;
+    if ((e = cudaHostAlloc(&g->h_result, sizeof(HostResult), cudaHostAllocDefault)) != cudaSuccess) break;
     if ((e = alloc_copy<int8_t>(&g->d_tmp, nullptr, N, g->stream)) != cudaSuccess) break;
     if ((e = alloc_copy(&g->d_class_items, plan.class_item_begin.data(),
                         plan.class_item_begin.size(), g->stream)) != cudaSuccess) break;
@@ -1735,14 +1801,20 @@ int ising_set_spins(ising_graph* g, const int8_t* in, int on_device) {
   const int grid = grid_for(g->n, 256, g->num_sms * 8);
   const int8_t* source = in;
   if (on_device) {
-    ISING_CUDA(g, cudaMemsetAsync(g->d_flag, 0, sizeof(int32_t), g->stream));
+    HostResult* result = static_cast<HostResult*>(g->h_result);
+    result->bad = 0;
     g->launches++;
-  check_spins_kernel<<<grid, 256, 0, g->stream>>>(in, g->n, g->d_flag);
+    if (g->n <= kOneBlockSpins)
+      check_scatter_spins_kernel<<<1, 1024, 0, g->stream>>>(g->d_spins, in, g->d_pos, g->n, result);
+    else
+      check_spins_kernel<<<grid, 256, 0, g->stream>>>(in, g->n, result);
     ISING_CUDA(g, cudaGetLastError());
-    int32_t bad = 0;
-    ISING_CUDA(g, cudaMemcpyAsync(&bad, g->d_flag, sizeof(bad), cudaMemcpyDeviceToHost, g->stream));
     ISING_CUDA(g, cudaStreamSynchronize(g->stream));
-    if (bad) return ISING_EINVAL;
+    if (result->bad) return ISING_EINVAL;
+    if (g->n <= kOneBlockSpins) {
+      g->parity = 0;
+      return ISING_OK;
+    }
   } else {
     for (int32_t o = 0; o < g->n; ++o)
       if (in[o] != 1 && in[o] != -1) return ISING_EINVAL;

@@ -50,8 +50,8 @@ struct ising_graph {
   isingx::WorkItem* d_items = nullptr;
   unsigned long long* d_slice_acc = nullptr;
   int32_t* d_slice_parts = nullptr;
-  unsigned long long* d_energy = nullptr;
-  int32_t* d_flag = nullptr;
+  unsigned long long* d_energy = nullptr;  // energy accumulator and finished blocks (zero between calls)
+  void* h_result = nullptr;                // pinned: what a synchronising call reads (anneal.cu, HostResult)
   int8_t* d_tmp = nullptr;
   int32_t* d_class_items = nullptr;  // num_colours + 1 item offsets
   int32_t* d_class_begin = nullptr;  // num_colours + 1 first positions
