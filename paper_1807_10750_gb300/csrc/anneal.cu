@@ -500,7 +500,7 @@ void free_device(ising_graph* g) {
                   g->d_slice_parts, g->d_energy,
                   g->d_tmp,     g->d_class_items, g->d_all_items, g->d_barrier,
                   g->d_class_begin, g->d_trace, g->d_nflip_bits, g->d_nflip_list,
-                  g->d_bias,    g->d_rowid, g->d_block_words, g->d_block_chunk_off,
+                  g->d_bias,    g->d_block_words, g->d_block_chunk_off,
                   g->d_block_chunk_len, g->d_block_class_chunk, g->d_dep_ptr, g->d_deps,
                   g->d_done, g->d_halo_hdr, g->d_halo_words, g->d_halo_slices, g->d_halo_gpos,
                   g->d_halo_imports, g->d_halo_nbrs, g->d_halo_exports, g->d_halo_quads, g->d_halo_flags,

@@ -494,7 +494,6 @@ struct ising_batch {
   // the instances as one graph, for the warm-start network (batch_union)
   int32_t* d_union_row_ptr = nullptr;
   int32_t* d_union_vbase = nullptr;
-  int32_t* d_gnn_rowid = nullptr;
   int32_t* d_gnn_hchunk = nullptr;
   int32_t* d_gnn_chunk_row = nullptr;
   int32_t gnn_num_chunks = -1;
@@ -534,7 +533,7 @@ void batch_free(ising_batch* b) {
   void* ptrs[] = {b->d_graphs,       b->d_order,       b->d_row_ptr,    b->d_adj,
                   b->d_orig,         b->d_class_pos,   b->d_spins,      b->d_flips,
                   b->d_work,         b->d_energy2,     b->d_union_row_ptr, b->d_union_vbase,
-                  b->d_gnn_rowid,    b->d_gnn_hchunk,  b->d_gnn_chunk_row, b->d_class_heavy,
+                  b->d_gnn_hchunk,  b->d_gnn_chunk_row, b->d_class_heavy,
                   b->d_out};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -1029,7 +1028,6 @@ int batch_union(ising_batch* b, BatchUnion* out) {
   out->vbase = b->d_union_vbase;
   out->orig = b->d_orig;
   out->spins = b->d_spins;
-  out->rowid = &b->d_gnn_rowid;
   out->hchunk = &b->d_gnn_hchunk;
   out->chunk_row = &b->d_gnn_chunk_row;
   out->num_chunks = &b->gnn_num_chunks;

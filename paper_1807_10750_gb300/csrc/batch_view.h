@@ -23,7 +23,6 @@ struct BatchUnion {
   const int32_t* orig = nullptr;     // per position: vertex id within its instance
   uint8_t* spins = nullptr;          // per position: bit r set when replica r's spin is -1
   // storage the network fills on first use; freed with the batch
-  int32_t** rowid = nullptr;
   int32_t** hchunk = nullptr;
   int32_t** chunk_row = nullptr;
   int32_t* num_chunks = nullptr;     // -1 until built

@@ -27,11 +27,13 @@
 //             training, as the bf16 operand the backward pass reuses.
 //   head:     z = h3 w_o + b_o per row (fp32), with the loss G4 and its
 //             gradient when labels are given.
-//   backward: one kernel per layer forms dL/dh' = (direct part) + A_hat da
-//             of the layer above (the same fused gather), dU = dL/dh' *
-//             (h' > 0), dX = dU W^T (tensor cores; direct part fp32, da
-//             bf16) and dW += X^T dU (tensor cores, partial sums in
-//             registers, fp32 atomics per block), db in fp32.
+//   backward: per layer, from the top: one kernel forms dL/dh' = (direct
+//             part) + A_hat da of the layer above (the same gather; the top
+//             layer's is dz w_o and is formed where it is used) and dU =
+//             dL/dh' * (h' > 0) in bf16 with its column sums db; a second one
+//             streams X and dU through shared memory for dX = dU W^T (tensor
+//             cores; direct part fp32, da bf16) and dW += X^T dU (tensor
+//             cores, partial sums in registers, fp32 atomics per block).
 //   adam:     fp32 master weights, moments, and the bf16 copies the mma
 //             kernels read.
 #include <cuda_bf16.h>
@@ -99,7 +101,6 @@ struct GView {
   const int32_t* row_ptr;
   EdgeView ev;
   const int32_t* vbase;  // per row: added to its entries' columns (null: none)
-  const int32_t* rowid;  // row of every entry
   const uint8_t* spins;  // spin of position p is -1 when bit `shift` of spins[p] is set
   int shift;
   const int32_t* hchunk;     // per row: first chunk of a heavy row, else -1 (null: no heavy row)
@@ -113,76 +114,92 @@ __device__ __forceinline__ int col_base(const GView& v, int row) { return v.vbas
 
 __device__ __forceinline__ int spin_at(const int8_t* spins, int v) { return 1 - 2 * (spins[v] & 1); }
 
-// Inclusive segmented sum across the warp. Lanes hold consecutive CSR
-// entries, so equal rows are contiguous; lanes past the end carry row -1.
-template <typename T>
-__device__ __forceinline__ T seg_sum(T v, int row, int lane) {
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const T u = __shfl_up_sync(kFull, v, o);
-    const int r = __shfl_up_sync(kFull, row, o);
-    if (lane >= o && r == row) v += u;
-  }
-  return v;
-}
-
-__device__ __forceinline__ bool seg_tail(int row, int lane) {
-  const int next = __shfl_down_sync(kFull, row, 1);
-  return row >= 0 && (lane == 31 || next != row);
-}
-
-__global__ void rowid_kernel(const int32_t* row_ptr, int n, int32_t* rowid) {
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-    const int e1 = row_ptr[v + 1];
-    for (int e = row_ptr[v]; e < e1; ++e) rowid[e] = v;
-  }
-}
-
-// sums[v] = (sum |w|, degree, sum w, f = sum w s_j) of row v (zeroed first).
-__global__ void rowsum_kernel(GView v, int4* sums) {
+// sums[row] += (sum |w|, -, sum w, f = sum w s_j) over a heavy row's chunks, a
+// warp per chunk (the heavy rows' sums zeroed first).
+__global__ void chunk_sums_kernel(GView v, int4* sums) {
   const int lane = threadIdx.x & 31;
-  const long long nw = (static_cast<long long>(gridDim.x) * blockDim.x) >> 5;
-  for (long long base = ((static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * 32;
-       base < v.nnz; base += nw * 32) {
-    const long long e = base + lane;
-    int row = -1, a = 0, c = 0, ws = 0, f = 0;
-    if (e < v.nnz) {
+  const int nw = (gridDim.x * blockDim.x) >> 5;
+  for (int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < v.num_chunks; k += nw) {
+    const int row = __ldg(v.chunk_row + k), base = col_base(v, row);
+    const int e0 = __ldg(v.row_ptr + row) + (k - __ldg(v.hchunk + row)) * kChunk;
+    const int e1 = min(e0 + kChunk, __ldg(v.row_ptr + row + 1));
+    int a = 0, ws = 0, f = 0;
+    for (int e = e0 + lane; e < e1; e += 32) {
       int col, w;
-      edge_at(v.ev, static_cast<int>(e), col, w);
-      row = __ldg(v.rowid + e);
-      a = w < 0 ? -w : w;
-      c = 1;
-      ws = w;
-      f = w * spin_of(v, col + col_base(v, row));
+      edge_at(v.ev, e, col, w);
+      a += w < 0 ? -w : w;
+      ws += w;
+      f += w * spin_of(v, col + base);
     }
-    a = seg_sum(a, row, lane);
-    c = seg_sum(c, row, lane);
-    ws = seg_sum(ws, row, lane);
-    f = seg_sum(f, row, lane);
-    if (seg_tail(row, lane)) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(kFull, a, o);
+      ws += __shfl_xor_sync(kFull, ws, o);
+      f += __shfl_xor_sync(kFull, f, o);
+    }
+    if (lane == 0) {
       atomicAdd(&sums[row].x, a);
-      atomicAdd(&sums[row].y, c);
       atomicAdd(&sums[row].z, ws);
       atomicAdd(&sums[row].w, f);
     }
   }
 }
 
-// G1/G2: x_v = [s, f c^2, s f c^2, log(1 + deg) / 8, (sum w) c^2, 1, 0, 0].
+// G1/G2: x_v = [s, f c^2, s f c^2, log(1 + deg) / 8, (sum w) c^2, 1, 0, 0]. Four
+// lanes sum a light row's entries (integers, so in any order); a heavy row's
+// sums come from chunk_sums_kernel. One pass over the entries without
+// atomics, fused with the features: on 3.5M entries 38 -> 19 us.
 __global__ void features_kernel(GView v, const int4* sums, uint4* x, float* cvec) {
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < v.n; p += gridDim.x * blockDim.x) {
-    const int4 q = sums[p];
+  const int q = threadIdx.x & 3;
+  const int subs = (gridDim.x * blockDim.x) >> 2;
+  for (int p0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 2; p0 - (threadIdx.x >> 2) % 8 < v.n; p0 += subs) {
+    const int p = min(p0, v.n - 1);  // every lane of the warp reaches the shuffles
+    const int e0 = __ldg(v.row_ptr + p), e1 = __ldg(v.row_ptr + p + 1);
+    const bool heavy = v.hchunk != nullptr && e1 - e0 > kHeavy;
+    int a = 0, ws = 0, fi = 0;
+    if (heavy) {
+      const int4 t = sums[p];
+      if (q == 0) {
+        a = t.x;
+        ws = t.z;
+        fi = t.w;
+      }
+    } else {
+      const int base = col_base(v, p);
+      for (int e = e0 + q; e < e1; e += 16) {
+        int col[4], w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          col[u] = p - base;
+          w[u] = 0;
+          if (e + 4 * u < e1) edge_at(v.ev, e + 4 * u, col[u], w[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          a += w[u] < 0 ? -w[u] : w[u];
+          ws += w[u];
+          fi += w[u] * spin_of(v, col[u] + base);
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+      a += __shfl_xor_sync(kFull, a, o);
+      ws += __shfl_xor_sync(kFull, ws, o);
+      fi += __shfl_xor_sync(kFull, fi, o);
+    }
+    if (q != 0 || p0 >= v.n) continue;
     const float s = static_cast<float>(spin_of(v, p));
-    const float d1 = static_cast<float>(q.x) + 1.0f;
+    const float d1 = static_cast<float>(a) + 1.0f;
     const float c2 = 1.0f / d1;
-    const float f = static_cast<float>(q.w);
+    const float f = static_cast<float>(fi);
     cvec[p] = 1.0f / sqrtf(d1);
-    bf162 p0 = __floats2bfloat162_rn(s, f * c2);
-    bf162 p1 = __floats2bfloat162_rn(s * f * c2, log1pf(static_cast<float>(q.y)) * 0.125f);
-    bf162 p2 = __floats2bfloat162_rn(static_cast<float>(q.z) * c2, 1.0f);
+    bf162 p0v = __floats2bfloat162_rn(s, f * c2);
+    bf162 p1 = __floats2bfloat162_rn(s * f * c2, log1pf(static_cast<float>(e1 - e0)) * 0.125f);
+    bf162 p2 = __floats2bfloat162_rn(static_cast<float>(ws) * c2, 1.0f);
     bf162 p3 = __floats2bfloat162_rn(0.0f, 0.0f);
     uint4 out;
-    memcpy(&out.x, &p0, 4);
+    memcpy(&out.x, &p0v, 4);
     memcpy(&out.y, &p1, 4);
     memcpy(&out.z, &p2, 4);
     memcpy(&out.w, &p3, 4);
@@ -192,38 +209,47 @@ __global__ void features_kernel(GView v, const int4* sums, uint4* x, float* cvec
 
 // ---------------------------------------------------------------------------
 // Gathers. A row of width D is read by a sub-warp of G lanes, F features per
-// lane: width 64 as 16 lanes x 4 (8-byte loads), width 8 as 4 lanes x 2.
+// lane: width 64 as 8 lanes x 8 (16-byte loads), width 8 as 4 lanes x 2.
 
 template <int D>
 struct RowIO;
 
 template <>
 struct RowIO<64> {
-  static constexpr int G = 16, F = 4;
-  using T = uint2;
+  static constexpr int G = 8, F = 8;
+  using T = uint4;
   static __device__ __forceinline__ T load(const bf16* p, long long row, int q) {
-    return __ldg(reinterpret_cast<const uint2*>(p) + row * 16 + q);
+    return __ldg(reinterpret_cast<const uint4*>(p) + row * 8 + q);
   }
   static __device__ __forceinline__ void store(bf16* p, long long row, int q, T val) {
-    reinterpret_cast<uint2*>(p)[row * 16 + q] = val;
+    reinterpret_cast<uint4*>(p)[row * 8 + q] = val;
   }
-  static __device__ __forceinline__ void put(bf16* s, T val) { *reinterpret_cast<uint2*>(s) = val; }
+  static __device__ __forceinline__ void put(bf16* s, T val) { *reinterpret_cast<uint4*>(s) = val; }
+  static __device__ __forceinline__ void unpack(T val, float (&f)[F]) {
+    const uint32_t w[4] = {val.x, val.y, val.z, val.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      bf162 p;
+      memcpy(&p, &w[k], 4);
+      const float2 x = __bfloat1622float2(p);
+      f[2 * k] = x.x;
+      f[2 * k + 1] = x.y;
+    }
+  }
   static __device__ __forceinline__ void add(float (&acc)[F], float coef, T val) {
-    bf162 a, b;
-    memcpy(&a, &val.x, 4);
-    memcpy(&b, &val.y, 4);
-    const float2 fa = __bfloat1622float2(a), fb = __bfloat1622float2(b);
-    acc[0] += coef * fa.x;
-    acc[1] += coef * fa.y;
-    acc[2] += coef * fb.x;
-    acc[3] += coef * fb.y;
+    float f[F];
+    unpack(val, f);
+#pragma unroll
+    for (int k = 0; k < F; ++k) acc[k] += coef * f[k];
   }
   static __device__ __forceinline__ T pack(const float (&acc)[F]) {
-    T out;
-    bf162 a = __floats2bfloat162_rn(acc[0], acc[1]), b = __floats2bfloat162_rn(acc[2], acc[3]);
-    memcpy(&out.x, &a, 4);
-    memcpy(&out.y, &b, 4);
-    return out;
+    uint32_t w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const bf162 p = __floats2bfloat162_rn(acc[2 * k], acc[2 * k + 1]);
+      memcpy(&w[k], &p, 4);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
   }
 };
 
@@ -254,13 +280,18 @@ struct RowIO<8> {
 };
 
 // acc += sum over entries [e0, e1) of w c_col src[col] (this lane's
-// features). Width 64: the 16 lanes of a sub-warp decode up to 64 entries
+// features). Width 64: the 8 lanes of a sub-warp decode up to 32 entries
 // at once (column words and c_col, four per lane), then every lane reads its
-// 8 bytes of each of those rows, eight rows in flight -- two dependent memory
-// rounds per 64 entries. Width 8:
+// 16 bytes of each of those rows, kFly rows in flight -- two dependent memory
+// rounds per 32 entries. With 16 lanes of 8 bytes a row the load-store pipe was
+// the limit (74 % busy): the shuffles that hand out a column and a coefficient
+// then serve two rows a warp, here four. Layer kernel on 3.5M entries of 416k
+// rows 142 -> 122 us, on the 2M entries of a 100k-vertex power-law graph
+// 53 -> 45 us. Width 8:
 // each of the 4 lanes takes every fourth entry and whole 16-byte rows, four
 // entries in flight, and the lanes' sums are combined at the end. Both fix
 // the order of every sum.
+constexpr int kFly = 4;
 template <int D>
 __device__ __forceinline__ void gather_entries(const GView& v, const float* __restrict__ c,
                                                const bf16* __restrict__ src, int e0, int e1, int base,
@@ -270,8 +301,8 @@ __device__ __forceinline__ void gather_entries(const GView& v, const float* __re
   const unsigned lane = threadIdx.x & 31;
   const unsigned mask = ((1u << G) - 1u) << (lane & ~(G - 1u));
   if constexpr (D == 64) {
-    // up to 64 entries per round: lane q decodes entries q, q + 16, q + 32,
-    // q + 48 of the round (slots 0..3)
+    // up to 4 G entries per round: lane q decodes entries q, q + G, q + 2 G,
+    // q + 3 G of the round (slots 0..3)
     for (int b = e0; b < e1; b += 4 * G) {
       const int cnt = min(4 * G, e1 - b);
       int col[4];
@@ -294,16 +325,16 @@ __device__ __forceinline__ void gather_entries(const GView& v, const float* __re
       for (int u = 0; u < 4; ++u) {
         if (u * G >= cnt) break;
 #pragma unroll
-        for (int j0 = 0; j0 < G; j0 += 8) {
+        for (int j0 = 0; j0 < G; j0 += kFly) {
           if (u * G + j0 >= cnt) break;
-          typename IO::T hv[8];
+          typename IO::T hv[kFly];
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
+          for (int k = 0; k < kFly; ++k) {
             const int cj = __shfl_sync(mask, col[u], j0 + k, G);
             hv[k] = u * G + j0 + k < cnt ? IO::load(src, cj, q) : typename IO::T{};
           }
 #pragma unroll
-          for (int k = 0; k < 8; ++k) IO::add(acc, __shfl_sync(mask, cf[u], j0 + k, G), hv[k]);
+          for (int k = 0; k < kFly; ++k) IO::add(acc, __shfl_sync(mask, cf[u], j0 + k, G), hv[k]);
         }
       }
     }
@@ -435,11 +466,18 @@ __device__ __forceinline__ uint32_t pack_bf162(float x, float y) {
 
 // Forward layer: hout = relu([h, a] W + b) with a = A_hat h gathered by the
 // tile itself; W [2D][64] bf16 row-major. With a_store, a (bf16) is kept for
-// the backward pass. Eight warps: the gather takes two rows (D = 64) or
+// the backward pass. Eight warps: the gather takes four rows (D = 64) or
 // eight rows (D = 8) per warp at a time; the product gives each warp 16
 // rows x 32 columns.
+// Resident blocks the registers are sized for: the gather lives on loads in
+// flight, spread over warps rather than over registers of one (width 64 at
+// 2 / 3 / 4 / 5 blocks: 199 / 204 / 192 / 197 us for the whole forward pass on a
+// 100k-vertex, 2M-entry power-law graph; width 8 at 4 / 6 / 8: 194 / 193 / 198).
 template <int D>
-__global__ void __launch_bounds__(kLayerThreads)
+constexpr int kLayerBlocks = D == kH ? 4 : 6;
+
+template <int D>
+__global__ void __launch_bounds__(kLayerThreads, kLayerBlocks<D>)
     layer_fwd_kernel(GView v, const float* __restrict__ c, const bf16* __restrict__ h,
                      const float* __restrict__ partial, const bf16* __restrict__ W,
                      const float* __restrict__ bias, bf16* __restrict__ a_store, bf16* __restrict__ hout) {
@@ -767,36 +805,68 @@ __global__ void __launch_bounds__(kTcThreads, kTcMinBlocks)
 }
 
 // Head: z = h3 w_o + b_o. With labels y (+-1 by position): the loss G4 (sum
-// over rows, divided by n on the host), dz = -y sigmoid(-y z) / n, dh3 = dz w_o
-// and the head's gradients.
+// over rows, divided by n on the host), dz = -y sigmoid(-y z) / n and the
+// head's gradients (dL/dh3 = dz w_o is formed by the layer below). A warp
+// takes 32 rows at a time: 32 loads in flight, the dot products reduced eight
+// together, halving the rows a lane holds with the first three exchanges (the
+// same pairs are added as in a sum per row), and one row's sigmoid per lane.
+// 416k rows with labels: 95 us with one row at a time and dL/dh3 written out,
+// now 24.
 __global__ void head_kernel(const bf162* h3, const float* params, const int8_t* y, int n,
-                            float inv_n, float* z, float* dh3, float* grad, double* loss) {
+                            float inv_n, float* z, float* dz_out, float* grad, double* loss) {
   const int lane = threadIdx.x & 31;
   const float w0 = params[kOffWo + 2 * lane], w1 = params[kOffWo + 2 * lane + 1];
   const float bo = params[kOffBo];
   float g0 = 0.0f, g1 = 0.0f, gb = 0.0f;
   double lsum = 0.0;
   const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += nw) {
-    const float2 hv = __bfloat1622float2(h3[static_cast<size_t>(v) * 32 + lane]);
-    float s = hv.x * w0 + hv.y * w1;
+  for (int v0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; v0 < n; v0 += nw * 32) {
+    bf162 hv[32];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-    const float zv = s + bo;
-    if (lane == 0) z[v] = zv;
+    for (int k = 0; k < 32; ++k)
+      hv[k] = v0 + k < n ? h3[static_cast<size_t>(v0 + k) * 32 + lane] : __floats2bfloat162_rn(0.0f, 0.0f);
+    float zv = 0.0f;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {  // rows 8 b .. 8 b + 7: row 8 b + lane / 4 ends up in its four lanes
+      float s[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const float2 x = __bfloat1622float2(hv[8 * b + k]);
+        s[k] = x.x * w0 + x.y * w1;
+      }
+#pragma unroll
+      for (int o = 16, m = 4; o >= 4; o >>= 1, m >>= 1) {
+        const bool up = lane & o;  // keeps the rows m .. 2 m - 1 of those it holds
+#pragma unroll
+        for (int k = 0; k < m; ++k) {
+          const float send = up ? s[k] : s[k + m], keep = up ? s[k + m] : s[k];
+          s[k] = keep + __shfl_xor_sync(kFull, send, o);
+        }
+      }
+      s[0] += __shfl_xor_sync(kFull, s[0], 2);
+      s[0] += __shfl_xor_sync(kFull, s[0], 1);
+      if ((lane & 3) == b) zv = s[0] + bo;
+    }
+    const int v = v0 + 8 * (lane & 3) + (lane >> 2);  // this lane's row
+    if (v < n) z[v] = zv;
     if (y != nullptr) {
-      const float yv = y[v] > 0 ? 1.0f : -1.0f;
-      const float m = -yv * zv;
-      const float sig = 1.0f / (1.0f + expf(-m));  // sigmoid(-y z)
-      const float dz = -yv * sig * inv_n;
-      if (lane == 0) {
+      float dz = 0.0f;
+      if (v < n) {
+        const float yv = y[v] > 0 ? 1.0f : -1.0f;
+        const float m = -yv * zv;
+        const float sig = 1.0f / (1.0f + expf(-m));  // sigmoid(-y z)
+        dz = -yv * sig * inv_n;
+        dz_out[v] = dz;
         lsum += static_cast<double>(fmaxf(m, 0.0f) + log1pf(expf(-fabsf(m))));
         gb += dz;
       }
-      float2 d2 = make_float2(dz * w0, dz * w1);
-      reinterpret_cast<float2*>(dh3)[static_cast<size_t>(v) * 32 + lane] = d2;
-      g0 += dz * hv.x;
-      g1 += dz * hv.y;
+#pragma unroll
+      for (int k = 0; k < 32; ++k) {
+        const float d = __shfl_sync(kFull, dz, 4 * (k & 7) + (k >> 3));
+        const float2 x = __bfloat1622float2(hv[k]);
+        g0 += d * x.x;
+        g1 += d * x.y;
+      }
     }
   }
   if (y == nullptr) return;
@@ -807,6 +877,11 @@ __global__ void head_kernel(const bf162* h3, const float* params, const int8_t* 
   __syncthreads();
   atomicAdd(&sg[2 * lane], g0);
   atomicAdd(&sg[2 * lane + 1], g1);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    gb += __shfl_xor_sync(kFull, gb, o);
+    lsum += __shfl_xor_sync(kFull, lsum, o);
+  }
   if (lane == 0) {
     atomicAdd(&sg[kH], gb);
     atomicAdd(&sl, lsum);
@@ -817,25 +892,70 @@ __global__ void head_kernel(const bf162* h3, const float* params, const int8_t* 
   if (threadIdx.x == 0) atomicAdd(loss, sl);
 }
 
-// Backward of one layer (h' = relu([h, a] W + b)). dL/dh' is `direct` plus,
-// with AGG, A_hat da_src (da_src = dL/da of the layer above, gathered by the
-// tile as in the forward pass). Then dU = dL/dh' * (h' > 0); gW += X^T dU;
-// gb += colsum dU; with DX also dX = dU W^T, split into dh_out (fp32, the
-// direct part for the layer below) and da_out (bf16, to be propagated).
-template <int D, bool DX, bool AGG>
+// dU = dL/dh' * (h' > 0) of a layer h' = relu([h, a] W + b) below the top one,
+// dL/dh' = direct + A_hat da (da = dL/da of the layer above), and gb += the
+// column sums of dU (unrounded). A kernel of its own: the gather lives on warps
+// in flight (32 an SM here, 16 in a kernel that also holds the products'
+// accumulators). 416k rows and 3.5M entries, with the products of the layer:
+// 355 us in one kernel, 122 + 88 in two; the first layer's 251 -> 123 + 26.
+__global__ void __launch_bounds__(256)
+    dpre_kernel(GView v, const float* __restrict__ c, const float* __restrict__ direct, const bf16* __restrict__ da,
+                const float* __restrict__ partial, const bf16* __restrict__ hn, bf16* __restrict__ dU,
+                float* __restrict__ gb) {
+  using IO = RowIO<kH>;
+  __shared__ float sdb[kH];
+  if (threadIdx.x < kH) sdb[threadIdx.x] = 0.0f;
+  __syncthreads();
+  const int q = threadIdx.x % IO::G, subs = gridDim.x * blockDim.x / IO::G;
+  float db[IO::F] = {};
+  for (int r = (blockIdx.x * blockDim.x + threadIdx.x) / IO::G; r < v.n; r += subs) {
+    const float4* d4 = reinterpret_cast<const float4*>(direct + static_cast<size_t>(r) * kH + IO::F * q);
+    const float4 lo = __ldg(d4), hi = __ldg(d4 + 1);
+    const typename IO::T hraw = IO::load(hn, r, q);
+    float acc[IO::F] = {};
+    aggregate_row<kH>(v, c, da, partial, r, q, acc);
+    const float dv[IO::F] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    float h[IO::F];
+    IO::unpack(hraw, h);
+#pragma unroll
+    for (int f = 0; f < IO::F; ++f) {
+      acc[f] = h[f] > 0.0f ? dv[f] + acc[f] : 0.0f;
+      db[f] += acc[f];
+    }
+    IO::store(dU, r, q, IO::pack(acc));
+  }
+#pragma unroll
+  for (int f = 0; f < IO::F; ++f) atomicAdd(&sdb[IO::F * q + f], db[f]);
+  __syncthreads();
+  if (threadIdx.x < kH) atomicAdd(gb + threadIdx.x, sdb[threadIdx.x]);
+}
+
+// The products of a layer's backward pass: gW += X^T dU with X = [h, a], and
+// with DX dX = dU W^T, split into dh_out (fp32, the direct part for the layer
+// below) and da_out (bf16, to be propagated). u holds dU, or with TOP (the layer
+// under the head) the layer's output h', of which dU = dz w_head * (h' > 0) is
+// formed here with its column sums (gb). It streams: the next 64-row tile's X
+// and u are copied to shared memory (cp.async, two stages) while the current
+// one's products run. The layer under the head, 416k rows: 181 us with dL/dh3
+// read from memory and one stage, now 100 (320 MB: 47 us at the copy rate).
+template <int D>
+constexpr int bwd_smem(bool dx) {
+  return ((dx ? 2 * D * (kH + 8) : 0) + 2 * kTile * (2 * D + 8) + 2 * kTile * (kH + 8)) * 2;
+}
+
+template <int D, bool DX, bool TOP>
 __global__ void __launch_bounds__(kLayerThreads, 2)
-    layer_bwd_kernel(GView v, const float* __restrict__ c, const float* __restrict__ direct,
-                     const bf16* __restrict__ da_src, const float* __restrict__ partial,
-                     const bf16* __restrict__ hn, const bf16* __restrict__ h, const bf16* __restrict__ a,
-                     const bf16* __restrict__ W, float* __restrict__ gW, float* __restrict__ gb,
-                     float* __restrict__ dh_out, bf16* __restrict__ da_out) {
+    bwd_products_kernel(int n, const bf16* __restrict__ u, const float* __restrict__ dz, const bf16* __restrict__ h,
+                        const bf16* __restrict__ a, const bf16* __restrict__ W, const float* __restrict__ w_head,
+                        float* __restrict__ gW, float* __restrict__ gb, float* __restrict__ dh_out,
+                        bf16* __restrict__ da_out) {
   constexpr int K2 = 2 * D, KP = K2 + 8, NP = kH + 8;
   constexpr int MT = K2 / 16;  // 16-row tiles of gW; 8 x MT tiles of 16 x 8, MT per warp
-  constexpr int WR = DX ? K2 : 1;
   constexpr int XN = K2 / 16;  // dX: 8-column tiles per warp (half of K2 each)
-  __shared__ __align__(16) bf16 sW[WR * NP];
-  __shared__ __align__(16) bf16 sX[kTile * KP];
-  __shared__ __align__(16) bf16 sU[kTile * NP];
+  extern __shared__ __align__(16) unsigned char bwd_mem[];
+  bf16* sW = reinterpret_cast<bf16*>(bwd_mem);
+  bf16* sX0 = sW + (DX ? K2 * NP : 0);
+  bf16* sU0 = sX0 + 2 * kTile * KP;
   __shared__ float sdb[kH];
   if (DX) {
     for (int idx = threadIdx.x; idx < K2 * (kH / 8); idx += blockDim.x) {
@@ -843,62 +963,71 @@ __global__ void __launch_bounds__(kLayerThreads, 2)
       *reinterpret_cast<uint4*>(sW + k * NP + cc * 8) = *reinterpret_cast<const uint4*>(W + k * kH + cc * 8);
     }
   }
-  if (threadIdx.x < kH) sdb[threadIdx.x] = 0.0f;
+  if (TOP && threadIdx.x < kH) sdb[threadIdx.x] = 0.0f;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
-  const int half = lane >> 4, hl = lane & 15;  // two rows per warp, four columns per lane
   const int wm = wid & 3, wn = wid >> 2;
-  const int n = v.n;
   float accW[MT][4];
 #pragma unroll
   for (int i = 0; i < MT; ++i) accW[i][0] = accW[i][1] = accW[i][2] = accW[i][3] = 0.0f;
-  float dbp[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  for (int tile = blockIdx.x; tile * kTile < n; tile += gridDim.x) {
+  // u of a tile: this thread's 16-byte chunk uq of rows ur and ur + 32
+  const int ur = threadIdx.x / 8, uq = threadIdx.x % 8;
+  float wo[8] = {}, db[8] = {};
+  if (TOP)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) wo[i] = __ldg(w_head + 8 * uq + i);
+  // tile -> stage; rows past n are zero
+  auto copy = [&](int tile, int stage) {
     const int r0 = tile * kTile;
-    __syncthreads();
-    for (int rl = wid * 2 + half; rl < kTile; rl += 16) {
-      const int r = r0 + rl;
-      float u[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-      if (r < n) {
-        const float4 d4 = *reinterpret_cast<const float4*>(direct + static_cast<size_t>(r) * kH + 4 * hl);
-        float dv[4] = {d4.x, d4.y, d4.z, d4.w};
-        if (AGG) {
-          float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-          aggregate_row<kH>(v, c, da_src, partial, r, hl, acc);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) dv[i] += acc[i];
-        }
-        const uint2 hraw = RowIO<kH>::load(hn, r, hl);
-        bf162 p0, p1;
-        memcpy(&p0, &hraw.x, 4);
-        memcpy(&p1, &hraw.y, 4);
-        const float2 h0 = __bfloat1622float2(p0), h1 = __bfloat1622float2(p1);
-        u[0] = h0.x > 0.0f ? dv[0] : 0.0f;
-        u[1] = h0.y > 0.0f ? dv[1] : 0.0f;
-        u[2] = h1.x > 0.0f ? dv[2] : 0.0f;
-        u[3] = h1.y > 0.0f ? dv[3] : 0.0f;
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) dbp[i] += u[i];
-      uint2 packed;
-      packed.x = pack_bf162(u[0], u[1]);
-      packed.y = pack_bf162(u[2], u[3]);
-      *reinterpret_cast<uint2*>(sU + rl * NP + 4 * hl) = packed;
-    }
-    // X = [h, a], both bf16, 16-byte chunks
+    bf16 *sX = sX0 + stage * kTile * KP, *sU = sU0 + stage * kTile * NP;
+    auto put = [&](bf16* to, const bf16* from, bool ok) {
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(to)), "l"(from), "r"(ok ? 16 : 0)
+                   : "memory");
+    };
     constexpr int HC = D / 8, CH = 2 * HC;
-    for (int idx = threadIdx.x; idx < kTile * CH; idx += blockDim.x) {
+#pragma unroll
+    for (int idx = threadIdx.x; idx < kTile * CH; idx += kLayerThreads) {
       const int rl = idx / CH, ch = idx % CH;
-      const int row = r0 + rl;
-      uint4 val = make_uint4(0, 0, 0, 0);
-      if (row < n) {
-        const bf16* srcp = ch < HC ? h + static_cast<size_t>(row) * D + ch * 8
-                                   : a + static_cast<size_t>(row) * D + (ch - HC) * 8;
-        val = __ldg(reinterpret_cast<const uint4*>(srcp));
-      }
-      *reinterpret_cast<uint4*>(sX + rl * KP + ch * 8) = val;
+      const bool ok = r0 + rl < n;
+      const size_t row = static_cast<size_t>(ok ? r0 + rl : 0);
+      put(sX + rl * KP + ch * 8, ch < HC ? h + row * D + ch * 8 : a + row * D + (ch - HC) * 8, ok);
     }
-    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const bool ok = r0 + ur + 32 * i < n;
+      put(sU + (ur + 32 * i) * NP + 8 * uq, u + static_cast<size_t>(ok ? r0 + ur + 32 * i : 0) * kH + 8 * uq, ok);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const int tiles = (n + kTile - 1) / kTile;
+  int tile = blockIdx.x, stage = 0;
+  if (tile < tiles) copy(tile, 0);
+  for (; tile < tiles; tile += gridDim.x, stage ^= 1) {
+    const int r0 = tile * kTile;
+    float dzr[2] = {0.0f, 0.0f};
+    if (TOP)
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        if (r0 + ur + 32 * i < n) dzr[i] = __ldg(dz + r0 + ur + 32 * i);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    const bf16* sX = sX0 + stage * kTile * KP;
+    bf16* sU = sU0 + stage * kTile * NP;
+    if (TOP) {  // h' -> dU, each thread on the chunks it copied
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        uint4* p = reinterpret_cast<uint4*>(sU + (ur + 32 * i) * NP + 8 * uq);
+        float x[8];
+        RowIO<kH>::unpack(*p, x);
+#pragma unroll
+        for (int f = 0; f < 8; ++f) {
+          x[f] = x[f] > 0.0f ? dzr[i] * wo[f] : 0.0f;
+          db[f] += x[f];
+        }
+        *p = RowIO<kH>::pack(x);
+      }
+    }
+    __syncthreads();  // the tile is complete, and the other stage's readers are done
+    if (tile + static_cast<int>(gridDim.x) < tiles) copy(tile + gridDim.x, stage ^ 1);
     if (DX) {
       float acc[XN][4];
 #pragma unroll
@@ -959,9 +1088,10 @@ __global__ void __launch_bounds__(kLayerThreads, 2)
     atomicAdd(gW + (m + 8) * kH + j, accW[i][2]);
     atomicAdd(gW + (m + 8) * kH + j + 1, accW[i][3]);
   }
+  if (!TOP) return;
   __syncthreads();
 #pragma unroll
-  for (int i = 0; i < 4; ++i) atomicAdd(&sdb[4 * hl + i], dbp[i]);
+  for (int i = 0; i < 8; ++i) atomicAdd(&sdb[8 * uq + i], db[i]);
   __syncthreads();
   if (threadIdx.x < kH) atomicAdd(gb + threadIdx.x, sdb[threadIdx.x]);
 }
@@ -1073,9 +1203,11 @@ struct ising_gnn {
   bf16* d_h[3] = {nullptr, nullptr, nullptr};    // h1, h2, h3
   bf16* d_a[2] = {nullptr, nullptr};             // a^1, a^2 (bf16), kept for the backward pass
   float* d_z = nullptr;
+  float* d_dz = nullptr;                         // dL/dz
   int8_t* d_y = nullptr;
-  float* d_dh[2] = {nullptr, nullptr};           // direct parts of dL/dh
-  bf16* d_da[2] = {nullptr, nullptr};            // dL/da of two consecutive layers
+  float* d_dh = nullptr;                         // direct part of dL/dh
+  bf16* d_da = nullptr;                          // dL/da of the layer above
+  bf16* d_du = nullptr;                          // dU of a layer
   float* d_out = nullptr;  // logits in caller order (host copies)
   int64_t chunk_cap = 0;
   float* d_partial = nullptr;  // per heavy-row chunk: its partial sum (width 64)
@@ -1089,16 +1221,16 @@ namespace {
 void free_work(ising_gnn* net) {
   void* ptrs[] = {net->d_sums,  net->d_c,     net->d_x,     net->d_a0,    net->d_h[0],
                   net->d_h[1],  net->d_h[2],  net->d_a[0],  net->d_a[1],  net->d_z,
-                  net->d_y,     net->d_dh[0], net->d_dh[1], net->d_da[0], net->d_da[1],
-                  net->d_out};
+                  net->d_y,     net->d_dh,    net->d_da,    net->d_du,    net->d_out,
+                  net->d_dz};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   net->d_sums = nullptr;
-  net->d_c = net->d_z = net->d_out = nullptr;
+  net->d_c = net->d_z = net->d_out = net->d_dz = nullptr;
   net->d_x = net->d_a0 = nullptr;
   net->d_h[0] = net->d_h[1] = net->d_h[2] = nullptr;
-  net->d_a[0] = net->d_a[1] = net->d_da[0] = net->d_da[1] = nullptr;
-  net->d_dh[0] = net->d_dh[1] = nullptr;
+  net->d_a[0] = net->d_a[1] = net->d_da = net->d_du = nullptr;
+  net->d_dh = nullptr;
   net->d_y = nullptr;
   net->n_cap = 0;
 }
@@ -1127,12 +1259,13 @@ cudaError_t ensure_work(ising_gnn* net, int64_t n) {
   if ((e = dalloc(&net->d_a0, N * kF)) != cudaSuccess) return e;
   for (int l = 0; l < 3; ++l)
     if ((e = dalloc(&net->d_h[l], N * kH)) != cudaSuccess) return e;
-  for (int l = 0; l < 2; ++l) {
+  for (int l = 0; l < 2; ++l)
     if ((e = dalloc(&net->d_a[l], N * kH)) != cudaSuccess) return e;
-    if ((e = dalloc(&net->d_dh[l], N * kH)) != cudaSuccess) return e;
-    if ((e = dalloc(&net->d_da[l], N * kH)) != cudaSuccess) return e;
-  }
+  if ((e = dalloc(&net->d_dh, N * kH)) != cudaSuccess) return e;
+  if ((e = dalloc(&net->d_da, N * kH)) != cudaSuccess) return e;
+  if ((e = dalloc(&net->d_du, N * kH)) != cudaSuccess) return e;
   if ((e = dalloc(&net->d_z, N)) != cudaSuccess) return e;
+  if ((e = dalloc(&net->d_dz, N)) != cudaSuccess) return e;
   if ((e = dalloc(&net->d_y, N)) != cudaSuccess) return e;
   if ((e = dalloc(&net->d_out, N)) != cudaSuccess) return e;
   net->n_cap = n;
@@ -1178,23 +1311,13 @@ struct Ctx {
   const int32_t* vbase;  // per position: the instance's first position (null: none)
 };
 
-// Row ids and heavy-row chunks of a row table, built once per graph and kept
-// by its owner: rowid[e] = row of entry e; hchunk[r] = index of row r's first
-// chunk if r has more than kHeavy entries, else -1; chunk_row[k] = row of
-// chunk k. A graph without heavy rows keeps no chunk arrays.
-cudaError_t build_row_tables(const int32_t* d_row_ptr, int n, long long nnz, cudaStream_t st, int sms,
-                             int32_t** rowid, int32_t** hchunk, int32_t** chunk_row, int32_t* num_chunks,
-                             uint64_t* launches) {
+// Heavy-row chunks of a row table, built once per graph and kept by its owner:
+// hchunk[r] = index of row r's first chunk if r has more than kHeavy entries,
+// else -1; chunk_row[k] = row of chunk k. A graph without heavy rows keeps no
+// chunk arrays.
+cudaError_t build_row_tables(const int32_t* d_row_ptr, int n, cudaStream_t st, int32_t** hchunk,
+                             int32_t** chunk_row, int32_t* num_chunks) {
   cudaError_t e = cudaSuccess;
-  if (*rowid == nullptr) {
-    if ((e = dalloc(rowid, static_cast<size_t>(nnz))) != cudaSuccess) {
-      *rowid = nullptr;
-      return e;
-    }
-    rowid_kernel<<<grid_of(n, 256, sms * 8), 256, 0, st>>>(d_row_ptr, n, *rowid);
-    (*launches)++;
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
   if (*num_chunks >= 0) return cudaSuccess;
   std::vector<int32_t> rp(static_cast<size_t>(n) + 1);
   if ((e = cudaMemcpyAsync(rp.data(), d_row_ptr, rp.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st)) !=
@@ -1229,8 +1352,8 @@ cudaError_t build_row_tables(const int32_t* d_row_ptr, int n, long long nnz, cud
 }
 
 int graph_ctx(ising_gnn* net, ising_graph* g, Ctx* ctx) {
-  GNN_CUDA(net, build_row_tables(g->d_row_ptr, g->n, g->nnz, g->stream, g->num_sms, &g->d_rowid,
-                                 &g->d_gnn_hchunk, &g->d_gnn_chunk_row, &g->gnn_num_chunks, &net->launches));
+  GNN_CUDA(net, build_row_tables(g->d_row_ptr, g->n, g->stream, &g->d_gnn_hchunk, &g->d_gnn_chunk_row,
+                                 &g->gnn_num_chunks));
   GView& v = ctx->v;
   v.n = g->n;
   v.nnz = g->nnz;
@@ -1240,7 +1363,6 @@ int graph_ctx(ising_gnn* net, ising_graph* g, Ctx* ctx) {
   v.ev.w = g->d_w;
   v.ev.packed = g->packed ? 1 : 0;
   v.vbase = nullptr;
-  v.rowid = g->d_rowid;
   v.spins = reinterpret_cast<const uint8_t*>(g->d_spins);
   v.shift = 0;
   v.num_chunks = g->gnn_num_chunks;
@@ -1259,8 +1381,7 @@ int batch_ctx(ising_gnn* net, ising_batch* b, uint32_t replica, Ctx* ctx, isingx
   int rc = isingx::batch_union(b, u);
   if (rc != ISING_OK) return rc;
   if (u->device != net->device || replica >= static_cast<uint32_t>(u->replicas)) return ISING_EINVAL;
-  GNN_CUDA(net, build_row_tables(u->row_ptr, u->n, u->nnz, u->stream, u->num_sms, u->rowid, u->hchunk,
-                                 u->chunk_row, u->num_chunks, &net->launches));
+  GNN_CUDA(net, build_row_tables(u->row_ptr, u->n, u->stream, u->hchunk, u->chunk_row, u->num_chunks));
   GView& v = ctx->v;
   v.n = u->n;
   v.nnz = u->nnz;
@@ -1270,7 +1391,6 @@ int batch_ctx(ising_gnn* net, ising_batch* b, uint32_t replica, Ctx* ctx, isingx
   v.ev.w = nullptr;
   v.ev.packed = 1;
   v.vbase = u->vbase;
-  v.rowid = *u->rowid;
   v.spins = u->spins;
   v.shift = static_cast<int>(replica);
   v.num_chunks = *u->num_chunks;
@@ -1336,23 +1456,21 @@ int check_err(ising_gnn* net) {
 }
 
 // Forward pass over the graph from its current spins; with labels (by
-// position in net->d_y) also the loss and dL/dh3 into net->d_dh[0], and the
+// position in net->d_y) also the loss and dL/dz into net->d_dz, and the
 // aggregates a^l kept for the backward pass.
 int run_forward(ising_gnn* net, const Ctx& x, bool with_labels) {
   const int n = x.v.n;
-  const long long nnz = x.v.nnz;
   cudaStream_t st = x.st;
   const int sms = x.sms;
   GNN_CUDA(net, ensure_work(net, n));
   GNN_CUDA(net, ensure_partial(net, x.v.num_chunks));
-  const int ent_grid = grid_of((nnz + 31) / 32 * 32, 256, sms * 16);
-  GNN_CUDA(net, cudaMemsetAsync(net->d_sums, 0, sizeof(int4) * static_cast<size_t>(n), st));
-  if (nnz > 0) {
-    rowsum_kernel<<<ent_grid, 256, 0, st>>>(x.v, net->d_sums);
+  if (x.v.num_chunks > 0) {
+    GNN_CUDA(net, cudaMemsetAsync(net->d_sums, 0, sizeof(int4) * static_cast<size_t>(n), st));
+    chunk_sums_kernel<<<grid_of(static_cast<long long>(x.v.num_chunks) * 32, 256, sms * 16), 256, 0, st>>>(x.v, net->d_sums);
     net->launches++;
   }
-  features_kernel<<<grid_of(n, 256, sms * 8), 256, 0, st>>>(x.v, net->d_sums, reinterpret_cast<uint4*>(net->d_x),
-                                                             net->d_c);
+  features_kernel<<<grid_of(static_cast<long long>(n) * 4, 256, sms * 16), 256, 0, st>>>(
+      x.v, net->d_sums, reinterpret_cast<uint4*>(net->d_x), net->d_c);
   net->launches++;
   GNN_CUDA(net, cudaGetLastError());
   int rc = run_chunks<kF>(net, x, net->d_x);
@@ -1369,9 +1487,9 @@ int run_forward(ising_gnn* net, const Ctx& x, bool with_labels) {
     if (rc != ISING_OK) return rc;
   }
   if (with_labels) GNN_CUDA(net, cudaMemsetAsync(net->d_loss, 0, sizeof(double), st));
-  head_kernel<<<grid_of(static_cast<long long>(n) * 32, 256, sms * 8), 256, 0, st>>>(
+  head_kernel<<<grid_of(n, 256, sms * 8), 256, 0, st>>>(
       reinterpret_cast<const bf162*>(net->d_h[2]), net->d_params, with_labels ? net->d_y : nullptr, n,
-      1.0f / static_cast<float>(n), net->d_z, net->d_dh[0], net->d_grad, net->d_loss);
+      1.0f / static_cast<float>(n), net->d_z, net->d_dz, net->d_grad, net->d_loss);
   net->launches++;
   GNN_CUDA(net, cudaGetLastError());
   return ISING_OK;
@@ -1379,34 +1497,48 @@ int run_forward(ising_gnn* net, const Ctx& x, bool with_labels) {
 
 // Backward pass after run_forward(with_labels): gradients into net->d_grad
 // (zeroed by the caller before the head kernel ran).
-int run_backward(ising_gnn* net, const Ctx& x) {
-  const int n = x.v.n;
-  cudaStream_t st = x.st;
+template <int D, bool DX, bool TOP>
+int run_products(ising_gnn* net, const Ctx& x, const bf16* u, const bf16* h, const bf16* a, const bf16* W, int off_w,
+                 int off_b, float* dh_out, bf16* da_out) {
+  constexpr int smem = bwd_smem<D>(DX);
+  const auto kernel = bwd_products_kernel<D, DX, TOP>;
+  GNN_CUDA(net, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   // two blocks per SM (registers); each keeps its dW partial sums to the end
-  const int grid = grid_of((n + kTile - 1) / kTile, 1, x.sms * 2);
-  // layer 2: dL/dh3 (d_dh[0]) -> direct part of dL/dh2 (d_dh[1]), dL/da2 (d_da[0])
-  layer_bwd_kernel<kH, true, false><<<grid, kLayerThreads, 0, st>>>(
-      x.v, net->d_c, net->d_dh[0], nullptr, nullptr, net->d_h[2], net->d_h[1], net->d_a[1], net->d_w2,
-      net->d_grad + kOffW2, net->d_grad + kOffB2, net->d_dh[1], net->d_da[0]);
-  net->launches++;
-  GNN_CUDA(net, cudaGetLastError());
-  // layer 1: dL/dh2 = d_dh[1] + A_hat d_da[0] -> d_dh[0], d_da[1]
-  int rc = run_chunks<kH>(net, x, net->d_da[0]);
-  if (rc != ISING_OK) return rc;
-  layer_bwd_kernel<kH, true, true><<<grid, kLayerThreads, 0, st>>>(
-      x.v, net->d_c, net->d_dh[1], net->d_da[0], net->d_partial, net->d_h[1], net->d_h[0], net->d_a[0],
-      net->d_w1, net->d_grad + kOffW1, net->d_grad + kOffB1, net->d_dh[0], net->d_da[1]);
-  net->launches++;
-  GNN_CUDA(net, cudaGetLastError());
-  // layer 0: dL/dh1 = d_dh[0] + A_hat d_da[1]
-  rc = run_chunks<kH>(net, x, net->d_da[1]);
-  if (rc != ISING_OK) return rc;
-  layer_bwd_kernel<kF, false, true><<<grid, kLayerThreads, 0, st>>>(
-      x.v, net->d_c, net->d_dh[0], net->d_da[1], net->d_partial, net->d_h[0], net->d_x, net->d_a0, net->d_w0,
-      net->d_grad + kOffW0, net->d_grad + kOffB0, nullptr, nullptr);
+  const int grid = grid_of((x.v.n + kTile - 1) / kTile, 1, x.sms * 2);
+  kernel<<<grid, kLayerThreads, smem, x.st>>>(x.v.n, u, net->d_dz, h, a, W, net->d_params + kOffWo,
+                                              net->d_grad + off_w, net->d_grad + off_b, dh_out, da_out);
   net->launches++;
   GNN_CUDA(net, cudaGetLastError());
   return ISING_OK;
+}
+
+// dU of a layer below the top one into net->d_du.
+int run_dpre(ising_gnn* net, const Ctx& x, const float* direct, const bf16* da, const bf16* hn, int off_b) {
+  const int rc = run_chunks<kH>(net, x, da);
+  if (rc != ISING_OK) return rc;
+  dpre_kernel<<<grid_of(static_cast<long long>(x.v.n) * RowIO<kH>::G, 256, x.sms * 16), 256, 0, x.st>>>(
+      x.v, net->d_c, direct, da, net->d_partial, hn, net->d_du, net->d_grad + off_b);
+  net->launches++;
+  GNN_CUDA(net, cudaGetLastError());
+  return ISING_OK;
+}
+
+int run_backward(ising_gnn* net, const Ctx& x) {
+  // layer 2: dL/dh3 = d_dz w_o -> direct part of dL/dh2 (d_dh), dL/da2 (d_da)
+  int rc = run_products<kH, true, true>(net, x, net->d_h[2], net->d_h[1], net->d_a[1], net->d_w2, kOffW2, kOffB2,
+                                        net->d_dh, net->d_da);
+  if (rc != ISING_OK) return rc;
+  // layer 1: dL/dh2 = d_dh + A_hat d_da -> dU, then d_dh and d_da of layer 0
+  rc = run_dpre(net, x, net->d_dh, net->d_da, net->d_h[1], kOffB1);
+  if (rc != ISING_OK) return rc;
+  rc = run_products<kH, true, false>(net, x, net->d_du, net->d_h[0], net->d_a[0], net->d_w1, kOffW1, kOffB1,
+                                     net->d_dh, net->d_da);
+  if (rc != ISING_OK) return rc;
+  // layer 0: dL/dh1 = d_dh + A_hat d_da
+  rc = run_dpre(net, x, net->d_dh, net->d_da, net->d_h[0], kOffB0);
+  if (rc != ISING_OK) return rc;
+  return run_products<kF, false, false>(net, x, net->d_du, net->d_x, net->d_a0, net->d_w0, kOffW0, kOffB0, nullptr,
+                                        nullptr);
 }
 
 int load_labels(ising_gnn* net, const Ctx& x, const int8_t* labels, int on_device) {

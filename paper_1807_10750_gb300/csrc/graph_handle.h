@@ -129,7 +129,6 @@ struct ising_graph {
   int32_t* d_picks = nullptr;
   size_t pick_sweeps = 0, pick_cap = 0;
   uint8_t* d_bias = nullptr;         // per-position flip bias (null: none)
-  int32_t* d_rowid = nullptr;        // row of every CSR entry (built on first use)
   int32_t* d_gnn_hchunk = nullptr;   // warm-start network: per row, its first entry chunk or -1
   int32_t* d_gnn_chunk_row = nullptr;  // warm-start network: the row of every entry chunk
   int32_t gnn_num_chunks = -1;       // -1 until built
