@@ -148,7 +148,9 @@ enum {
                                   blocks sum the hubs' fields from the other vertices and run the
                                   other classes with a bounded grid barrier after each.
                                   Deterministic linear schedule (flip bias allowed); otherwise runs
-                                  as PERSISTENT_GRID */
+                                  as PERSISTENT_GRID. What AUTO runs as HUB takes the spin-map form
+                                  on one cluster of blocks while the spins fit in a block's shared
+                                  memory (about 115,000 vertices) */
 };
 
 /* ising_create flags. */

@@ -508,7 +508,7 @@ void free_device(ising_graph* g) {
                   g->d_hub_flips, g->d_hub_bits, g->d_hub_pflips, g->d_hub_blk,
                   g->d_gnn_hchunk, g->d_gnn_chunk_row, g->d_map_blocks, g->d_map_task,
                   g->d_map_words, g->d_map_weights, g->d_map_row_pos, g->d_map_row_orig,
-                  g->d_map_class, g->d_map_steps, g->d_map_msg, g->d_map_index, g->d_map_mail,
+                  g->d_map_class, g->d_map_steps, g->d_map_msg, g->d_map_index, g->d_map_late, g->d_map_mail,
                   g->d_pick_count, g->d_picks};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -958,17 +958,21 @@ cudaError_t launch_hub(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint64
 template <int MODE>
 const void* map_kernel_of(bool wide, int stage) {
   using isingx::map_kernel;
-  if (wide) return stage <= 2 ? reinterpret_cast<const void*>(map_kernel<MODE, true, 2>)
-                              : reinterpret_cast<const void*>(map_kernel<MODE, true, 4>);
-  if (stage <= 1) return reinterpret_cast<const void*>(map_kernel<MODE, false, 1>);
-  if (stage <= 2) return reinterpret_cast<const void*>(map_kernel<MODE, false, 2>);
-  if (stage <= 4) return reinterpret_cast<const void*>(map_kernel<MODE, false, 4>);
-  return reinterpret_cast<const void*>(map_kernel<MODE, false, 8>);
+  if (wide) return stage <= 2 ? reinterpret_cast<const void*>(map_kernel<MODE, true, 2, false>)
+                              : reinterpret_cast<const void*>(map_kernel<MODE, true, 4, false>);
+  if (stage <= 1) return reinterpret_cast<const void*>(map_kernel<MODE, false, 1, false>);
+  if (stage <= 2) return reinterpret_cast<const void*>(map_kernel<MODE, false, 2, false>);
+  if (stage <= 4) return reinterpret_cast<const void*>(map_kernel<MODE, false, 4, false>);
+  return reinterpret_cast<const void*>(map_kernel<MODE, false, 8, false>);
 }
 
-const void* map_kernel_for(int mode, bool wide, int stage) {
+const void* map_kernel_for(int mode, bool wide, int stage, bool split) {
   if (mode == isingx::kMapBlock) return map_kernel_of<isingx::kMapBlock>(wide, stage);
   if (mode == isingx::kMapBlockStream) return map_kernel_of<isingx::kMapBlockStream>(wide, stage);
+  constexpr int kSplitG = isingx::kMapPartEntries / 128;
+  if (mode == isingx::kMapCluster && split)
+    return wide ? reinterpret_cast<const void*>(isingx::map_kernel<isingx::kMapCluster, true, kSplitG, true>)
+                : reinterpret_cast<const void*>(isingx::map_kernel<isingx::kMapCluster, false, kSplitG, true>);
   if (mode == isingx::kMapCluster) return map_kernel_of<isingx::kMapCluster>(wide, stage);
   return map_kernel_of<isingx::kMapGrid>(wide, stage);
 }
@@ -995,7 +999,7 @@ void map_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int mode, in
 // Whether the device can run a plan: shared memory, a cluster of that size, or
 // K co-resident blocks.
 bool map_fits(const isingx::MapPlan& mp, bool wide) {
-  const void* kernel = map_kernel_for(mp.mode, wide, mp.stage);
+  const void* kernel = map_kernel_for(mp.mode, wide, mp.stage, mp.hubs > 0);
   bool fits = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, mp.smem_bytes) == cudaSuccess;
   if (fits && mp.mode == isingx::kMapCluster) {
     fits = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
@@ -1027,20 +1031,22 @@ bool map_fits(const isingx::MapPlan& mp, bool wide) {
 // (100,000 vertices and 5M edges, 360,000 a class: 84 against 62 us). Lattices
 // wait for a halo plan: until then the cluster up to 100,000 vertices (9.8
 // against 11.6 us by item dataflow at 90,300, 14.3 against 13.3 at 160,000).
-void choose_map_plan(const HostGraph& hg, int num_sms, int device, bool wide, bool lattice,
+// Graphs with hubs (split) go to the cluster wherever their spins fit, up to
+// about 115,000 vertices (110,000: 65 us a sweep against 95 by the hub engine).
+void choose_map_plan(const HostGraph& hg, int num_sms, int device, bool wide, bool lattice, bool split,
                      isingx::MapPlan* mp) {
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
   const int64_t work = hg.nnz + 8 * static_cast<int64_t>(hg.n), classes = std::max(1, hg.num_colours);
   auto build = [&](int mode, int K) {
-    isingx::build_map_plan(hg, mode, K, wide, optin, mp);
+    isingx::build_map_plan(hg, mode, K, wide, optin, mp, split);
     return mp->ok && map_fits(*mp, wide);
   };
-  if (work <= 4000 * classes && (build(isingx::kMapBlock, 1) || build(isingx::kMapBlockStream, 1))) return;
+  if (!split && work <= 4000 * classes && (build(isingx::kMapBlock, 1) || build(isingx::kMapBlockStream, 1))) return;
   if ((lattice ? hg.n <= 100000 : work <= 300000 * classes) &&
       (build(isingx::kMapCluster, 16) || build(isingx::kMapCluster, 8)))
     return;
-  if (!lattice && build(isingx::kMapGrid, std::min(num_sms, std::max(1, hg.n / 32)))) return;
+  if (!split && !lattice && build(isingx::kMapGrid, std::min(num_sms, std::max(1, hg.n / 32)))) return;
   mp->ok = false;
 }
 
@@ -1072,15 +1078,18 @@ cudaError_t upload_map_plan(ising_graph* g, const isingx::MapPlan& mp) {
   if ((e = alloc_copy<unsigned long long>(&g->d_map_mail, nullptr,
                                            2 * static_cast<size_t>(mp.K) * static_cast<size_t>(mp.mail_stride), g->stream)) != cudaSuccess)
     return e;
+  if ((e = alloc_copy(&g->d_map_late, mp.late.data(), mp.late.size(), g->stream)) != cudaSuccess) return e;
+  const int2* late = reinterpret_cast<const int2*>(g->d_map_late);
   const dim3 grid(static_cast<unsigned>(mp.K), mp.mode == isingx::kMapGrid ? 4u : 32u);
   if (g->packed)
     isingx::map_fill_kernel<true><<<grid, 256, 0, g->stream>>>(
         g->dev(), g->d_map_blocks, reinterpret_cast<const int4*>(g->d_map_task), mp.warps, g->d_map_row_pos,
-        g->d_map_index, reinterpret_cast<int4*>(g->d_map_words), nullptr);
+        g->d_map_index, late, mp.hubs, reinterpret_cast<int4*>(g->d_map_words), nullptr);
   else
     isingx::map_fill_kernel<false><<<grid, 256, 0, g->stream>>>(
         g->dev(), g->d_map_blocks, reinterpret_cast<const int4*>(g->d_map_task), mp.warps, g->d_map_row_pos,
-        g->d_map_index, reinterpret_cast<int4*>(g->d_map_words), reinterpret_cast<int4*>(g->d_map_weights));
+        g->d_map_index, late, mp.hubs, reinterpret_cast<int4*>(g->d_map_words),
+        reinterpret_cast<int4*>(g->d_map_weights));
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   g->map_mode = mp.mode;
   g->map_K = mp.K;
@@ -1092,6 +1101,7 @@ cudaError_t upload_map_plan(ising_graph* g, const isingx::MapPlan& mp) {
   g->map_groups = mp.max_groups;
   g->map_stage = mp.stage;
   g->map_stride = mp.mail_stride;
+  g->map_accs = mp.max_acc;
   g->map_ok = true;
   return cudaSuccess;
 }
@@ -1099,7 +1109,7 @@ cudaError_t upload_map_plan(ising_graph* g, const isingx::MapPlan& mp) {
 cudaError_t launch_map(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint64_t T, uint64_t T0,
                        uint32_t replica, const isingx::PhiloxRounds& rk, uint32_t n0, int par0) {
   const bool wide = !g->packed;
-  const void* kernel = map_kernel_for(g->map_mode, wide, g->map_stage);
+  const void* kernel = map_kernel_for(g->map_mode, wide, g->map_stage, g->map_accs > 0);
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, g->map_smem);
   if (e != cudaSuccess) return e;
   if (g->map_mode == isingx::kMapCluster &&
@@ -1128,6 +1138,7 @@ cudaError_t launch_map(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint64
   a.tasks_max = g->map_tasks;
   a.rows_max = g->map_rows;
   a.groups_max = g->map_groups;
+  a.accs = g->map_accs;
   a.budget = g->wait_budget_ns > 0 ? static_cast<long long>(g->wait_budget_ns) : isingx::kBarrierBudgetNs;
   a.error = &g->d_barrier->error;
   a.skip_block = g->fault_kind == ISING_FAULT_SKIP_ARRIVAL ? 1 : 0;
@@ -1379,9 +1390,10 @@ int ising_create(int32_t n, int64_t m, const int32_t* src, const int32_t* dst, c
     // graphs the halo engine may take keep their host graph for its plan
     keep_host = g->packed && !block.ok && hg.num_colours <= isingx::kHaloMaxClasses &&
                 hg.max_degree <= isingx::kHaloMaxWidth && hg.n >= 64 * g->num_sms;
-    // small graphs and graphs without hubs: the spin-map engine
-    if (block.ok || hub_end.empty()) choose_map_plan(hg, g->num_sms, g->device, !g->packed, keep_host, &map_plan);
-    if (!map_plan.ok) have_deps = isingx::build_item_deps(hg, plan, &dep_ptr, &deps);
+    // the spin-map engine; graphs with hubs keep the engines that AUTO does not pick
+    const bool split = !block.ok && !hub_end.empty();
+    choose_map_plan(hg, g->num_sms, g->device, !g->packed, keep_host, split, &map_plan);
+    if (!map_plan.ok || split) have_deps = isingx::build_item_deps(hg, plan, &dep_ptr, &deps);
   } catch (const std::bad_alloc&) {
     delete g;
     return ISING_ENOMEM;
@@ -1667,7 +1679,11 @@ static int anneal_impl(ising_graph* g, const ising_schedule* sched, uint32_t swe
   }
   if (engine == ISING_ENGINE_HUB) {
     if (mode == ISING_MODE_DET && !nflip && g->hub_ok) {
-      const cudaError_t e = launch_hub(g, sched->t_begin, sweeps, sched->t_total, T0, sched->replica, rk);
+      // AUTO: the spin-map engine's form for graphs with hubs, where there is a plan
+      const bool map = g->engine == ISING_ENGINE_AUTO && g->map_ok && g->fault_kind != ISING_FAULT_SHORT_COPY;
+      const cudaError_t e =
+          map ? launch_map(g, sched->t_begin, sweeps, sched->t_total, T0, sched->replica, rk, 0u, par0)
+              : launch_hub(g, sched->t_begin, sweeps, sched->t_total, T0, sched->replica, rk);
       if (e == cudaSuccess) {
         g->engine_used = ISING_ENGINE_HUB;
         return ISING_OK;
@@ -1690,7 +1706,7 @@ static int anneal_impl(ising_graph* g, const ising_schedule* sched, uint32_t swe
   }
   // the spin-map form of the block engine, of the item-dataflow engine and of
   // what AUTO runs as PERSISTENT
-  const bool use_map = g->map_ok && mode == ISING_MODE_DET && g->fault_kind != ISING_FAULT_SHORT_COPY &&
+  const bool use_map = g->map_ok && g->map_accs == 0 && mode == ISING_MODE_DET && g->fault_kind != ISING_FAULT_SHORT_COPY &&
                        (engine == ISING_ENGINE_ITEMFLOW ||
                         (engine == ISING_ENGINE_PERSISTENT && (g->block_ok || g->engine == ISING_ENGINE_AUTO)));
   if (use_map && !(engine == ISING_ENGINE_ITEMFLOW && (nflip || !unsliced))) {

@@ -113,7 +113,7 @@ struct ising_graph {
   // spin-map engine (map.cuh)
   bool map_ok = false;
   int map_mode = 0, map_K = 0, map_warps = 0, map_smem = 0;
-  int32_t map_bytes = 0, map_tasks = 0, map_rows = 0, map_groups = 0, map_stage = 0, map_stride = 0;
+  int32_t map_bytes = 0, map_tasks = 0, map_rows = 0, map_groups = 0, map_stage = 0, map_stride = 0, map_accs = 0;
   isingx::MapBlock* d_map_blocks = nullptr;
   isingx::MapTask* d_map_task = nullptr;
   int32_t* d_map_words = nullptr;
@@ -124,6 +124,7 @@ struct ising_graph {
   int32_t* d_map_steps = nullptr;      // class_bytes, class_msg: C + 1 each
   int32_t* d_map_msg = nullptr;
   int32_t* d_map_index = nullptr;      // position -> map index
+  int32_t* d_map_late = nullptr;       // per split row: its entries in the class before
   unsigned long long* d_map_mail = nullptr;
   uint32_t* d_pick_count = nullptr;    // Algorithm 1's picks of a launch (grown on use)
   int32_t* d_picks = nullptr;

@@ -225,11 +225,23 @@ void build_halo_plan(const HostGraph& g, int32_t parts, int32_t sweeps_per_epoch
 // A block's work of a sweep is a table of rounds of `warps` tasks, class by
 // class; a task is a unit, a word of 32 flip draws for the next sweep, both
 // or neither. The draws go to the warps without a unit where there are any.
+//
+// Split rows (a cluster's plan of a graph with hubs): a hub's unit sums only
+// its neighbours in the class before; the other entries are summed while that
+// class's spins are on their way, in parts of kMapPartEntries entries, each a
+// task of that class's rounds in some block (entry 32 (4 g + k) + l of the part
+// in word 4 g + k of lane l) that adds into the row's partial sum in its own
+// block's shared memory.
 constexpr int32_t kMapSlots = 16;
 constexpr int32_t kMapMaxWarps = 16;
 constexpr int32_t kMapMaxBlocks = 1024;
 constexpr int32_t kMapMaxDegree = 4096;
 constexpr int32_t kMapMaxVertices = 200 * 1024;
+constexpr int32_t kMapSplitShift = 18;  // rows of a block below 2^18
+constexpr int32_t kMapMaxSplit = (1 << (31 - kMapSplitShift)) - 2;  // split rows of a block, parts of a row
+constexpr int32_t kMapPart = 6;
+constexpr int32_t kMapPartEntries = 256;
+constexpr int32_t kMapOwnerShift = 14;  // partial sums of a block below 2^14, 16 blocks
 constexpr int32_t kMapFlipShift = 18;  // map indices below 2^18, flip words below 2^14 - 1
 // One block with its entries in shared memory, or read from L2 as in the other
 // two: the blocks of one cluster, and one block per SM.
@@ -237,9 +249,11 @@ enum MapMode { kMapBlock = 0, kMapBlockStream = 1, kMapCluster = 2, kMapGrid = 3
 
 struct MapTask {
   int32_t words;  // first group of the unit within its block's groups
-  int32_t base;   // map index of the unit's first row | (flip word + 1) << kMapFlipShift
+  int32_t base;   // map index of the unit's first row | (flip word + 1) << kMapFlipShift;
+                  // a part: its row's partial sum | its block << kMapOwnerShift | the same
   int32_t row;    // its first row among the block's rows | 1 << 31 on a class's last round
-  int32_t shape;  // rows | log2(L) << 8 | groups << 16; 0: no unit
+                  // | (partial sum of a split row + 1, or a part's number) << kMapSplitShift
+  int32_t shape;  // rows | log2(L) << 8 | groups << 16; 0: no unit; L = kMapPart: a part
 };
 
 // Per block, offsets into the flat arrays.
@@ -247,7 +261,7 @@ struct MapBlock {
   int32_t task0, rounds;   // `tasks`: rounds * warps entries
   int32_t words0, groups;  // the entries (in groups of 32 int4)
   int32_t row0, rows;      // `row_pos`, `row_orig` (rows a multiple of 32)
-  int32_t pad0, pad1;
+  int32_t last0, pad1;     // the block's first task of the last class
 };
 
 struct MapPlan {
@@ -257,6 +271,7 @@ struct MapPlan {
   int32_t map_bytes = 0;     // bytes of the map (a multiple of 16)
   int32_t mail_stride = 0;   // messages of the largest class (grid)
   int32_t max_tasks = 0, max_rows = 0, max_groups = 0;  // over the blocks
+  int32_t hubs = 0, max_acc = 0;           // split rows (positions below `hubs`), the most of a block
   int32_t smem_bytes = 0;
   std::vector<MapBlock> blocks;
   std::vector<MapTask> tasks;
@@ -264,28 +279,34 @@ struct MapPlan {
   std::vector<int32_t> row_pos, row_orig;  // per block row: position and caller id, -1 for padding
   std::vector<int32_t> class_row;   // K x (C + 1): a block's first row of every class
   std::vector<int32_t> class_seg;   // K x (C + 1): the map index of that row
-  std::vector<int32_t> block_msg;   // K x (C + 1): its first message of every class (grid)
+  std::vector<int32_t> block_msg;   // K x (C + 1): its first message of every class (grid);
+                                    // split rows: bytes of the partial sums it receives
   std::vector<int32_t> class_bytes; // C + 1: bytes every block receives in a class (cluster)
   std::vector<int32_t> class_msg;   // C + 1: first message of every class (grid)
   std::vector<int32_t> msg;         // per message of 32 rows: (map index / 4) << 4 | words it
                                     // fills; every block has one or more per class
   std::vector<int32_t> map_index;   // position -> map index
+  std::vector<int32_t> late;        // per split row: its entries [first, end) in the class before
 };
 
 // Fills mp (ok = true) for K blocks of `mode` and `warps` warps when the graph
 // has at most kMapMaxVertices vertices and kMapMaxDegree entries a row and a
 // block's tables fit in smem_limit bytes, its entries among them in mode
-// kMapBlock. wide: 32-bit weights.
-void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int64_t smem_limit, MapPlan* mp);
+// kMapBlock. wide: 32-bit weights. split: the hubs' rows are split (kMapCluster
+// only; they may be longer than kMapMaxDegree).
+void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int64_t smem_limit, MapPlan* mp,
+                    bool split = false);
 
 // Shared memory of a block (map.cuh lays it out in this order): the map, the
 // resident entries (and weights), the tasks, the class tables (rows, map
 // segments, messages or received bytes, class messages), the rows' ids, two
-// sweeps of flip bits, the rows' biases, and 64 bytes for the barriers.
+// sweeps of flip bits, the rows' biases, 64 bytes for the barriers, and the
+// split rows' partial sums.
 inline int64_t map_smem_bytes(int32_t map_bytes, int64_t entry_groups, int32_t tasks, int32_t classes,
-                              int32_t rows) {
+                              int32_t rows, int32_t accs = 0) {
   return int64_t(map_bytes) + entry_groups * 512 + int64_t(tasks) * 16 + 4 * ((int64_t(classes) + 4) / 4 * 4) * 4 +
-         int64_t(rows) * 4 + int64_t(rows) / 32 * 8 + int64_t(rows) + 64;
+         int64_t(rows) * 4 + int64_t(rows) / 32 * 8 + int64_t(rows) + 64 +
+         (accs > 0 ? 4 * (int64_t(accs) + 32) : 0);
 }
 
 // Returns 0, or a negative ISING_* status.

@@ -40,6 +40,19 @@
 // classes, cluster: 48 -> 6.4; 30,011 vertices, 600k wide edges, 16 classes,
 // cluster: 97 -> 17; 100,000 vertices, 5M edges, 30 classes, grid: 253 -> 62.
 //
+// Graphs with hubs (SPLIT). A power-law graph's hubs form a near-clique, so it
+// has tens of classes of a few hubs each, whose rows hold thousands of entries;
+// a row summed by one warp, in its own step, made that step 1 to 2 us. Only the
+// terms from the class before need the step to wait: the rest of a row is
+// summed one step earlier, in parts of 256 entries that go to whichever block
+// has the fewest tasks then, and reach the row's partial sum with a red.async
+// counted on the same mbarrier as the spins. A step is then its exchange (0.55
+// to 0.8 us). Two staged groups: the units' padding is what more would cost (67
+// against 63 us a sweep at four). Microseconds a sweep on power-law graphs, int8
+// weights, engine before (hub.cuh, one block for the hub classes) / rows whole /
+// split, parts in the row's own block / as it is: 5,000 vertices 46 / 17 / 16 /
+// 16, 20,000 vertices 63 / 48 / 34 / 32, 100,000 vertices 93 / 154 / 83 / 63.
+//
 // Every wait is bounded (the handle's budget): then the error flag is set,
 // every block leaves its loop, and the blocks of a cluster meet once more
 // before they exit, so that no store reaches a block that has gone.
@@ -78,6 +91,7 @@ struct MapArgs {
   const uint32_t* pick_count;  // Algorithm 1: flips after each sweep of the launch (or null)
   const int32_t* picks;        // their map indices, pick_stride per sweep
   int32_t pick_stride;
+  int32_t accs;                // split rows of a block, at most
 };
 
 // The bounded wait for a message of sequence number seq.
@@ -139,7 +153,8 @@ __device__ __forceinline__ int map_row_sum(int f, int lg) {
 }
 
 // K blocks; sweeps t_begin .. t_begin + sweeps - 1.
-template <int MODE, bool WIDE, int G>
+// SPLIT: a cluster's plan with split rows (no Algorithm 1); G covers a part.
+template <int MODE, bool WIDE, int G, bool SPLIT>
 __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
     map_kernel(DevGraph d, MapArgs a, uint64_t t_begin, uint32_t sweeps, uint64_t T, uint64_t T0,
                uint32_t replica, PhiloxRounds rk) {
@@ -167,13 +182,17 @@ __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
   uint64_t* bars = reinterpret_cast<uint64_t*>(bias + a.rows_max);
   const int flip_words = a.rows_max / 32;
 
+  int32_t* acc = reinterpret_cast<int32_t*>(bars + 8);
+  if (SPLIT)
+    for (int i = tid; i < a.accs + 32; i += threads) acc[i] = 0;
   for (int p = tid; p < a.n; p += threads)
     map[__ldg(a.map_index + p)] = static_cast<int8_t>(spin_of(d.spins[p]));
   for (int i = tid; i < B.rounds * warps; i += threads) tasks[i] = __ldg(a.tasks + B.task0 + i);
   for (int c = tid; c <= C; c += threads) {
     crow[c] = __ldg(a.class_row + k_me * (C + 1) + c);
     cseg[c] = __ldg(a.class_seg + k_me * (C + 1) + c);
-    cbytes[c] = MODE == kMapGrid ? __ldg(a.block_msg + k_me * (C + 1) + c) : __ldg(a.class_bytes + c);
+    cbytes[c] = MODE == kMapGrid || SPLIT ? __ldg(a.block_msg + k_me * (C + 1) + c) : 0;
+    if (MODE != kMapGrid) cbytes[c] += __ldg(a.class_bytes + c);
     cmsg[c] = __ldg(a.class_msg + c);
   }
   for (int r = tid; r < B.rows; r += threads) {
@@ -246,6 +265,30 @@ __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
       }
     }
   };
+  // where a part's row has its partial sum: the address in that block of the
+  // address `at` here, plus the sum's place with sum = 1
+  auto owner = [&](uint32_t at, int sum, const int4& task) {
+    const int to = (task.y & ((1 << kMapFlipShift) - 1)) >> kMapOwnerShift;
+    return cluster_addr(at + 4 * sum * (task.y & ((1 << kMapOwnerShift) - 1)), to);
+  };
+  if (SPLIT) {
+    // the parts of the first class, which later sweeps sum in the last class's
+    // step, once every block has its map and cleared its partial sums
+    cluster_sync();
+    for (int i = B.last0 + warp; i < B.rounds * warps; i += warps) {
+      const int4 x = tasks[i];
+      if (((x.w >> 8) & 0xff) != kMapPart) continue;
+      int f = 0;
+      for (int g = 0; g < (x.w >> 16); ++g) {
+        const int4 w = __ldg(words + (x.x + g) * 32);
+        f += map_group<WIDE>(map, w, WIDE ? __ldg(weights + (x.x + g) * 32) : w);
+      }
+      f = __reduce_add_sync(kFullMask, f);
+      if (lane == 0)
+        asm volatile("red.relaxed.cluster.shared::cluster.add.s32 [%0], %1;" ::"r"(owner(smem_u32(acc), 1, x)), "r"(f)
+                     : "memory");
+    }
+  }
   const int4* const tasks_end = tasks + B.rounds * warps;
   const int4* next = tasks + warp;  // the task after the staged one
   int4 t = *next;
@@ -281,12 +324,24 @@ __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
     }
     for (int c = 0; c < C;) {
       const int draw = static_cast<int>(static_cast<unsigned>(t.y) >> kMapFlipShift) - 1;
-      if (t.w != 0) {
+      if (SPLIT && ((t.w >> 8) & 0xff) == kMapPart) {
+        int f = 0;
+#pragma unroll
+        for (int g = 0; g < G; ++g) f += map_group<WIDE>(map, st.w[g], st.c[WIDE ? g : 0]);
+        f = __reduce_add_sync(kFullMask, f);
+        if (lane == 0 && ok && !skip)
+          asm volatile("red.async.relaxed.cluster.shared::cluster.mbarrier::complete_tx::bytes.add.s32 [%0], %1, [%2];" ::"r"(
+                           owner(smem_u32(acc), 1, t)),
+                       "r"(f), "r"(owner(bar + 8 * (step & 1u), 0, t))
+                       : "memory");
+      } else if (t.w != 0) {
         // 1. the unit's fields
         const int lg = (t.w >> 8) & 0xff, groups = t.w >> 16;
         const int r = lane & ((32 >> lg) - 1);
-        const int own = (t.y & ((1 << kMapFlipShift) - 1)) + r, row = (t.z & 0x7fffffff) + r;
-        int f = 0;
+        const int own = (t.y & ((1 << kMapFlipShift) - 1)) + r, row = (t.z & ((1 << kMapSplitShift) - 1)) + r;
+        const int part = SPLIT ? static_cast<int>((t.z & 0x7fffffff) >> kMapSplitShift) : 0;
+        int f = 0, early = 0;
+        if (part != 0) early = acc[part - 1 + r];
 #pragma unroll
         for (int g = 0; g < G; ++g) f += map_group<WIDE>(map, st.w[g], st.c[WIDE ? g : 0]);
         const int hold = map[own] >> 1;  // f > hold: spin -1 (f = 0 keeps the old spin)
@@ -296,7 +351,8 @@ __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
           f += map_group<WIDE>(map, w, WIDE ? map_load<RES>(weights + (t.x + g) * 32) : w);
         }
         // 2. every lane of a row decides it: Eq. 2, then the flip
-        f = map_row_sum(f, lg);
+        f = map_row_sum(f, lg) + early;
+        if (part != 0 && lane < (t.w & 0xff)) acc[part - 1 + lane] = 0;
         const bool neg = (f > hold) != flip;
         // 3. the new spins into the maps
         if (CLUSTER) {
@@ -419,25 +475,36 @@ done:
 template <bool PACKED>
 __global__ void __launch_bounds__(256)
     map_fill_kernel(DevGraph d, const MapBlock* __restrict__ blocks, const int4* __restrict__ tasks, int warps,
-                    const int32_t* __restrict__ row_pos, const int32_t* __restrict__ map_index, int4* words,
-                    int4* weights) {
+                    const int32_t* __restrict__ row_pos, const int32_t* __restrict__ map_index,
+                    const int2* __restrict__ late, int hubs, int4* words, int4* weights) {
   const MapBlock B = blocks[blockIdx.x];
   const int lane = threadIdx.x & 31;
   for (int i = blockIdx.y * 8 + (threadIdx.x >> 5); i < B.rounds * warps; i += gridDim.y * 8) {
     const int4 t = __ldg(tasks + B.task0 + i);
     const int rows = t.w & 0xff, lg = (t.w >> 8) & 0xff, groups = t.w >> 16;
-    const int r = lane & ((32 >> lg) - 1), none = (t.y & ((1 << kMapFlipShift) - 1)) << 8;  // weight 0, a valid index
-    int e0 = 0, e1 = 0;
-    if (r < rows && groups > 0) {
-      const int p = __ldg(row_pos + B.row0 + (t.z & 0x7fffffff) + r);
-      e0 = __ldg(d.row_ptr + p) + (lane >> (5 - lg));
+    const int first = t.z & ((1 << kMapSplitShift) - 1), none = lg == kMapPart ? 0 : (t.y & ((1 << kMapFlipShift) - 1)) << 8;  // weight 0, a valid index
+    // entry 4 g + s of the lane: e0 + ((4 g + s) << step), past a gap of `gap`
+    // entries from e_gap on
+    int e0 = 0, e1 = 0, e_gap = 0x7fffffff, gap = 0, step = lg;
+    if (lg == kMapPart) {
+      const int p = __ldg(row_pos + blocks[(t.y & ((1 << kMapFlipShift) - 1)) >> kMapOwnerShift].row0 + first);
+      const int2 l = __ldg(late + p);
+      step = 5;
+      e0 = __ldg(d.row_ptr + p) + static_cast<int>((t.z & 0x7fffffff) >> kMapSplitShift) * kMapPartEntries + lane;
       e1 = __ldg(d.row_ptr + p + 1);
+      e_gap = l.x;
+      gap = l.y - l.x;
+    } else if ((lane & ((32 >> lg) - 1)) < rows && groups > 0) {
+      const int p = __ldg(row_pos + B.row0 + first + (lane & ((32 >> lg) - 1)));
+      e0 = (p < hubs ? __ldg(late + p).x : __ldg(d.row_ptr + p)) + (lane >> (5 - lg));
+      e1 = p < hubs ? __ldg(late + p).y : __ldg(d.row_ptr + p + 1);
     }
     for (int g = 0; g < groups; ++g) {
       int w[4], c[4];
 #pragma unroll
       for (int s = 0; s < 4; ++s) {
-        const int e = e0 + ((4 * g + s) << lg);
+        int e = e0 + ((4 * g + s) << step);
+        if (e >= e_gap) e += gap;
         Edge<PACKED> x;
         x.load(d, e, e < e1);
         c[s] = e < e1 ? x.weight() : 0;

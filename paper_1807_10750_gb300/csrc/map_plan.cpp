@@ -13,24 +13,57 @@ struct Unit {
   int32_t pos;  // first position
   int32_t rows, lg, groups;
   int32_t words, row, base;  // its place in the block
+  int32_t acc;  // split rows: the first row's partial sum + 1
+};
+
+// A part of a split row (host_graph.h) of block `owner`.
+struct Part {
+  int32_t owner, acc, row, part, groups, words;
 };
 
 }  // namespace
 
-void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int64_t smem_limit, MapPlan* mp) {
+void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int64_t smem_limit, MapPlan* mp,
+                    bool split) {
   *mp = MapPlan();
   const int32_t C = g.num_colours;
-  if (g.n < 1 || g.n > kMapMaxVertices || g.max_degree > kMapMaxDegree || C < 1 || C > 4096 || K < 1 ||
-      K > kMapMaxBlocks || (mode <= kMapBlockStream && K != 1) || (mode == kMapCluster && (K > 16 || (K & (K - 1)) != 0)))
+  if (g.n < 1 || g.n > kMapMaxVertices || (!split && g.max_degree > kMapMaxDegree) || C < 1 || C > 4096 || K < 1 ||
+      K > kMapMaxBlocks || (mode <= kMapBlockStream && K != 1) || (mode == kMapCluster && (K > 16 || (K & (K - 1)) != 0)) ||
+      (split && mode != kMapCluster))
     return;
   const bool cluster = mode == kMapCluster;
   const size_t stride = static_cast<size_t>(C) + 1;
   // a unit's rows in the block's row order: whole aligned words of the map
   // where they are stored as words
+  // split rows (the hubs): the entries in the class before, which its step
+  // must wait for
+  const int32_t hubs = split ? g.num_hubs : 0;
+  mp->hubs = hubs;
+  mp->late.resize(2 * static_cast<size_t>(hubs));
+  for (int32_t c = 0; c < C && g.class_begin[static_cast<size_t>(c)] < hubs; ++c) {
+    const size_t before = static_cast<size_t>((c + C - 1) % C);
+    for (int32_t v = g.class_begin[static_cast<size_t>(c)]; v < g.class_begin[static_cast<size_t>(c) + 1]; ++v) {
+      const auto b = g.col.begin() + g.row_ptr[static_cast<size_t>(v)], e = g.col.begin() + g.row_ptr[static_cast<size_t>(v) + 1];
+      mp->late[2 * static_cast<size_t>(v)] = static_cast<int32_t>(std::lower_bound(b, e, g.class_begin[before]) - g.col.begin());
+      mp->late[2 * static_cast<size_t>(v) + 1] = static_cast<int32_t>(std::lower_bound(b, e, g.class_begin[before + 1]) - g.col.begin());
+    }
+  }
+  // entries that a row's unit sums, and the most of rows [v, e)
+  auto length = [&](int32_t v) {
+    return v < hubs ? mp->late[2 * static_cast<size_t>(v) + 1] - mp->late[2 * static_cast<size_t>(v)]
+                    : g.row_ptr[static_cast<size_t>(v) + 1] - g.row_ptr[static_cast<size_t>(v)];
+  };
+  auto longest = [&](int32_t v, int32_t e) {
+    int32_t d = length(v);
+    if (v < hubs)  // the others stand in order of their length
+      while (++v < e) d = std::max(d, length(v));
+    return d;
+  };
   auto width = [&](const Unit& u) { return cluster ? std::max(4, 32 >> u.lg) : u.rows; };
   // units, dealt to the blocks in turn over all classes
   std::vector<std::vector<Unit>> of(static_cast<size_t>(K));  // per block: its units in order
   std::vector<int32_t> first(stride * static_cast<size_t>(K), 0);  // per block and class: its first unit
+  std::vector<int32_t> accs(static_cast<size_t>(K), 0);
   int64_t turn = 0;
   for (int32_t c = 0; c < C; ++c) {
     for (int32_t k = 0; k < K; ++k)
@@ -40,7 +73,7 @@ void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int6
     // entries a lane: the class's units at kMapSlots against one round of every warp
     int64_t lanes = 0;
     for (int32_t v = g.class_begin[static_cast<size_t>(c)]; v < ve; ++v) {
-      const int32_t d = g.row_ptr[static_cast<size_t>(v) + 1] - g.row_ptr[static_cast<size_t>(v)];
+      const int32_t d = length(v);
       int32_t lg = 0;
       while (lg < 5 && ((d + (1 << lg) - 1) >> lg) > kMapSlots) ++lg;
       lanes += 1 << lg;
@@ -50,20 +83,28 @@ void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int6
     int32_t least = 0;
     while (least < 5 && ((int64_t(ve) - g.class_begin[static_cast<size_t>(c)]) << (least + 1)) <= int64_t(32) * K) ++least;
     for (int32_t v = g.class_begin[static_cast<size_t>(c)]; v < ve;) {
-      const int32_t d = g.row_ptr[static_cast<size_t>(v) + 1] - g.row_ptr[static_cast<size_t>(v)];
-      int32_t lg = 0;
+      int32_t lg = 0, d = longest(v, std::min(v + 32, ve));
       while (lg < 5 && ((d + (1 << lg) - 1) >> lg) > max_slots) ++lg;
       // and so do the last rows of a class, up to four entries a lane
       while (lg < 5 && ((d + (1 << lg) - 1) >> lg) > 4 && (lg < least || (32 >> (lg + 1)) >= ve - v)) ++lg;
       const int32_t rows = std::min(32 >> lg, ve - v);
+      d = longest(v, v + rows);
       const int32_t slots = (d + (1 << lg) - 1) >> lg;
-      of[static_cast<size_t>(turn++ % K)].push_back({v, rows, lg, (slots + 3) / 4, 0, 0, 0});
+      const size_t k = static_cast<size_t>(turn++ % K);
+      Unit u{v, rows, lg, (slots + 3) / 4, 0, 0, 0, 0};
+      if (v < hubs) {
+        u.acc = accs[k] + 1;
+        accs[k] += rows;
+        mp->max_acc = std::max(mp->max_acc, accs[k]);
+      }
+      of[k].push_back(u);
       v += rows;
     }
     if (cluster)
       // every block sends something in every class: a block without a unit
-      // gets one without rows
-      for (; turn < first_turn + K; ++turn) of[static_cast<size_t>(turn % K)].push_back({0, 0, 5, 0, 0, 0, 0});
+      // gets one without rows (and the next class's first unit is the next
+      // block's all the same)
+      for (int64_t k = turn; k < first_turn + K; ++k) of[static_cast<size_t>(k % K)].push_back({0, 0, 5, 0, 0, 0, 0, 0});
   }
   for (int32_t k = 0; k < K; ++k)
     first[static_cast<size_t>(k) * stride + static_cast<size_t>(C)] = static_cast<int32_t>(of[static_cast<size_t>(k)].size());
@@ -77,12 +118,12 @@ void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int6
   mp->class_msg.assign(stride, 0);
   mp->map_index.assign(static_cast<size_t>(g.n), 0);
   // the blocks' rows and entries
+  std::vector<std::vector<Part>> parts(hubs > 0 ? static_cast<size_t>(K) * static_cast<size_t>(C) : 0);  // by the class whose step sums them
   int32_t row0 = 0, widest = 1;
   int64_t words0 = 0;
   for (int32_t k = 0; k < K; ++k) {
     MapBlock& b = mp->blocks[static_cast<size_t>(k)];
     b.row0 = row0;
-    b.words0 = static_cast<int32_t>(words0);
     int32_t row = 0, groups = 0;
     for (int32_t c = 0; c < C; ++c) {
       const size_t t = static_cast<size_t>(k) * stride + static_cast<size_t>(c);
@@ -107,10 +148,44 @@ void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int6
     b.rows = row;
     b.groups = groups;
     row0 += row;
-    words0 += groups;
     mp->max_rows = std::max(mp->max_rows, b.rows);
+  }
+  // the parts of class c's rows, each to the block with the fewest tasks in
+  // the step of the class before; the row's block waits for their bytes
+  std::vector<int32_t> received(hubs > 0 ? stride * static_cast<size_t>(K) : 0, 0);
+  for (int32_t c = 0; c < C && hubs > 0; ++c) {
+    const size_t at = static_cast<size_t>((c + C - 1) % C);
+    std::vector<int32_t> busy(static_cast<size_t>(K));
+    for (int32_t k = 0; k < K; ++k) {
+      const size_t t = static_cast<size_t>(k) * stride + at;
+      busy[static_cast<size_t>(k)] = first[t + 1] - first[t];
+    }
+    for (int32_t k = 0; k < K; ++k) {
+      const size_t t = static_cast<size_t>(k) * stride + static_cast<size_t>(c);
+      for (int32_t i = first[t]; i < first[t + 1]; ++i) {
+        const Unit& u = of[static_cast<size_t>(k)][static_cast<size_t>(i)];
+        for (int32_t r = 0; u.acc != 0 && r < u.rows; ++r) {
+          const size_t v = static_cast<size_t>(u.pos + r);
+          const int32_t early = g.row_ptr[v + 1] - g.row_ptr[v] - length(u.pos + r);
+          for (int32_t p = 0; p * kMapPartEntries < early; ++p) {
+            const size_t to = static_cast<size_t>(std::min_element(busy.begin(), busy.end()) - busy.begin());
+            const int32_t gr = (std::min(kMapPartEntries, early - p * kMapPartEntries) + 127) / 128;
+            parts[to * static_cast<size_t>(C) + at].push_back({k, u.acc - 1 + r, u.row + r, p, gr, mp->blocks[to].groups});
+            mp->blocks[to].groups += gr;
+            mp->stage = std::max(mp->stage, gr);
+            widest = std::max(widest, ++busy[to]);
+            received[static_cast<size_t>(k) * stride + at] += 4;
+          }
+        }
+      }
+    }
+  }
+  for (MapBlock& b : mp->blocks) {
+    b.words0 = static_cast<int32_t>(std::min<int64_t>(words0, 1 << 24));
+    words0 += b.groups;
     mp->max_groups = std::max(mp->max_groups, b.groups);
   }
+  if (mp->max_acc > kMapMaxSplit || g.max_degree / kMapPartEntries > kMapMaxSplit) return;
   if (words0 >= (int64_t(1) << 24) || mp->max_rows / 32 >= (1 << (32 - kMapFlipShift - 1)) - 1) return;
   // the map: class by class, block by block, a segment for a block's rows of
   // the class
@@ -145,6 +220,7 @@ void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int6
   }
   for (int32_t k = 0; k < K; ++k)
     mp->block_msg[static_cast<size_t>(k) * stride + static_cast<size_t>(C)] = static_cast<int32_t>(mp->msg.size());
+  if (hubs > 0) mp->block_msg = received;
   mp->map_bytes = static_cast<int32_t>((at + 32 + 15) & ~int64_t(15));
   // the tasks; as many warps as the largest class has units and draws
   const int32_t class_draws = (mp->max_rows / 32 + C - 1) / C;
@@ -156,12 +232,19 @@ void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int6
     b.task0 = static_cast<int32_t>(mp->tasks.size());
     for (int32_t c = 0; c < C; ++c) {
       const size_t t = static_cast<size_t>(k) * stride + static_cast<size_t>(c);
-      const int32_t rounds = std::max(1, (first[t + 1] - first[t] + warps - 1) / warps);
+      static const std::vector<Part> none;
+      const std::vector<Part>& early = hubs > 0 ? parts[static_cast<size_t>(k) * static_cast<size_t>(C) + static_cast<size_t>(c)] : none;
+      const int32_t units = first[t + 1] - first[t];
+      const int32_t rounds = std::max(1, (units + static_cast<int32_t>(early.size()) + warps - 1) / warps);
+      if (c == C - 1) b.last0 = static_cast<int32_t>(mp->tasks.size()) - b.task0;
       for (int32_t i = 0; i < rounds * warps; ++i) {
         MapTask x{0, 0, 0, 0};
-        if (first[t] + i < first[t + 1]) {
+        if (i < units) {
           const Unit& u = mine[static_cast<size_t>(first[t] + i)];
-          x = {u.words, u.base, u.row, u.rows | (u.lg << 8) | (u.groups << 16)};
+          x = {u.words, u.base, u.row | (u.acc << kMapSplitShift), u.rows | (u.lg << 8) | (u.groups << 16)};
+        } else if (i - units < static_cast<int32_t>(early.size())) {
+          const Part& p = early[static_cast<size_t>(i - units)];
+          x = {p.words, p.acc | (p.owner << kMapOwnerShift), p.row | (p.part << kMapSplitShift), (kMapPart << 8) | (p.groups << 16)};
         }
         if (i >= (rounds - 1) * warps) x.row |= static_cast<int32_t>(0x80000000u);
         mp->tasks.push_back(x);
@@ -192,7 +275,7 @@ void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int6
     mp->max_tasks = std::max(mp->max_tasks, b.rounds * warps);
   }
   const int64_t entries = mode == kMapBlock ? int64_t(mp->max_groups) * (wide ? 2 : 1) : 0;
-  const int64_t smem = map_smem_bytes(mp->map_bytes, entries, mp->max_tasks, C, mp->max_rows);
+  const int64_t smem = map_smem_bytes(mp->map_bytes, entries, mp->max_tasks, C, mp->max_rows, mp->max_acc);
   if (smem > smem_limit) return;
   mp->smem_bytes = static_cast<int32_t>(smem);
   // rows

@@ -2,7 +2,7 @@
 // kernels do -- every block's rounds of tasks, the entries by lane, the
 // stores, words or messages that carry the new spins -- with every index
 // checked against its array, and compares the spins of three sweeps with a
-// plain sweep over the rows. Usage: map_plan_check KIND N M WMAX MODE K WIDE SEED
+// plain sweep over the rows. Usage: map_plan_check KIND N M WMAX MODE K WIDE SEED [SPLIT]
 #include <cstdint>
 #include <cstdio>
 #include <cstdlib>
@@ -32,7 +32,8 @@ static uint32_t spin_bytes(uint32_t bits) {
 }
 
 int main(int argc, char** argv) {
-  CHECK(argc == 9);
+  CHECK(argc == 9 || argc == 10);
+  const bool split = argc == 10 && std::atoi(argv[9]) != 0;
   const int kind = std::atoi(argv[1]), n = std::atoi(argv[2]), m = std::atoi(argv[3]), wmax = std::atoi(argv[4]);
   const int mode = std::atoi(argv[5]), K = std::atoi(argv[6]);
   const bool wide = std::atoi(argv[7]) != 0;
@@ -48,17 +49,19 @@ int main(int argc, char** argv) {
   else if (kind == 1)  // complete graph
     for (int i = 0; i < n; ++i)
       for (int j = i + 1; j < n; ++j) edge(i, j);
-  else  // m long rows on a cycle
+  else  // m long rows on a cycle, with hubs (kind 3) of 256 to 1500 entries, many of them each other's
     for (int i = 0; i < n; ++i) {
       edge(i, (i + 1) % n);
       if (i < m)
-        for (int j = 0; j < 200; ++j) edge(i, m + static_cast<int>(rng() % static_cast<uint32_t>(n - m)));
+        for (int j = 0; j < (kind == 2 ? 200 : 256 + 1500 * i / m); ++j)
+          edge(i, kind == 2 || j % 3 != 0 ? m + static_cast<int>(rng() % static_cast<uint32_t>(n - m))
+                                          : static_cast<int>(rng() % static_cast<uint32_t>(m)));
     }
   HostGraph g;
   CHECK(build_host_graph(n, static_cast<int64_t>(src.size()), src.data(), dst.data(), w.data(), &g) == 0);
   const int64_t limit = 232448;
   MapPlan mp;
-  build_map_plan(g, mode, K, wide, limit, &mp);
+  build_map_plan(g, mode, K, wide, limit, &mp, split);
   if (!mp.ok) {
     std::printf("no plan\n");
     return 2;
@@ -79,6 +82,37 @@ int main(int argc, char** argv) {
     CHECK(b.words0 + b.groups <= mp.total_groups);
     CHECK(static_cast<size_t>(b.row0 + b.rows) <= mp.row_pos.size() && mp.row_pos.size() == mp.row_orig.size());
   }
+  CHECK(mp.hubs == (split ? g.num_hubs : 0) && mp.late.size() == 2 * static_cast<size_t>(mp.hubs));
+  // a part of a split row, summed in class c's step: none of its terms from that class
+  std::vector<std::vector<long>> acc(static_cast<size_t>(K), std::vector<long>(static_cast<size_t>(mp.max_acc) + 32, 0));
+  std::vector<std::vector<int>> summed(static_cast<size_t>(K), std::vector<int>(static_cast<size_t>(mp.max_acc) + 32, 0));
+  std::vector<int> got(static_cast<size_t>(K), 0);
+  auto add_part = [&](int k, const MapTask& x, int c) {
+    const MapBlock& b = mp.blocks[static_cast<size_t>(k)];
+    const int slot = x.base & ((1 << kMapOwnerShift) - 1), groups = x.shape >> 16;
+    const int owner = (x.base & ((1 << kMapFlipShift) - 1)) >> kMapOwnerShift;
+    CHECK(owner < K);
+    got[static_cast<size_t>(owner)] += 4;
+    const int p = mp.row_pos[static_cast<size_t>(mp.blocks[static_cast<size_t>(owner)].row0 + (x.row & ((1 << kMapSplitShift) - 1)))];
+    CHECK(slot < mp.max_acc && p >= 0 && p < mp.hubs && groups <= mp.stage && x.words + groups <= b.groups);
+    CHECK(p >= g.class_begin[(c + 1) % C] && p < g.class_begin[(c + 1) % C + 1]);
+    const int l0 = mp.late[2 * p], l1 = mp.late[2 * p + 1];
+    CHECK(l0 >= g.row_ptr[p] && l0 <= l1 && l1 <= g.row_ptr[p + 1]);
+    for (int lane = 0; lane < 32; ++lane)
+      for (int s = 0; s < 4 * groups; ++s) {
+        int e = g.row_ptr[p] + ((x.row & 0x7fffffff) >> kMapSplitShift) * kMapPartEntries + lane + 32 * s;
+        if (e >= l0) e += l1 - l0;
+        if (e >= g.row_ptr[p + 1]) continue;
+        CHECK(g.col[e] < g.class_begin[c] || g.col[e] >= g.class_begin[c + 1]);
+        acc[static_cast<size_t>(owner)][static_cast<size_t>(slot)] += static_cast<long>(g.w[e]) * maps[k][mp.map_index[g.col[e]]];
+        summed[static_cast<size_t>(owner)][static_cast<size_t>(slot)]++;
+      }
+  };
+  for (int k = 0; k < K && split; ++k)
+    for (int i = mp.blocks[k].last0; i < mp.blocks[k].rounds * mp.warps; ++i) {
+      const MapTask x = mp.tasks[static_cast<size_t>(mp.blocks[k].task0 + i)];
+      if (((x.shape >> 8) & 0xff) == kMapPart) add_part(k, x, C - 1);
+    }
   std::vector<int> filled(static_cast<size_t>(mp.total_groups), 0);
   for (int sweep = 0; sweep < 3; ++sweep) {
     std::vector<int> round(static_cast<size_t>(K), 0);
@@ -94,6 +128,7 @@ int main(int argc, char** argv) {
       for (size_t i = 0; i < now.size(); ++i) spin[static_cast<size_t>(g.class_begin[c]) + i] = now[i];
       std::vector<std::pair<int, uint32_t>> stores, messages;  // cluster: words; grid: message and bits
       long bytes = 0;
+      std::vector<std::pair<int, MapTask>> parts;
       for (int k = 0; k < K; ++k) {
         const MapBlock& b = mp.blocks[k];
         const size_t t = static_cast<size_t>(k) * stride + static_cast<size_t>(c);
@@ -111,8 +146,13 @@ int main(int argc, char** argv) {
             if (warp == 0) more = x.row >= 0;
             CHECK(more == (x.row >= 0));
             if (x.shape == 0) continue;
+            if (((x.shape >> 8) & 0xff) == kMapPart) {
+              parts.push_back({k, x});
+              continue;
+            }
             ++units;
-            const int base = x.base & ((1 << kMapFlipShift) - 1), row = x.row & 0x7fffffff;
+            const int base = x.base & ((1 << kMapFlipShift) - 1), row = x.row & ((1 << kMapSplitShift) - 1);
+            const int slot = (x.row & 0x7fffffff) >> kMapSplitShift;
             const int rows = x.shape & 0xff, lg = (x.shape >> 8) & 0xff, groups = x.shape >> 16;
             CHECK(lg <= 5 && rows <= (32 >> lg) && groups <= mp.stage && x.words + groups <= b.groups);
             CHECK(row >= mp.class_row[t] && row + rows <= mp.class_row[t + 1] && base + 32 <= mp.map_bytes);
@@ -123,15 +163,24 @@ int main(int argc, char** argv) {
               const int r = lane & ((32 >> lg) - 1);
               if (r >= rows) continue;
               const int p = mp.row_pos[static_cast<size_t>(b.row0 + row + r)];
-              if (lane == r) entries += g.row_ptr[p + 1] - g.row_ptr[p];
+              CHECK((slot != 0) == (p < mp.hubs));
+              const int begin = p < mp.hubs ? mp.late[2 * p] : g.row_ptr[p], end = p < mp.hubs ? mp.late[2 * p + 1] : g.row_ptr[p + 1];
+              if (lane == r) entries += end - begin;
               for (int s = 0; s < 4 * groups; ++s) {
-                const int e = g.row_ptr[p] + (lane >> (5 - lg)) + (s << lg);
-                if (e >= g.row_ptr[p + 1]) continue;
+                const int e = begin + (lane >> (5 - lg)) + (s << lg);
+                if (e >= end) continue;
                 f[r] += static_cast<long>(g.w[e]) * maps[k][mp.map_index[g.col[e]]];
                 ++terms;
               }
             }
             CHECK(terms == entries);
+            for (int r = 0; r < rows && slot != 0; ++r) {
+              const size_t i = static_cast<size_t>(slot - 1 + r);
+              const int p = mp.row_pos[static_cast<size_t>(b.row0 + row + r)];
+              CHECK(summed[k][i] + mp.late[2 * p + 1] - mp.late[2 * p] == g.row_ptr[p + 1] - g.row_ptr[p]);
+              f[r] += acc[k][i];
+              acc[k][i] = summed[k][i] = 0;
+            }
             for (int gp = 0; gp < groups; ++gp) CHECK(!filled[b.words0 + x.words + gp]++ || sweep > 0);
             uint32_t bits = 0;
             for (int r = 0; r < rows; ++r) {
@@ -167,13 +216,16 @@ int main(int argc, char** argv) {
           }
         }
       }
+      got.assign(static_cast<size_t>(K), 0);
+      for (const auto& x : parts) add_part(x.first, x.second, c);
+      for (int k = 0; k < K && split; ++k) CHECK(got[k] == mp.block_msg[static_cast<size_t>(k) * stride + static_cast<size_t>(c)]);
       if (mode == kMapCluster) CHECK(bytes == mp.class_bytes[c] && bytes < (1 << 20));
       if (mode == kMapGrid) {
         const int count = mp.class_msg[c + 1] - mp.class_msg[c];
         CHECK(static_cast<int>(messages.size()) == count && count <= mp.mail_stride);
-        std::vector<int> got(static_cast<size_t>(count), 0);
+        std::vector<int> came(static_cast<size_t>(count), 0);
         for (const auto& x : messages) {
-          CHECK(x.first >= mp.class_msg[c] && x.first < mp.class_msg[c + 1] && !got[x.first - mp.class_msg[c]]++);
+          CHECK(x.first >= mp.class_msg[c] && x.first < mp.class_msg[c + 1] && !came[x.first - mp.class_msg[c]]++);
           for (int q = 0; q < (mp.msg[x.first] & 15); ++q)
             stores.push_back({(mp.msg[x.first] >> 4) * 4 + 4 * q, spin_bytes(x.second >> (4 * q))});
         }

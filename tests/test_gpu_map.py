@@ -1,7 +1,7 @@
 """The spin-map engine against the CPU oracle, bit for bit, at the sizes where
 its forms change: one block (entries resident or streamed), a cluster, the
 whole grid; narrow and wide weights, units of 1 to 32 lanes a row, partial
-units and single-row classes, flip bias, both schedules, resumed runs. And its
+units and single-row classes, graphs with hubs, flip bias, both schedules, resumed runs. And its
 bounded waits: a block that sends nothing is reported, not waited for."""
 
 import numpy as np
@@ -42,7 +42,32 @@ def _long_rows():
     return synth.Graph(9001, src, dst, synth.draw_weights("int8", src.size, rng))
 
 
+def _hubs(n, hubs, weights="int8"):
+    # rows of 256 to n / 2 entries, a third of them the other hubs', on a cycle
+    rng = np.random.default_rng(n + hubs)
+    ring = np.arange(n, dtype=np.int32)
+    src, dst = [ring], [np.roll(ring, -1)]
+    for i in range(hubs):
+        d = 256 + (n // 2 - 256) * i // hubs
+        src.append(np.full(d, i, np.int32))
+        dst.append(np.where(np.arange(d) % 3 == 0, rng.integers(0, hubs, d), rng.integers(hubs, n, d)).astype(np.int32))
+    src, dst = np.concatenate(src), np.concatenate(dst)
+    keep = src != dst
+    return synth.Graph(n, src[keep], dst[keep], synth.draw_weights(weights, int(keep.sum()), rng))
+
+
+def _star(n):
+    src = np.zeros(n - 1, np.int32)
+    return synth.Graph(n, src, np.arange(1, n, dtype=np.int32), np.where(np.arange(n - 1) % 3 == 0, 5, -4).astype(np.int32))
+
+
 GRAPHS = {
+    "split_star": lambda: _star(4097),
+    "split_one_hub": lambda: _hubs(4100, 1),
+    "split_hubs": lambda: _hubs(6000, 17),
+    "split_wide": lambda: _wide(_hubs(9001, 60)),
+    "split_zipf": lambda: synth.zipf_config_graph(20011, 2.1, 4, 3000, 5),
+    "split_zipf_large": lambda: synth.zipf_config_graph(110003, 2.1, 4, 10000, 5),
     "block_n31": lambda: _er(31, 6),
     "block_er800": lambda: _er(800, 48, weights="one"),
     "block_wide": lambda: _wide(_er(500, 20)),
@@ -79,7 +104,7 @@ def test_matches_oracle(P, name):
             assert np.array_equal(P.ising_get_spins(h), want), n0
 
 
-@pytest.mark.parametrize("name", ["block_er800", "cluster_er2001", "grid_er"])
+@pytest.mark.parametrize("name", ["block_er800", "cluster_er2001", "split_hubs", "grid_er"])
 def test_flip_bias(P, name):
     g = GRAPHS[name]()
     s0 = oracle.init_spins(g.n, 5)
@@ -92,8 +117,8 @@ def test_flip_bias(P, name):
         assert np.array_equal(P.ising_get_spins(h), want)
 
 
-@pytest.mark.parametrize("name", ["cluster_er2001", "grid_er"])
-@pytest.mark.parametrize("nflip", [False, True])
+@pytest.mark.parametrize("name,nflip", [("cluster_er2001", False), ("cluster_er2001", True), ("split_hubs", False),
+                                        ("grid_er", False), ("grid_er", True)])
 def test_a_silent_block_reports_timeout(P, name, nflip):
     g = GRAPHS[name]()
     kw = dict(kind=P.ISING_SCHED_NFLIP, n0=20) if nflip else dict(p0=0.1)

@@ -9,7 +9,7 @@ import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_1807_10750_gb300", "csrc")
-PAIRS, COMPLETE, LONG_ROWS = 0, 1, 2
+PAIRS, COMPLETE, LONG_ROWS, HUBS = 0, 1, 2, 3
 BLOCK, BLOCK_STREAM, CLUSTER, GRID = 0, 1, 2, 3
 
 
@@ -35,6 +35,17 @@ def test_plan_sweeps_like_the_rows(check, kind, n, m, wmax, mode, K):
         # 2: the tables do not fit (resident entries of a large graph, a map of
         # 200,000 spins beside too many tasks)
         assert r.returncode == 0 or (r.returncode == 2 and n * max(m, n) > 10 ** 6), r.stdout
+
+
+@pytest.mark.parametrize("kind,n,m", [(HUBS, 4097, 1), (HUBS, 9001, 40), (HUBS, 30000, 300), (COMPLETE, 300, 0),
+                                      (PAIRS, 5000, 4000)])
+@pytest.mark.parametrize("K", [1, 8, 16])
+def test_split_rows_sweep_like_the_rows(check, kind, n, m, K):
+    for wide in (0, 1):
+        r = subprocess.run([check] + [str(x) for x in (kind, n, m, 5, CLUSTER, K, wide, 3, 1)], capture_output=True,
+                           text=True)
+        # 2: the tables of 30,000 rows do not fit in one block, nor a map of 300 classes on 16
+        assert r.returncode == (2 if (n, K) in ((30000, 1), (300, 16)) else 0), r.stdout
 
 
 @pytest.mark.parametrize("K", [1, 2, 4, 8, 16])
