@@ -955,26 +955,31 @@ cudaError_t launch_hub(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint64
 }
 
 // The spin-map engine (map.cuh) on the handle's plan.
-template <int MODE>
+template <int MODE, bool RES>
 const void* map_kernel_of(bool wide, int stage) {
   using isingx::map_kernel;
-  if (wide) return stage <= 2 ? reinterpret_cast<const void*>(map_kernel<MODE, true, 2, false>)
-                              : reinterpret_cast<const void*>(map_kernel<MODE, true, 4, false>);
-  if (stage <= 1) return reinterpret_cast<const void*>(map_kernel<MODE, false, 1, false>);
-  if (stage <= 2) return reinterpret_cast<const void*>(map_kernel<MODE, false, 2, false>);
-  if (stage <= 4) return reinterpret_cast<const void*>(map_kernel<MODE, false, 4, false>);
-  return reinterpret_cast<const void*>(map_kernel<MODE, false, 8, false>);
+  if (wide) return stage <= 2 ? reinterpret_cast<const void*>(map_kernel<MODE, true, 2, false, RES>)
+                              : reinterpret_cast<const void*>(map_kernel<MODE, true, 4, false, RES>);
+  if (stage <= 1) return reinterpret_cast<const void*>(map_kernel<MODE, false, 1, false, RES>);
+  if (stage <= 2) return reinterpret_cast<const void*>(map_kernel<MODE, false, 2, false, RES>);
+  if (stage <= 4) return reinterpret_cast<const void*>(map_kernel<MODE, false, 4, false, RES>);
+  return reinterpret_cast<const void*>(map_kernel<MODE, false, 8, false, RES>);
 }
 
-const void* map_kernel_for(int mode, bool wide, int stage, bool split) {
-  if (mode == isingx::kMapBlock) return map_kernel_of<isingx::kMapBlock>(wide, stage);
-  if (mode == isingx::kMapBlockStream) return map_kernel_of<isingx::kMapBlockStream>(wide, stage);
-  constexpr int kSplitG = isingx::kMapPartEntries / 128;
-  if (mode == isingx::kMapCluster && split)
-    return wide ? reinterpret_cast<const void*>(isingx::map_kernel<isingx::kMapCluster, true, kSplitG, true>)
-                : reinterpret_cast<const void*>(isingx::map_kernel<isingx::kMapCluster, false, kSplitG, true>);
-  if (mode == isingx::kMapCluster) return map_kernel_of<isingx::kMapCluster>(wide, stage);
-  return map_kernel_of<isingx::kMapGrid>(wide, stage);
+template <bool RES>
+const void* map_split_kernel(bool wide) {
+  constexpr int G = isingx::kMapPartEntries / 128;
+  return wide ? reinterpret_cast<const void*>(isingx::map_kernel<isingx::kMapCluster, true, G, true, RES>)
+              : reinterpret_cast<const void*>(isingx::map_kernel<isingx::kMapCluster, false, G, true, RES>);
+}
+
+const void* map_kernel_for(int mode, bool wide, int stage, bool split, bool resident) {
+  if (mode == isingx::kMapBlock) return map_kernel_of<isingx::kMapBlock, true>(wide, stage);
+  if (mode == isingx::kMapBlockStream) return map_kernel_of<isingx::kMapBlockStream, false>(wide, stage);
+  if (mode == isingx::kMapGrid) return map_kernel_of<isingx::kMapGrid, false>(wide, stage);
+  if (split) return resident ? map_split_kernel<true>(wide) : map_split_kernel<false>(wide);
+  return resident ? map_kernel_of<isingx::kMapCluster, true>(wide, stage)
+                  : map_kernel_of<isingx::kMapCluster, false>(wide, stage);
 }
 
 void map_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int mode, int K, int warps, int smem, cudaStream_t s) {
@@ -999,7 +1004,7 @@ void map_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int mode, in
 // Whether the device can run a plan: shared memory, a cluster of that size, or
 // K co-resident blocks.
 bool map_fits(const isingx::MapPlan& mp, bool wide) {
-  const void* kernel = map_kernel_for(mp.mode, wide, mp.stage, mp.hubs > 0);
+  const void* kernel = map_kernel_for(mp.mode, wide, mp.stage, mp.hubs > 0, mp.resident);
   bool fits = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, mp.smem_bytes) == cudaSuccess;
   if (fits && mp.mode == isingx::kMapCluster) {
     fits = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
@@ -1102,6 +1107,7 @@ cudaError_t upload_map_plan(ising_graph* g, const isingx::MapPlan& mp) {
   g->map_stage = mp.stage;
   g->map_stride = mp.mail_stride;
   g->map_accs = mp.max_acc;
+  g->map_resident = mp.resident;
   g->map_ok = true;
   return cudaSuccess;
 }
@@ -1109,7 +1115,7 @@ cudaError_t upload_map_plan(ising_graph* g, const isingx::MapPlan& mp) {
 cudaError_t launch_map(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint64_t T, uint64_t T0,
                        uint32_t replica, const isingx::PhiloxRounds& rk, uint32_t n0, int par0) {
   const bool wide = !g->packed;
-  const void* kernel = map_kernel_for(g->map_mode, wide, g->map_stage, g->map_accs > 0);
+  const void* kernel = map_kernel_for(g->map_mode, wide, g->map_stage, g->map_accs > 0, g->map_resident);
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, g->map_smem);
   if (e != cudaSuccess) return e;
   if (g->map_mode == isingx::kMapCluster &&

@@ -111,7 +111,7 @@ struct ising_graph {
   int32_t* d_hub_blk = nullptr;      // non-hub classes' work split over the worker blocks
   int32_t hub_grid = 0;              // blocks the split was made for
   // spin-map engine (map.cuh)
-  bool map_ok = false;
+  bool map_ok = false, map_resident = false;
   int map_mode = 0, map_K = 0, map_warps = 0, map_smem = 0;
   int32_t map_bytes = 0, map_tasks = 0, map_rows = 0, map_groups = 0, map_stage = 0, map_stride = 0, map_accs = 0;
   isingx::MapBlock* d_map_blocks = nullptr;

@@ -219,8 +219,8 @@ void build_halo_plan(const HostGraph& g, int32_t parts, int32_t sweeps_per_epoch
 // lane l is the row's entry L (4 g + k) + l / R, word (map index << 8) |
 // (w & 0xff), padded with weight 0; wide weights sit in a second array of the
 // same layout. L is the smallest power of two that leaves a lane at most
-// kMapSlots entries, twice as many in a class that would otherwise need more
-// than one round of every warp.
+// kMapSlots entries; half as many in graphs of short rows, twice as many in a
+// class that would otherwise need more than one round of every warp.
 //
 // A block's work of a sweep is a table of rounds of `warps` tasks, class by
 // class; a task is a unit, a word of 32 flip draws for the next sweep, both
@@ -273,6 +273,7 @@ struct MapPlan {
   int32_t max_tasks = 0, max_rows = 0, max_groups = 0;  // over the blocks
   int32_t hubs = 0, max_acc = 0;           // split rows (positions below `hubs`), the most of a block
   int32_t smem_bytes = 0;
+  bool resident = false;     // the entries are in shared memory (kMapBlock; a cluster's that fit)
   std::vector<MapBlock> blocks;
   std::vector<MapTask> tasks;
   int64_t total_groups = 0;  // entry groups of all blocks; map_fill_kernel writes them on the device

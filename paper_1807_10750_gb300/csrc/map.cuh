@@ -31,12 +31,16 @@
 // instruction of the one or two warps a scheduler has: hence few warps (8 to
 // 16), a task table that one counter walks, up to 16 entries a lane before a
 // row takes more lanes, rows strided over the lanes so that lane r ends up with
-// row r, and no branch in the sums (missing groups have weight 0). Entries
-// streamed from L2 a class ahead cost the same as resident ones on a cluster.
+// row r, and no branch in the sums (missing groups have weight 0). Entries are
+// read a task ahead, from shared memory where they fit beside the map: in a
+// class of several rounds the L2 latency shows (20,099-vertex torus 4.07 -> 3.63
+// us a sweep, 5,000-vertex power-law graph 16.6 -> 15.6; one round a class, the
+// same). Two tasks ahead costs more in moves than it hides (10,000 vertices, 100k
+// edges: 7.0 -> 7.6).
 // Microseconds a sweep on GB300, against the engine that ran before (a block
 // with its CSR in shared memory, item dataflow, or the grid barrier):
 // 800 vertices, 19k edges, 17 classes, one block: 12.1 -> 6.5; 20,099-vertex
-// torus, 4 classes, cluster: 12.5 -> 3.9; 10,000 vertices, 100k edges, 11
+// torus, 4 classes, cluster: 12.5 -> 3.6; 10,000 vertices, 100k edges, 11
 // classes, cluster: 48 -> 6.4; 30,011 vertices, 600k wide edges, 16 classes,
 // cluster: 97 -> 17; 100,000 vertices, 5M edges, 30 classes, grid: 253 -> 62.
 //
@@ -154,12 +158,12 @@ __device__ __forceinline__ int map_row_sum(int f, int lg) {
 
 // K blocks; sweeps t_begin .. t_begin + sweeps - 1.
 // SPLIT: a cluster's plan with split rows (no Algorithm 1); G covers a part.
-template <int MODE, bool WIDE, int G, bool SPLIT>
+// RES: the block's entries are in shared memory.
+template <int MODE, bool WIDE, int G, bool SPLIT, bool RES>
 __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
     map_kernel(DevGraph d, MapArgs a, uint64_t t_begin, uint32_t sweeps, uint64_t T, uint64_t T0,
                uint32_t replica, PhiloxRounds rk) {
   extern __shared__ __align__(128) unsigned char map_mem[];
-  constexpr bool RES = MODE == kMapBlock;
   constexpr bool CLUSTER = MODE == kMapCluster;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int threads = blockDim.x, warps = threads >> 5;
@@ -280,8 +284,8 @@ __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
       if (((x.w >> 8) & 0xff) != kMapPart) continue;
       int f = 0;
       for (int g = 0; g < (x.w >> 16); ++g) {
-        const int4 w = __ldg(words + (x.x + g) * 32);
-        f += map_group<WIDE>(map, w, WIDE ? __ldg(weights + (x.x + g) * 32) : w);
+        const int4 w = map_load<RES>(words + (x.x + g) * 32);
+        f += map_group<WIDE>(map, w, WIDE ? map_load<RES>(weights + (x.x + g) * 32) : w);
       }
       f = __reduce_add_sync(kFullMask, f);
       if (lane == 0)

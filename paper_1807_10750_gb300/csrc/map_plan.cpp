@@ -65,6 +65,20 @@ void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int6
   std::vector<int32_t> first(stride * static_cast<size_t>(K), 0);  // per block and class: its first unit
   std::vector<int32_t> accs(static_cast<size_t>(K), 0);
   int64_t turn = 0;
+  // entries a lane, at most l: a unit costs about its slots and four entries
+  // more, whatever its rows fill, so short rows are better off with 8 than with 16
+  // (a cluster's sweep at 60,000 vertices of 6 neighbours 12.4 -> 9.4 us, of 8 12.4 ->
+  // 10.7; 10,000 of 20: 7.0 at 16, 8.1 at 8). The grid's steps are bound by their
+  // exchange (150,000 vertices of 4: 22.3 at 16, 23.0 at 8)
+  auto row_lanes = [&](int32_t d, int32_t slots) {
+    int32_t lg = 0;
+    while (lg < 5 && ((d + (1 << lg) - 1) >> lg) > slots) ++lg;
+    return int64_t(1) << lg;
+  };
+  int64_t cost[2] = {0, 0};
+  for (int32_t v = hubs; v < g.n; ++v)
+    for (int i = 0; i < 2; ++i) cost[i] += row_lanes(length(v), kMapSlots >> i) * ((kMapSlots >> i) + 4);
+  const int32_t few_slots = !split && mode != kMapGrid && cost[1] < cost[0] ? kMapSlots / 2 : kMapSlots;
   for (int32_t c = 0; c < C; ++c) {
     for (int32_t k = 0; k < K; ++k)
       first[static_cast<size_t>(k) * stride + static_cast<size_t>(c)] = static_cast<int32_t>(of[static_cast<size_t>(k)].size());
@@ -72,13 +86,9 @@ void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int6
     const int64_t first_turn = turn;
     // entries a lane: the class's units at kMapSlots against one round of every warp
     int64_t lanes = 0;
-    for (int32_t v = g.class_begin[static_cast<size_t>(c)]; v < ve; ++v) {
-      const int32_t d = length(v);
-      int32_t lg = 0;
-      while (lg < 5 && ((d + (1 << lg) - 1) >> lg) > kMapSlots) ++lg;
-      lanes += 1 << lg;
-    }
-    const int32_t max_slots = lanes > int64_t(32) * kMapMaxWarps * K ? 2 * kMapSlots : kMapSlots;
+    for (int32_t v = g.class_begin[static_cast<size_t>(c)]; v < ve; ++v) lanes += row_lanes(length(v), few_slots);
+    const int32_t max_slots =
+        few_slots == kMapSlots && lanes > int64_t(32) * kMapMaxWarps * K ? 2 * kMapSlots : few_slots;
     // a class too small to give every block a unit uses more lanes a row
     int32_t least = 0;
     while (least < 5 && ((int64_t(ve) - g.class_begin[static_cast<size_t>(c)]) << (least + 1)) <= int64_t(32) * K) ++least;
@@ -274,8 +284,10 @@ void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int6
     b.rounds = (static_cast<int32_t>(mp->tasks.size()) - b.task0) / warps;
     mp->max_tasks = std::max(mp->max_tasks, b.rounds * warps);
   }
-  const int64_t entries = mode == kMapBlock ? int64_t(mp->max_groups) * (wide ? 2 : 1) : 0;
-  const int64_t smem = map_smem_bytes(mp->map_bytes, entries, mp->max_tasks, C, mp->max_rows, mp->max_acc);
+  const int64_t entries = int64_t(mp->max_groups) * (wide ? 2 : 1);
+  int64_t smem = map_smem_bytes(mp->map_bytes, 0, mp->max_tasks, C, mp->max_rows, mp->max_acc);
+  mp->resident = mode == kMapBlock || (cluster && smem + entries * 512 <= smem_limit);
+  if (mp->resident) smem += entries * 512;
   if (smem > smem_limit) return;
   mp->smem_bytes = static_cast<int32_t>(smem);
   // rows

@@ -43,14 +43,14 @@ def _long_rows():
 
 
 def _hubs(n, hubs, weights="int8"):
-    # rows of 256 to n / 2 entries, a third of them the other hubs', on a cycle
+    # rows of 400 to n / 2 drawn ends, a third of them the other hubs', on a cycle
     rng = np.random.default_rng(n + hubs)
     ring = np.arange(n, dtype=np.int32)
     src, dst = [ring], [np.roll(ring, -1)]
     for i in range(hubs):
-        d = 256 + (n // 2 - 256) * i // hubs
+        d = 400 + (n // 2 - 400) * i // hubs
         src.append(np.full(d, i, np.int32))
-        dst.append(np.where(np.arange(d) % 3 == 0, rng.integers(0, hubs, d), rng.integers(hubs, n, d)).astype(np.int32))
+        dst.append(np.where((np.arange(d) % 3 == 0) & (hubs > 1), rng.integers(0, hubs, d), rng.integers(hubs, n, d)).astype(np.int32))
     src, dst = np.concatenate(src), np.concatenate(dst)
     keep = src != dst
     return synth.Graph(n, src[keep], dst[keep], synth.draw_weights(weights, int(keep.sum()), rng))
@@ -77,6 +77,7 @@ GRAPHS = {
     "cluster_sparse": lambda: _er(8000, 3),
     "cluster_torus": lambda: synth.torus_graph(57, 2, "pm1", Ly=113),
     "cluster_wide": lambda: _wide(_er(9001, 31)),
+    "cluster_stream": lambda: _wide(_er(12007, 60)),
     "cluster_dense": lambda: _er(3000, 150),
     "cluster_long_rows": _long_rows,
     "grid_er": lambda: _er(60013, 90),
