@@ -145,14 +145,15 @@ __global__ void chunk_sums_kernel(GView v, int4* sums) {
   }
 }
 
-// G1/G2: x_v = [s, f c^2, s f c^2, log(1 + deg) / 8, (sum w) c^2, 1, 0, 0]. Four
+// G1/G2: x_v = [s, f c^2, s f c^2, log(1 + deg) / 8, (sum w) c^2, 1, 0, 0]. L
 // lanes sum a light row's entries (integers, so in any order); a heavy row's
 // sums come from chunk_sums_kernel. One pass over the entries without
 // atomics, fused with the features: on 3.5M entries 38 -> 19 us.
+template <int L>
 __global__ void features_kernel(GView v, const int4* sums, uint4* x, float* cvec) {
-  const int q = threadIdx.x & 3;
-  const int subs = (gridDim.x * blockDim.x) >> 2;
-  for (int p0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 2; p0 - (threadIdx.x >> 2) % 8 < v.n; p0 += subs) {
+  const int q = threadIdx.x % L;
+  const int subs = (gridDim.x * blockDim.x) / L;
+  for (int p0 = (blockIdx.x * blockDim.x + threadIdx.x) / L; p0 - (threadIdx.x / L) % (32 / L) < v.n; p0 += subs) {
     const int p = min(p0, v.n - 1);  // every lane of the warp reaches the shuffles
     const int e0 = __ldg(v.row_ptr + p), e1 = __ldg(v.row_ptr + p + 1);
     const bool heavy = v.hchunk != nullptr && e1 - e0 > kHeavy;
@@ -166,13 +167,13 @@ __global__ void features_kernel(GView v, const int4* sums, uint4* x, float* cvec
       }
     } else {
       const int base = col_base(v, p);
-      for (int e = e0 + q; e < e1; e += 16) {
+      for (int e = e0 + q; e < e1; e += 4 * L) {
         int col[4], w[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           col[u] = p - base;
           w[u] = 0;
-          if (e + 4 * u < e1) edge_at(v.ev, e + 4 * u, col[u], w[u]);
+          if (e + L * u < e1) edge_at(v.ev, e + L * u, col[u], w[u]);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -183,7 +184,7 @@ __global__ void features_kernel(GView v, const int4* sums, uint4* x, float* cvec
       }
     }
 #pragma unroll
-    for (int o = 1; o < 4; o <<= 1) {
+    for (int o = 1; o < L; o <<= 1) {
       a += __shfl_xor_sync(kFull, a, o);
       ws += __shfl_xor_sync(kFull, ws, o);
       fi += __shfl_xor_sync(kFull, fi, o);
@@ -292,7 +293,7 @@ struct RowIO<8> {
 // entries in flight, and the lanes' sums are combined at the end. Both fix
 // the order of every sum.
 constexpr int kFly = 4;
-template <int D>
+template <int D, int FLY = kFly>
 __device__ __forceinline__ void gather_entries(const GView& v, const float* __restrict__ c,
                                                const bf16* __restrict__ src, int e0, int e1, int base,
                                                int q, float (&acc)[RowIO<D>::F]) {
@@ -322,30 +323,26 @@ __device__ __forceinline__ void gather_entries(const GView& v, const float* __re
       for (int u = 0; u < 4; ++u)
         if (u * G + q < cnt) cf[u] *= __ldg(c + col[u]);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (u * G >= cnt) break;
+      for (int j0 = 0; j0 < 4 * G; j0 += FLY) {
+        if (j0 >= cnt) break;
+        typename IO::T hv[FLY];
 #pragma unroll
-        for (int j0 = 0; j0 < G; j0 += kFly) {
-          if (u * G + j0 >= cnt) break;
-          typename IO::T hv[kFly];
-#pragma unroll
-          for (int k = 0; k < kFly; ++k) {
-            const int cj = __shfl_sync(mask, col[u], j0 + k, G);
-            hv[k] = u * G + j0 + k < cnt ? IO::load(src, cj, q) : typename IO::T{};
-          }
-#pragma unroll
-          for (int k = 0; k < kFly; ++k) IO::add(acc, __shfl_sync(mask, cf[u], j0 + k, G), hv[k]);
+        for (int k = 0; k < FLY; ++k) {
+          const int cj = __shfl_sync(mask, col[(j0 + k) / G], (j0 + k) % G, G);
+          hv[k] = j0 + k < cnt ? IO::load(src, cj, q) : typename IO::T{};
         }
+#pragma unroll
+        for (int k = 0; k < FLY; ++k) IO::add(acc, __shfl_sync(mask, cf[(j0 + k) / G], (j0 + k) % G, G), hv[k]);
       }
     }
   } else {
     float a8[8] = {};
-    for (int b = e0 + q; b < e1; b += 4 * G) {
-      int col[4];
-      float cf[4];
-      uint4 hv[4];
+    for (int b = e0 + q; b < e1; b += FLY * G) {
+      int col[FLY];
+      float cf[FLY];
+      uint4 hv[FLY];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < FLY; ++u) {
         col[u] = 0;
         cf[u] = 0.0f;
         if (b + u * G < e1) {
@@ -356,13 +353,13 @@ __device__ __forceinline__ void gather_entries(const GView& v, const float* __re
         }
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < FLY; ++u) {
         const bool ok = b + u * G < e1;
         cf[u] *= ok ? __ldg(c + col[u]) : 0.0f;
         hv[u] = ok ? __ldg(reinterpret_cast<const uint4*>(src) + col[u]) : make_uint4(0, 0, 0, 0);
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < FLY; ++u) {
         const uint32_t words[4] = {hv[u].x, hv[u].y, hv[u].z, hv[u].w};
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -386,7 +383,7 @@ __device__ __forceinline__ void gather_entries(const GView& v, const float* __re
 
 // a_r = c_r * sum_j w_rj c_j src_j for one row (this lane's features): a
 // light row by its entries, a heavy row by its chunks' partial sums.
-template <int D>
+template <int D, int FLY = kFly>
 __device__ __forceinline__ void aggregate_row(const GView& v, const float* __restrict__ c,
                                               const bf16* __restrict__ src, const float* __restrict__ partial,
                                               int r, int q, float (&acc)[RowIO<D>::F]) {
@@ -401,7 +398,7 @@ __device__ __forceinline__ void aggregate_row(const GView& v, const float* __res
       for (int f = 0; f < F; ++f) acc[f] += pp[f];
     }
   } else {
-    gather_entries<D>(v, c, src, e0, e1, col_base(v, r), q, acc);
+    gather_entries<D, FLY>(v, c, src, e0, e1, col_base(v, r), q, acc);
   }
   const float cr = __ldg(c + r);
 #pragma unroll
@@ -409,9 +406,15 @@ __device__ __forceinline__ void aggregate_row(const GView& v, const float* __res
 }
 
 // partial[k] = sum over chunk k's entries of w c_col src[col] (width D), one
-// sub-warp per chunk.
-template <int D>
-__global__ void __launch_bounds__(256)
+// sub-warp per chunk. A chunk is a chain of dependent loads, and a small graph
+// has few of them: blocks of two warps so that they reach every SM, and 16 rows
+// in flight up to kFewChunks chunks an SM (45,787-vertex power-law graph, whole
+// forward pass: 139 us at 8, 133 at 16; at 100,000 vertices, where the warps hide
+// the loads, 188.5 and 191).
+constexpr int kChunkThreads = 64;
+constexpr int kFewChunks = 64;
+template <int D, int FLY>
+__global__ void __launch_bounds__(kChunkThreads)
     chunk_partial_kernel(GView v, const float* __restrict__ c, const bf16* __restrict__ src,
                          float* __restrict__ partial) {
   using IO = RowIO<D>;
@@ -422,7 +425,7 @@ __global__ void __launch_bounds__(256)
     const int e0 = __ldg(v.row_ptr + row) + (k - __ldg(v.hchunk + row)) * kChunk;
     const int e1 = min(e0 + kChunk, __ldg(v.row_ptr + row + 1));
     float acc[IO::F] = {};
-    gather_entries<D>(v, c, src, e0, e1, col_base(v, row), q, acc);
+    gather_entries<D, FLY>(v, c, src, e0, e1, col_base(v, row), q, acc);
     float* out = partial + static_cast<size_t>(k) * D + q * IO::F;
 #pragma unroll
     for (int f = 0; f < IO::F; ++f) out[f] = acc[f];
@@ -473,11 +476,17 @@ __device__ __forceinline__ uint32_t pack_bf162(float x, float y) {
 // flight, spread over warps rather than over registers of one (width 64 at
 // 2 / 3 / 4 / 5 blocks: 199 / 204 / 192 / 197 us for the whole forward pass on a
 // 100k-vertex, 2M-entry power-law graph; width 8 at 4 / 6 / 8: 194 / 193 / 198).
-template <int D>
-constexpr int kLayerBlocks = D == kH ? 4 : 6;
+// A graph of at most kFewTiles tiles an SM cannot fill those blocks, and a row is
+// a chain of loads: there kFewFly rows are in flight (8,352-vertex power-law
+// graph, whole forward pass: 104 us at kFly, 93 with both this and the chunks'
+// deeper gather; at four tiles an SM it costs: 30,000 vertices 53 -> 57).
+template <int D, int FLY>
+constexpr int kLayerBlocks = FLY > kFly ? 2 : D == kH ? 4 : 6;
+constexpr int kFewFly = 8;
+constexpr int kFewTiles = 2;
 
-template <int D>
-__global__ void __launch_bounds__(kLayerThreads, kLayerBlocks<D>)
+template <int D, int FLY>
+__global__ void __launch_bounds__(kLayerThreads, kLayerBlocks<D, FLY>)
     layer_fwd_kernel(GView v, const float* __restrict__ c, const bf16* __restrict__ h,
                      const float* __restrict__ partial, const bf16* __restrict__ W,
                      const float* __restrict__ bias, bf16* __restrict__ a_store, bf16* __restrict__ hout) {
@@ -506,7 +515,7 @@ __global__ void __launch_bounds__(kLayerThreads, kLayerBlocks<D>)
       if (r < n) {
         own = IO::load(h, r, q);
         float acc[IO::F] = {};
-        aggregate_row<D>(v, c, h, partial, r, q, acc);
+        aggregate_row<D, FLY>(v, c, h, partial, r, q, acc);
         ab = IO::pack(acc);
         if (a_store != nullptr) IO::store(a_store, r, q, ab);
       }
@@ -1407,8 +1416,10 @@ int batch_ctx(ising_gnn* net, ising_batch* b, uint32_t replica, Ctx* ctx, isingx
 template <int D>
 int run_chunks(ising_gnn* net, const Ctx& x, const bf16* src) {
   if (x.v.num_chunks <= 0) return ISING_OK;
-  chunk_partial_kernel<D><<<grid_of(static_cast<long long>(x.v.num_chunks) * RowIO<D>::G, 256, x.sms * 16), 256, 0,
-                            x.st>>>(x.v, net->d_c, src, net->d_partial);
+  const bool few = x.v.num_chunks <= kFewChunks * x.sms;
+  (few ? chunk_partial_kernel<D, 16> : chunk_partial_kernel<D, 8>)<<<
+      grid_of(static_cast<long long>(x.v.num_chunks) * RowIO<D>::G, kChunkThreads, x.sms * 32), kChunkThreads, 0,
+      x.st>>>(x.v, net->d_c, src, net->d_partial);
   net->launches++;
   GNN_CUDA(net, cudaGetLastError());
   return ISING_OK;
@@ -1436,8 +1447,9 @@ int run_layer(ising_gnn* net, const Ctx& x, const bf16* h, const bf16* W, const 
       layer_fwd_tc_kernel<D><<<grid, kTcThreads, smem, x.st>>>(x.v, net->d_c, h, net->d_partial, W, bias, a_store,
                                                                hout, net->d_err);
   } else {
-    layer_fwd_kernel<D><<<(n + kTile - 1) / kTile, kLayerThreads, 0, x.st>>>(x.v, net->d_c, h, net->d_partial, W,
-                                                                            bias, a_store, hout);
+    const int tiles = (n + kTile - 1) / kTile;
+    (tiles <= kFewTiles * x.sms ? layer_fwd_kernel<D, kFewFly> : layer_fwd_kernel<D, kFly>)<<<
+        tiles, kLayerThreads, 0, x.st>>>(x.v, net->d_c, h, net->d_partial, W, bias, a_store, hout);
   }
   net->launches++;
   GNN_CUDA(net, cudaGetLastError());
@@ -1466,10 +1478,17 @@ int run_forward(ising_gnn* net, const Ctx& x, bool with_labels) {
   GNN_CUDA(net, ensure_partial(net, x.v.num_chunks));
   if (x.v.num_chunks > 0) {
     GNN_CUDA(net, cudaMemsetAsync(net->d_sums, 0, sizeof(int4) * static_cast<size_t>(n), st));
-    chunk_sums_kernel<<<grid_of(static_cast<long long>(x.v.num_chunks) * 32, 256, sms * 16), 256, 0, st>>>(x.v, net->d_sums);
+    chunk_sums_kernel<<<grid_of(static_cast<long long>(x.v.num_chunks) * 32, 128, sms * 16), 128, 0, st>>>(x.v,
+                                                                                                               net->d_sums);
     net->launches++;
   }
-  features_kernel<<<grid_of(static_cast<long long>(n) * 4, 256, sms * 16), 256, 0, st>>>(
+  // a row's lanes: sixteen, a light row's entries in one round, while that
+  // leaves the rows on one wave of threads; else four, since a row has about ten
+  // entries (8,352-vertex power-law graph: 8.1 us at 4 lanes, 5.1 at 16)
+  const bool few_rows = static_cast<long long>(n) * 16 <= sms * 2048LL;
+  const int lanes = few_rows ? 16 : 4;
+  (few_rows ? features_kernel<16> : features_kernel<4>)<<<grid_of(static_cast<long long>(n) * lanes, 128, sms * 16),
+                                                         128, 0, st>>>(
       x.v, net->d_sums, reinterpret_cast<uint4*>(net->d_x), net->d_c);
   net->launches++;
   GNN_CUDA(net, cudaGetLastError());

@@ -17,7 +17,8 @@ P = pytest.importorskip("paper_1807_10750_gb300")
 
 
 @pytest.mark.parametrize("n,hub", [(31, 30), (33, 32), (63, 62), (64, 63), (65, 64), (127, 65), (128, 127),
-                                   (129, 128), (257, 129), (320, 319), (4097, 640)])
+                                   (129, 128), (257, 129), (320, 319), (4097, 640),
+                                   (19500, 129), (25000, 700)])
 def test_logits_and_gradients_at_tile_edges(n, hub):
     rng = np.random.default_rng(n)
     src = np.concatenate([np.zeros(hub, np.int64), rng.integers(1, n, 2 * n)])
