@@ -9,12 +9,11 @@
 // A graph handle, or a batch's instances taken together as one graph (their
 // disjoint union), is seen through a GView; everything runs by graph
 // position (colour order) on the graph's stream:
-//   rowsum:   per-row sums of |w|, 1, w and w * s_j over the CSR entries,
-//             lanes over entries, segmented warp sums, int atomics at row
-//             ends (exact).
-//   features: x (n x 8 bf16) and c = (d + 1)^-1/2 (G1, G2).
+//   features: per-row sums of |w|, w and w * s_j (integers), a few lanes a
+//             row, a heavy row's from its chunks (int atomics, exact); then
+//             x (n x 8 bf16) and c = (d + 1)^-1/2 (G1, G2).
 //   chunks:   rows with more than kHeavy entries (hubs) are summed in chunks
-//             of kChunk entries, one warp per chunk, into per-chunk partial
+//             of kChunk entries, one sub-warp per chunk, into per-chunk partial
 //             sums of c_j w_rj h_j; the layer kernels add a heavy row's
 //             partials in order. Every aggregate is thus summed in a fixed
 //             order (no float atomics) and no tile waits on a hub.

@@ -216,17 +216,19 @@ __global__ void __launch_bounds__(kHaloBlock, 1)
     __syncthreads();
     // the epoch's flip decisions (Algorithm 2 with R5's draws): one Philox
     // evaluation per quad and sweep sets the bit of every member row that
-    // flips in sweep i's bitmap
-    for (int i = 0; i < se; ++i) {
-      const uint32_t thr0 = sthr[i];
-      if (thr0 == 0u) continue;
-      const uint32_t t = static_cast<uint32_t>(t0) + static_cast<uint32_t>(i);
-      unsigned* bits = sflip + i * nslices;
-      for (int q = threadIdx.x; q < nquads; q += kHaloBlock) {
-        const uint4 x = philox4x32_10(squad[3 * q], t, replica, 0u, rk);
-        const uint32_t s01 = squad[3 * q + 1], s23 = squad[3 * q + 2];
+    // flips in sweep i's bitmap. A third of the kernel's instructions were
+    // these; what a quad's sweeps share of the first two rounds is formed once
+    // (1024 x 1024 torus, 200 sweeps: 1222 -> 1207 us).
+    for (int q = threadIdx.x; q < nquads; q += kHaloBlock) {
+      const PhiloxQuad quad = philox_quad(squad[3 * q], replica, 0u, rk);
+      const uint32_t s01 = squad[3 * q + 1], s23 = squad[3 * q + 2];
+      const uint32_t slot[4] = {s01 & 0xffffu, s01 >> 16, s23 & 0xffffu, s23 >> 16};
+      for (int i = 0; i < se; ++i) {
+        const uint32_t thr0 = sthr[i];
+        if (thr0 == 0u) continue;
+        unsigned* bits = sflip + i * nslices;
+        const uint4 x = philox_at(quad, static_cast<uint32_t>(t0) + static_cast<uint32_t>(i), replica, rk);
         const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
-        const uint32_t slot[4] = {s01 & 0xffffu, s01 >> 16, s23 & 0xffffu, s23 >> 16};
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           if (slot[k] == 0xffffu) continue;

@@ -78,6 +78,39 @@ __device__ __forceinline__ uint4 philox4x32_10(uint32_t x0, uint32_t x1, uint32_
   return make_uint4(x0, x1, x2, x3);
 }
 
+// Philox4x32-10 at counters (q, t, replica, s) for several t: what the first
+// two rounds make of q alone, and the rest.
+struct PhiloxQuad {
+  uint32_t x0, x1, x2;  // the second round's words, the third without t's part
+};
+
+__device__ __forceinline__ PhiloxQuad philox_quad(uint32_t q, uint32_t replica, uint32_t s, const PhiloxRounds& rk) {
+  const uint64_t pa = static_cast<uint64_t>(0xD2511F53u) * q;
+  const uint64_t pb = static_cast<uint64_t>(0xCD9E8D57u) * replica;
+  const uint32_t n2 = static_cast<uint32_t>(pa >> 32) ^ s ^ rk.hi[0];
+  const uint64_t pc = static_cast<uint64_t>(0xCD9E8D57u) * n2;
+  return {static_cast<uint32_t>(pc >> 32) ^ static_cast<uint32_t>(pb) ^ rk.lo[1], static_cast<uint32_t>(pc),
+          static_cast<uint32_t>(pa) ^ rk.hi[1]};
+}
+
+__device__ __forceinline__ uint4 philox_at(const PhiloxQuad& p, uint32_t t, uint32_t replica, const PhiloxRounds& rk) {
+  const uint64_t pb = static_cast<uint64_t>(0xCD9E8D57u) * replica;
+  const uint64_t pd = static_cast<uint64_t>(0xD2511F53u) * (static_cast<uint32_t>(pb >> 32) ^ t ^ rk.lo[0]);
+  uint32_t x0 = p.x0, x1 = p.x1, x2 = p.x2 ^ static_cast<uint32_t>(pd >> 32), x3 = static_cast<uint32_t>(pd);
+#pragma unroll
+  for (int r = 2; r < 10; ++r) {
+    const uint64_t a = static_cast<uint64_t>(0xD2511F53u) * x0;
+    const uint64_t b = static_cast<uint64_t>(0xCD9E8D57u) * x2;
+    const uint32_t n0 = static_cast<uint32_t>(b >> 32) ^ x1 ^ rk.lo[r];
+    const uint32_t n2 = static_cast<uint32_t>(a >> 32) ^ x3 ^ rk.hi[r];
+    x1 = static_cast<uint32_t>(b);
+    x3 = static_cast<uint32_t>(a);
+    x0 = n0;
+    x2 = n2;
+  }
+  return make_uint4(x0, x1, x2, x3);
+}
+
 // The draw of vertex o (original id) in sweep t of replica r on stream s (0
 // flips, 1 initial spins): word o mod 4 of counter (o / 4, t, r, s), so the
 // four vertices 4q .. 4q + 3 share one evaluation.
