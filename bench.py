@@ -99,21 +99,21 @@ def algorithmic_bytes_per_sweep(n: int, nnz: int, entry_bytes: int) -> int:
 # the sweeps. The entry holds only while the kernel sources hash to `sources`:
 # once they change the counters are stale and traffic is reported as null.
 NCU_TRAFFIC = {
-    "zipf1m": {"fixed": 99.3e6, "per_sweep": 11.61e6, "kernel": "hub_kernel", "engine": "hub",
+    "zipf1m": {"fixed": 97.6e6, "per_sweep": 12.38e6, "kernel": "hub_kernel", "engine": "hub",
                "files": ('hub.cuh', 'sweep.cuh', 'philox.cuh', 'anneal.cu'),
-               "sources": "263febaf28510827",
-               "how": "ncu 4- and 12-sweep captures: 145.73 MB and 238.62 MB (read + write); the "
+               "sources": "3984244a39941fb0",
+               "how": "ncu 4- and 12-sweep captures: 147.13 MB and 246.21 MB (read + write); the "
                       "CSR is read from DRAM once and then mostly served from L2"},
-    "torus1024": {"fixed": 31.79e6, "per_sweep": 4.03e3, "kernel": "halo_kernel",
+    "torus1024": {"fixed": 31.80e6, "per_sweep": 3.32e3, "kernel": "halo_kernel",
                   "engine": "halo",
                   "files": ('halo.cuh', 'halo_plan.cpp', 'host_graph.h', 'philox.cuh', 'sweep.cuh'),
-                  "sources": "6bf5d71760ec383b",
-                  "how": "ncu 20- and 40-sweep captures: 31.870 MB and 31.951 MB, so the "
+                  "sources": "aa10d359c3f8355f",
+                  "how": "ncu 20- and 40-sweep captures: 31.869 MB and 31.936 MB, so the "
                          "working set is read once and then stays in shared memory and L2"},
-    "batched": {"fixed": 0.2126e9, "per_sweep": 0.2083e9, "kernel": "batch_anneal_kernel",
-                "files": ('batch.cu', 'philox.cuh'),
-                "sources": "cb30dcc0eb10999b",
-                "how": "ncu 20- and 60-sweep captures: 4.379 GB and 12.710 GB"},
+    "batched": {"fixed": 0.2490e9, "per_sweep": 0.1997e9, "kernel": "batch_map_kernel",
+                "files": ('batch.cu', 'batch_map.cuh', 'cluster.cuh', 'philox.cuh'),
+                "sources": "0a8224281505d3a7",
+                "how": "ncu 20- and 60-sweep captures: 4.243 GB and 12.231 GB"},
 }
 
 
@@ -401,7 +401,7 @@ def run_batched(args, world, rank, P, torch, dist):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": kernel_traffic("batched", T),
                      "peak_kind": peak_kind, "bytes_per_sweep": B, "bytes_per_launch": B * T,
-                     "kernel": "batch_anneal_kernel (one launch per step)"},
+                     "kernel": "batch_map_kernel (clusters by instance size) or, where tuned so, batch_anneal_kernel"},
         "cpu_baseline": None, "e2e": e2e, "gpu_launches": int(launches), "clocks": clocks.summary(),
     }
     print(json.dumps(line), flush=True)
@@ -593,9 +593,10 @@ def run_warmstart(args, world, rank, P, torch, dist):
 
 
 def gnn_forward_bytes(n: int, nnz: int) -> int:
-    """Compulsory bytes of one forward pass of the warm-start network: row
-    sums (CSR word, row id, neighbour spin per entry; an int4 per row out),
-    features (sums, spin in; 8 bf16 features and c out), three layers (per
+    """Algorithmic bytes of one forward pass of the warm-start network: row
+    sums (CSR word, row id, neighbour spin per entry; an int4 per row out, as
+    the form this figure began with; the current one needs neither id nor
+    int4), features (sums, spin in; 8 bf16 features and c out), three layers (per
     entry the CSR word, c_j and the neighbour's bf16 feature row; per row its
     row bounds, c, its own row in and its 64-wide bf16 output) and the head
     (h3 in, z out). The aggregate a never leaves the layer kernel, so it
@@ -680,11 +681,11 @@ def run_gnn(args, world, rank, P, torch, dist):
 # wavefronts (one wavefront moves up to 128 bytes) from ncu captures, slope
 # over the sweep count; valid while the kernel sources hash to `sources`.
 NCU_SMEM = {
-    "torus1024": {"wavefronts_per_sweep": 575_506,
+    "torus1024": {"wavefronts_per_sweep": 565_575,
                   "files": ('halo.cuh', 'halo_plan.cpp', 'host_graph.h', 'philox.cuh', 'sweep.cuh'),
-                  "sources": "6bf5d71760ec383b",
-                  "how": "l1tex__data_pipe_lsu_wavefronts_mem_shared.sum: 11,810,305 (20 sweeps) and "
-                         "23,320,433 (40 sweeps)"},
+                  "sources": "aa10d359c3f8355f",
+                  "how": "l1tex__data_pipe_lsu_wavefronts_mem_shared.sum: 11,646,942 (20 sweeps) and "
+                         "22,958,439 (40 sweeps)"},
 }
 
 
