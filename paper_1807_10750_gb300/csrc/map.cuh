@@ -20,9 +20,9 @@
 //   * the grid: messages of 32 spins and a 32-bit sequence number in one
 //     64-bit word, so a reader that polls the word gets data and arrival at
 //     once (one L2 round trip instead of a barrier's and a refresh's). Two
-//     buffers alternate by sweep: a block writes a message of sweep t + 2 only
-//     after it has read a message of sweep t + 1 from every block, each of which
-//     was sent after its block had read sweep t.
+//     buffers alternate by class step: a block writes a message of step t + 2 only
+//     after it has read a message of step t + 1 from every block, each of which
+//     was sent after its block had read step t.
 // The flips of sweep t + 1 are drawn while sweep t runs, by the warps with no
 // unit left, and Algorithm 1's picks by a kernel before this one (they do not
 // depend on the spins).
