@@ -40,6 +40,7 @@
 #include "halo.cuh"
 #include "hub.cuh"
 #include "map.cuh"
+#include "shared_limit.h"
 
 using isingx::HostGraph;
 using isingx::PhiloxKey;
@@ -678,8 +679,7 @@ cudaError_t launch_block(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint
   ba.wait_ns = static_cast<long long>(g->wait_budget_ns);
   ba.short_copy = g->fault_kind == ISING_FAULT_SHORT_COPY ? 1 : 0;
   const int smem = isingx::block_layout(ba.n, ba.num_chunks, ba.num_classes).total;
-  cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(block_kernel),
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = isingx::allow_shared(reinterpret_cast<const void*>(block_kernel), g->device, static_cast<size_t>(smem));
   if (e != cudaSuccess) return e;
   e = barrier_init(g);
   if (e != cudaSuccess) return e;
@@ -800,7 +800,7 @@ cudaError_t plan_halo(ising_graph* g, bool wait) {
   g->pending.reset();
   if (!hp.ok) return cudaSuccess;
   auto kernel = isingx::halo_kernel;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hp.smem_bytes);
+  cudaError_t e = isingx::allow_shared(reinterpret_cast<const void*>(kernel), g->device, static_cast<size_t>(hp.smem_bytes));
   if (e != cudaSuccess) {
     cudaGetLastError();
     return cudaSuccess;  // the device cannot give this much shared memory: no plan
@@ -896,7 +896,7 @@ cudaError_t launch_hub_t(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint
   const bool stage = STAGE;
   const int smem = isingx::hub_smem_bytes(g->num_hubs, g->hub_colours, bit_words, stage);
   if (smem > optin) return cudaErrorCooperativeLaunchTooLarge;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  e = isingx::allow_shared(reinterpret_cast<const void*>(kernel), g->device, static_cast<size_t>(smem));
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, isingx::kHubBlock, smem);
@@ -1003,9 +1003,9 @@ void map_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int mode, in
 
 // Whether the device can run a plan: shared memory, a cluster of that size, or
 // K co-resident blocks.
-bool map_fits(const isingx::MapPlan& mp, bool wide) {
+bool map_fits(const isingx::MapPlan& mp, bool wide, int device) {
   const void* kernel = map_kernel_for(mp.mode, wide, mp.stage, mp.hubs > 0, mp.resident);
-  bool fits = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, mp.smem_bytes) == cudaSuccess;
+  bool fits = isingx::allow_shared(kernel, device, static_cast<size_t>(mp.smem_bytes)) == cudaSuccess;
   if (fits && mp.mode == isingx::kMapCluster) {
     fits = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     cudaLaunchConfig_t cfg;
@@ -1014,10 +1014,9 @@ bool map_fits(const isingx::MapPlan& mp, bool wide) {
     int clusters = 0;
     fits = fits && cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters >= 1;
   } else if (fits && mp.mode == isingx::kMapGrid) {
-    int per_sm = 0, sms = 0, dev = 0, coop = 0;
-    fits = cudaGetDevice(&dev) == cudaSuccess &&
-           cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-           cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop != 0 &&
+    int per_sm = 0, sms = 0, coop = 0;
+    fits = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) == cudaSuccess &&
+           cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device) == cudaSuccess && coop != 0 &&
            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * mp.warps,
                                                          static_cast<size_t>(mp.smem_bytes)) == cudaSuccess &&
            per_sm * sms >= mp.K;
@@ -1045,7 +1044,7 @@ void choose_map_plan(const HostGraph& hg, int num_sms, int device, bool wide, bo
   const int64_t work = hg.nnz + 8 * static_cast<int64_t>(hg.n), classes = std::max(1, hg.num_colours);
   auto build = [&](int mode, int K) {
     isingx::build_map_plan(hg, mode, K, wide, optin, mp, split);
-    return mp->ok && map_fits(*mp, wide);
+    return mp->ok && map_fits(*mp, wide, device);
   };
   if (!split && work <= 4000 * classes && (build(isingx::kMapBlock, 1) || build(isingx::kMapBlockStream, 1))) return;
   if ((lattice ? hg.n <= 100000 : work <= 300000 * classes) &&
@@ -1116,7 +1115,7 @@ cudaError_t launch_map(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint64
                        uint32_t replica, const isingx::PhiloxRounds& rk, uint32_t n0, int par0) {
   const bool wide = !g->packed;
   const void* kernel = map_kernel_for(g->map_mode, wide, g->map_stage, g->map_accs > 0, g->map_resident);
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, g->map_smem);
+  cudaError_t e = isingx::allow_shared(kernel, g->device, static_cast<size_t>(g->map_smem));
   if (e != cudaSuccess) return e;
   if (g->map_mode == isingx::kMapCluster &&
       (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)

@@ -31,6 +31,7 @@
 #include "batch_view.h"
 #include "host_graph.h"
 #include "philox.cuh"
+#include "shared_limit.h"
 
 namespace {
 
@@ -638,7 +639,7 @@ cudaError_t group_upload(ising_batch* b, const isingx::BatchMapPlan& p, const in
                          bool* runs) {
   const void* kernel = batch_map_kernel_for(p.K > 1, p.unit);
   int clusters = 0;
-  *runs = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem) == cudaSuccess;
+  *runs = isingx::allow_shared(kernel, b->device, static_cast<size_t>(p.smem)) == cudaSuccess;
   if (p.K == 1) {
     *runs = *runs && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&clusters, kernel, isingx::kBatchMapThreads,
                                                                    static_cast<size_t>(p.smem)) == cudaSuccess;
@@ -749,7 +750,7 @@ int groups_launch(ising_batch* b, uint64_t t_begin, uint32_t sweeps, uint64_t T,
   for (size_t i = 0; i < b->groups.size(); ++i) {
     BatchMapGroup& g = b->groups[i];
     const void* kernel = batch_map_kernel_for(g.K > 1, g.unit);
-    BATCH_CUDA(b, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, g.smem));
+    BATCH_CUDA(b, isingx::allow_shared(kernel, b->device, static_cast<size_t>(g.smem)));
     if (g.K > 1) BATCH_CUDA(b, cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     isingx::BatchMapArgs a{};
     a.inst = g.inst;
@@ -796,8 +797,7 @@ int batch_launch(ising_batch* b, uint64_t t_begin, uint32_t sweeps, uint64_t T, 
   if (!b->groups.empty() && !b->tuned) return groups_launch(b, t_begin, sweeps, T, T0, seed);
   const size_t smem = static_cast<size_t>(std::max(b->max_n, 1));
   const void* kernel = batch_kernel_for(b->block, b->split);
-  BATCH_CUDA(b, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(smem)));
+  BATCH_CUDA(b, isingx::allow_shared(kernel, b->device, smem));
   const int grid = batch_grid(b, b->block, b->split, smem);
   BatchDev d = b->dev();
   int num_graphs = b->num_graphs;
