@@ -1054,6 +1054,12 @@ void choose_map_plan(const HostGraph& hg, int num_sms, int device, bool wide, bo
   mp->ok = false;
 }
 
+// Algorithm 1's picks for the launches of a handle: made with it, so that an
+// anneal neither allocates nor waits and a captured one keeps its addresses. Of
+// kPickInts + 8 n picks, 1,300 sweeps of 200 or eight of n; at most kPickSweeps.
+constexpr size_t kPickInts = size_t(1) << 18;
+constexpr size_t kPickSweeps = size_t(1) << 14;
+
 cudaError_t upload_map_plan(ising_graph* g, const isingx::MapPlan& mp) {
   cudaError_t e;
   if ((e = alloc_copy(&g->d_map_blocks, mp.blocks.data(), mp.blocks.size(), g->stream)) != cudaSuccess) return e;
@@ -1083,6 +1089,11 @@ cudaError_t upload_map_plan(ising_graph* g, const isingx::MapPlan& mp) {
                                            2 * static_cast<size_t>(mp.K) * static_cast<size_t>(mp.mail_stride), g->stream)) != cudaSuccess)
     return e;
   if ((e = alloc_copy(&g->d_map_late, mp.late.data(), mp.late.size(), g->stream)) != cudaSuccess) return e;
+  if (mp.hubs == 0) {
+    g->pick_cap = kPickInts + 8 * static_cast<size_t>(g->n);
+    if ((e = cudaMalloc(reinterpret_cast<void**>(&g->d_pick_count), kPickSweeps * sizeof(uint32_t))) != cudaSuccess) return e;
+    if ((e = cudaMalloc(reinterpret_cast<void**>(&g->d_picks), g->pick_cap * sizeof(int32_t))) != cudaSuccess) return e;
+  }
   const int2* late = reinterpret_cast<const int2*>(g->d_map_late);
   const dim3 grid(static_cast<unsigned>(mp.K), mp.mode == isingx::kMapGrid ? 4u : 32u);
   if (g->packed)
@@ -1147,27 +1158,11 @@ cudaError_t launch_map(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint64
   a.budget = g->wait_budget_ns > 0 ? static_cast<long long>(g->wait_budget_ns) : isingx::kBarrierBudgetNs;
   a.error = &g->d_barrier->error;
   a.skip_block = g->fault_kind == ISING_FAULT_SKIP_ARRIVAL ? 1 : 0;
-  // Algorithm 1: the picks of as many sweeps as kPickInts holds, then those
-  // sweeps, and so on
-  constexpr size_t kPickInts = size_t(1) << 22;
+  // Algorithm 1: the picks of as many sweeps as the handle's buffer holds (n0 <=
+  // n of them a sweep), then those sweeps, and so on
   size_t chunk = sweeps;
   if (n0 != 0u) {
-    chunk = std::min<size_t>(sweeps, std::max<size_t>(1, kPickInts / n0));
-    if (chunk > g->pick_sweeps || chunk * n0 > g->pick_cap) {
-      cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-      if ((e = cudaStreamIsCapturing(g->stream, &capture)) != cudaSuccess) return e;
-      if (capture != cudaStreamCaptureStatusNone) return cudaErrorMemoryAllocation;
-      if ((e = cudaStreamSynchronize(g->stream)) != cudaSuccess) return e;
-      cudaFree(g->d_pick_count);
-      cudaFree(g->d_picks);
-      g->d_pick_count = nullptr;
-      g->d_picks = nullptr;
-      g->pick_sweeps = g->pick_cap = 0;
-      if ((e = cudaMalloc(reinterpret_cast<void**>(&g->d_pick_count), chunk * sizeof(uint32_t))) != cudaSuccess) return e;
-      if ((e = cudaMalloc(reinterpret_cast<void**>(&g->d_picks), chunk * n0 * sizeof(int32_t))) != cudaSuccess) return e;
-      g->pick_sweeps = chunk;
-      g->pick_cap = chunk * n0;
-    }
+    chunk = std::min<size_t>({chunk, kPickSweeps, g->pick_cap / n0});
     a.pick_count = g->d_pick_count;
     a.picks = g->d_picks;
     a.pick_stride = static_cast<int32_t>(n0);
@@ -1718,10 +1713,8 @@ static int anneal_impl(ising_graph* g, const ising_schedule* sched, uint32_t swe
     g->engine_used = engine == ISING_ENGINE_ITEMFLOW ? ISING_ENGINE_ITEMFLOW
                      : g->block_ok                   ? ISING_ENGINE_USED_BLOCK
                                                      : ISING_ENGINE_PERSISTENT_GRID;
-    const cudaError_t e = launch_map(g, sched->t_begin, sweeps, sched->t_total, T0, sched->replica, rk, n0, par0);
-    if (e == cudaSuccess) return ISING_OK;
-    if (e != cudaErrorMemoryAllocation) return cuda_fail(g, e);
-    cudaGetLastError();  // no room for Algorithm 1's picks: an engine that draws them as it goes
+    ISING_CUDA(g, launch_map(g, sched->t_begin, sweeps, sched->t_total, T0, sched->replica, rk, n0, par0));
+    return ISING_OK;
   }
   if (engine == ISING_ENGINE_ITEMFLOW) {
     if (mode == ISING_MODE_DET && !nflip && g->itemflow_ok) {

@@ -126,9 +126,9 @@ struct ising_graph {
   int32_t* d_map_index = nullptr;      // position -> map index
   int32_t* d_map_late = nullptr;       // per split row: its entries in the class before
   unsigned long long* d_map_mail = nullptr;
-  uint32_t* d_pick_count = nullptr;    // Algorithm 1's picks of a launch (grown on use)
+  uint32_t* d_pick_count = nullptr;    // Algorithm 1's picks of a launch: how many after each sweep
   int32_t* d_picks = nullptr;
-  size_t pick_sweeps = 0, pick_cap = 0;
+  size_t pick_cap = 0;
   uint8_t* d_bias = nullptr;         // per-position flip bias (null: none)
   int32_t* d_gnn_hchunk = nullptr;   // warm-start network: per row, its first entry chunk or -1
   int32_t* d_gnn_chunk_row = nullptr;  // warm-start network: the row of every entry chunk
