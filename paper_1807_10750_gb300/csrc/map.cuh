@@ -57,9 +57,12 @@
 // split, parts in the row's own block / as it is: 5,000 vertices 46 / 17 / 16 /
 // 16, 20,000 vertices 63 / 48 / 34 / 32, 100,000 vertices 93 / 154 / 83 / 63.
 //
-// Every wait is bounded (the handle's budget): then the error flag is set,
-// every block leaves its loop, and the blocks of a cluster meet once more
-// before they exit, so that no store reaches a block that has gone.
+// Every wait is bounded (the handle's budget): then the error flag is set, the
+// other blocks' waits end by it, every block leaves its loop, and the blocks of
+// a cluster meet once more before they exit, so that no store reaches a block
+// that has gone. A sweep with Algorithm 1's flips ends in a cluster barrier that
+// a block still at work counts on: a warp whose wait ran out goes straight to it
+// and says so in every block, and all of them leave together behind it.
 #pragma once
 
 #include <cstdint>
@@ -184,6 +187,7 @@ __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
   uint32_t* flips = reinterpret_cast<uint32_t*>(orig + a.rows_max);
   uint8_t* bias = reinterpret_cast<uint8_t*>(flips + 2 * (a.rows_max / 32));
   uint64_t* bars = reinterpret_cast<uint64_t*>(bias + a.rows_max);
+  volatile int* failed = reinterpret_cast<volatile int*>(bars + 2);  // cluster: a wait of some block ran out
   const int flip_words = a.rows_max / 32;
 
   int32_t* acc = reinterpret_cast<int32_t*>(bars + 8);
@@ -217,11 +221,12 @@ __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(warps) : "memory");
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar + 8), "r"(warps) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    *failed = 0;
   }
   // this lane's share of a unit's stores: 16 bytes at most, to one block. The
   // failure-detection tests' block sends nothing.
   const bool skip = a.skip_block == k_me + 1;
-  bool sends = CLUSTER && (lane & 15) < K && !skip;
+  const bool sends = CLUSTER && (lane & 15) < K && !skip;
   uint32_t map_to = 0, bar_to = 0;
   if (sends) {
     map_to = cluster_addr(smem_u32(map), lane & 15) + (lane & 16);
@@ -333,7 +338,7 @@ __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
 #pragma unroll
         for (int g = 0; g < G; ++g) f += map_group<WIDE>(map, st.w[g], st.c[WIDE ? g : 0]);
         f = __reduce_add_sync(kFullMask, f);
-        if (lane == 0 && ok && !skip)
+        if (lane == 0 && !skip)
           asm volatile("red.async.relaxed.cluster.shared::cluster.mbarrier::complete_tx::bytes.add.s32 [%0], %1, [%2];" ::"r"(
                            owner(smem_u32(acc), 1, t)),
                        "r"(f), "r"(owner(bar + 8 * (step & 1u), 0, t))
@@ -398,7 +403,7 @@ __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
       if (CLUSTER) {
         const uint32_t on = bar + 8 * (step & 1u);
         __syncwarp();
-        if (lane == 0 && ok) {
+        if (lane == 0) {
           if (warp == 0)
             asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(on), "r"(cbytes[c])
                          : "memory");
@@ -407,12 +412,13 @@ __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
         }
         const uint32_t parity = (step >> 1) & 1u;
         if (__any_sync(kFullMask, !map_try(on, parity))) {
-          if (ok) ok = __all_sync(kFullMask, map_wait(on, parity, a.error, a.budget));
-          // a warp whose wait ran out leaves for the last cluster barrier; under
-          // Algorithm 1 it runs on, without stores, arrivals or waits, through
-          // the barriers that every sweep has
-          sends = sends && ok;
-          if (!ok && a.pick_count == nullptr) goto done;
+          ok = __all_sync(kFullMask, map_wait(on, parity, a.error, a.budget));
+          if (!ok) {
+            // to the next cluster barrier: the sweep's, or the last one (N_t only
+            // falls, so no later sweep has one either)
+            if (npick == 0u) goto done;
+            break;
+          }
         }
       } else if (MODE != kMapGrid) {
         __syncthreads();
@@ -454,14 +460,21 @@ __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
     }
     // 6. Algorithm 1's flips of the sweep, into every block's map
     if (npick != 0u) {
-      for (uint32_t i = tid; i < npick; i += threads) {
+      for (uint32_t i = ok ? tid : npick; i < npick; i += threads) {
         const int p = i == static_cast<uint32_t>(tid) ? pick : __ldg(a.picks + static_cast<size_t>(k) * a.pick_stride + i);
         map[p] = static_cast<int8_t>(-map[p]);
       }
-      if (CLUSTER)
+      if (CLUSTER) {
+        if (!ok && lane < K)
+          asm volatile("st.shared::cluster.s32 [%0], 1;" ::"r"(cluster_addr(bar + 16, lane)) : "memory");
         cluster_sync();  // no block's next spins may come before this block's flips
-      else
+        if (*failed != 0) {
+          ok = false;
+          break;
+        }
+      } else {
         __syncthreads();
+      }
     }
   }
 done:
@@ -471,7 +484,10 @@ done:
       const int p = __ldg(a.row_pos + B.row0 + r);
       if (p >= 0) d.spins[p] = static_cast<int8_t>(state_byte(map[cseg[c] + r - crow[c]], a.par_end));
     }
-  if (CLUSTER) cluster_sync();
+  if (CLUSTER) {
+    if (!ok) __nanosleep(20000);  // its last stores may still be on their way (a fraction of a microsecond)
+    cluster_sync();
+  }
 }
 
 // The entries of a plan's units (host_graph.h, MapPlan) from the graph's rows:
