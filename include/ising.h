@@ -403,6 +403,15 @@ int ising_batch_set_tuning(ising_batch* b, int32_t block, int32_t row_split, int
  * split 1/2/4, tail 0/32; 0 before any autotune). Any pointer may be NULL. */
 int ising_batch_tuning(ising_batch* b, int32_t* out_block, int32_t* out_row_split, int32_t* out_tail,
                        float* out_probe_ms);
+/* ising_batch_debug_fault -- failure-detection test hook, as ising_debug_fault:
+ * ISING_FAULT_SKIP_ARRIVAL keeps the first block of every cluster from sending
+ * its spins, so that the clustered form's waits run out; wait_budget_ns bounds
+ * every wait of later anneals (0: the default, 2 s; at most 60 s). The next call
+ * that synchronises reports ISING_ETIMEOUT and latches it in the batch: cuts,
+ * get / set spins, autotune, and the warm-start network's calls on the batch (a
+ * train step on such spins leaves the weights as they are). The one-block
+ * kernel has no waits. */
+int ising_batch_debug_fault(ising_batch* b, int kind, uint64_t wait_budget_ns);
 /* ising_batch_info -- instances, total vertices, block size, kernel launches. */
 int ising_batch_info(ising_batch* b, int32_t* out_num_graphs, int64_t* out_vertices,
                      int32_t* out_block, uint64_t* out_launches);

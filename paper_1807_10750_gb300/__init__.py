@@ -58,7 +58,7 @@ EXPORTS = (
     "ising_engine_used", "ising_set_halo_sweeps", "ising_halo_info", "ising_plan_halo",
     "ising_convergence_region", "ising_batch_set_tuning", "ising_batch_tuning",
     "ising_gnn_batch_forward", "ising_gnn_batch_warm_start", "ising_gnn_batch_gradients",
-    "ising_gnn_batch_train_step", "ising_gnn_set_dense_path",
+    "ising_gnn_batch_train_step", "ising_gnn_set_dense_path", "ising_batch_debug_fault",
 )
 ISING_ENGINE_USED_BLOCK = 6
 ISING_FAULT_NONE = 0
@@ -154,6 +154,7 @@ def lib():
         L.ising_gnn_destroy.argtypes = [vp]
         L.ising_gnn_destroy.restype = None
         L.ising_debug_fault.argtypes = [vp, ctypes.c_int, ctypes.c_uint64]
+        L.ising_batch_debug_fault.argtypes = [vp, ctypes.c_int, ctypes.c_uint64]
         L.ising_engine_used.argtypes = [vp, ctypes.POINTER(ctypes.c_int32)]
         L.ising_set_halo_sweeps.argtypes = [vp, ctypes.c_uint32]
         L.ising_plan_halo.argtypes = [ctypes.c_int32, ctypes.c_int64, vp, vp, vp, ctypes.c_int32,
@@ -552,6 +553,11 @@ def ising_batch_tuning(b: IsingBatch) -> dict:
     _check(lib().ising_batch_tuning(b.ptr, ctypes.byref(blk), ctypes.byref(split), ctypes.byref(tail),
                                     probe.ctypes.data), "ising_batch_tuning")
     return {"block": blk.value, "row_split": split.value, "tail": tail.value, "probe_ms": probe.tolist()}
+
+
+def ising_batch_debug_fault(b: IsingBatch, kind: int, wait_budget_ns: int = 0) -> None:
+    """Failure-detection test hook (see include/ising.h)."""
+    _check(lib().ising_batch_debug_fault(b.ptr, kind, wait_budget_ns), "ising_batch_debug_fault")
 
 
 def ising_batch_info(b: IsingBatch) -> dict:

@@ -381,8 +381,9 @@ __global__ void batch_init_kernel(BatchDev d, uint32_t seed_lo, uint32_t seed_hi
   }
 }
 
-// twice the energy of every replica of every instance: sum_v s_v f_v (one block per instance)
-__global__ void batch_energy_kernel(BatchDev d, int replicas, long long* out2) {
+// twice the energy of every replica of every instance: sum_v s_v f_v (one block per instance);
+// behind them the error flag of the clustered form
+__global__ void batch_energy_kernel(BatchDev d, int replicas, const unsigned* error, long long* out2) {
   const BatchGraph G = d.graphs[blockIdx.x];
   const int32_t* rp = d.row_ptr + G.row_base;
   long long acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -409,6 +410,7 @@ __global__ void batch_energy_kernel(BatchDev d, int replicas, long long* out2) {
     for (int k = 0; k < static_cast<int>(blockDim.x >> 5); ++k) s += part[threadIdx.x][k];
     out2[static_cast<size_t>(blockIdx.x) * replicas + threadIdx.x] = s;
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) out2[static_cast<size_t>(gridDim.x) * replicas] = *error;
 }
 
 // One replica's spins of an instance by vertex id (+1 / -1) into out[0, n), the
@@ -490,6 +492,8 @@ struct ising_batch {
   std::vector<BatchMapGroup> groups;
   bool tuned = false;
   cudaEvent_t fork = nullptr;
+  int fault_kind = ISING_FAULT_NONE;  // ising_batch_debug_fault
+  uint64_t wait_budget_ns = 0;
   int8_t* d_out = nullptr;  // ising_batch_get_spins: max_n + 1 bytes, and their pinned copy
   int8_t* h_out = nullptr;
   // the instances as one graph, for the warm-start network (batch_union)
@@ -771,7 +775,8 @@ int groups_launch(ising_batch* b, uint64_t t_begin, uint32_t sweeps, uint64_t T,
     a.map_bytes = g.map_bytes;
     a.units_max = g.units_max;
     a.classes_max = g.classes_max;
-    a.budget = isingx::kBarrierBudgetNs;
+    a.budget = b->wait_budget_ns > 0 ? static_cast<long long>(b->wait_budget_ns) : isingx::kBarrierBudgetNs;
+    a.silent = b->fault_kind == ISING_FAULT_SKIP_ARRIVAL ? 1 : 0;
     uint32_t seed_lo = static_cast<uint32_t>(seed), seed_hi = static_cast<uint32_t>(seed >> 32);
     const cudaStream_t s = i == 0 ? b->stream : g.stream;
     if (i > 0) BATCH_CUDA(b, cudaStreamWaitEvent(s, b->fork, 0));
@@ -978,7 +983,7 @@ int ising_batch_create(int32_t num_graphs, const int32_t* n, const int64_t* m, c
     if ((e = cudaMalloc(reinterpret_cast<void**>(&b->d_flips), std::max<int64_t>(vtx, 16))) != cudaSuccess) break;
     if ((e = cudaMalloc(reinterpret_cast<void**>(&b->d_work), kBatchWork * sizeof(unsigned))) != cudaSuccess) break;
     if ((e = cudaMalloc(reinterpret_cast<void**>(&b->d_energy2),
-                        sizeof(long long) * (size_t)num_graphs * replicas)) != cudaSuccess) break;
+                        sizeof(long long) * ((size_t)num_graphs * replicas + 1))) != cudaSuccess) break;
     if ((e = cudaMemsetAsync(b->d_work, 0, kBatchWork * sizeof(unsigned), b->stream)) != cudaSuccess) break;
     if ((e = cudaStreamSynchronize(b->stream)) != cudaSuccess) break;
     if (map_rows_ok) try {
@@ -1028,6 +1033,8 @@ int batch_union(ising_batch* b, BatchUnion* out) {
   out->vbase = b->d_union_vbase;
   out->orig = b->d_orig;
   out->spins = b->d_spins;
+  out->error = b->d_work + kBatchError;
+  out->status = &b->status;
   out->hchunk = &b->d_gnn_hchunk;
   out->chunk_row = &b->d_gnn_chunk_row;
   out->num_chunks = &b->gnn_num_chunks;
@@ -1074,14 +1081,18 @@ int ising_batch_cuts(ising_batch* b, int64_t* out_cuts) {
   int rc = batch_enter(b);
   if (rc != ISING_OK) return rc;
   if (out_cuts == nullptr) return ISING_EINVAL;
-  batch_energy_kernel<<<b->num_graphs, 256, 0, b->stream>>>(b->dev(), b->replicas, b->d_energy2);
+  batch_energy_kernel<<<b->num_graphs, 256, 0, b->stream>>>(b->dev(), b->replicas, b->d_work + kBatchError,
+                                                            b->d_energy2);
   b->launches++;
   BATCH_CUDA(b, cudaGetLastError());
-  std::vector<long long> e2((size_t)b->num_graphs * b->replicas);
+  std::vector<long long> e2((size_t)b->num_graphs * b->replicas + 1);
   BATCH_CUDA(b, cudaMemcpyAsync(e2.data(), b->d_energy2, e2.size() * sizeof(long long),
                                 cudaMemcpyDeviceToHost, b->stream));
-  const int rc2 = batch_sync(b);
-  if (rc2 != ISING_OK) return rc2;
+  BATCH_CUDA(b, cudaStreamSynchronize(b->stream));
+  if (e2.back() != 0) {
+    b->status = ISING_ETIMEOUT;
+    return ISING_ETIMEOUT;
+  }
   for (int32_t gi = 0; gi < b->num_graphs; ++gi)
     for (int r = 0; r < b->replicas; ++r) {
       const size_t k = (size_t)gi * b->replicas + r;
@@ -1132,7 +1143,7 @@ int ising_batch_set_spins(ising_batch* b, int32_t graph, uint32_t replica, const
   std::vector<uint8_t> bytes((size_t)nn);
   uint8_t* dptr = b->d_spins + b->vtx_base[(size_t)graph];
   BATCH_CUDA(b, cudaMemcpyAsync(bytes.data(), dptr, (size_t)nn, cudaMemcpyDeviceToHost, b->stream));
-  BATCH_CUDA(b, cudaStreamSynchronize(b->stream));
+  if ((rc = batch_sync(b)) != ISING_OK) return rc;
   const std::vector<int32_t>& pos = b->pos[(size_t)graph];
   for (int32_t v = 0; v < nn; ++v) {
     uint8_t& x = bytes[(size_t)pos[(size_t)v]];
@@ -1201,7 +1212,18 @@ int ising_batch_autotune(ising_batch* b, uint32_t probe_sweeps, int32_t* out_blo
   b->split = kSplitChoices[(best / 2) % 3];
   b->tail = kTailChoices[best % 2];
   b->tuned = !clustered;
+  // a probe of the clustered form whose wait ran out has no time worth keeping
+  if ((rc = batch_sync(b)) != ISING_OK) return rc;
   if (out_block) *out_block = b->block;
+  return ISING_OK;
+}
+
+int ising_batch_debug_fault(ising_batch* b, int kind, uint64_t wait_budget_ns) {
+  if (b == nullptr) return ISING_EINVAL;
+  if (kind != ISING_FAULT_NONE && kind != ISING_FAULT_SKIP_ARRIVAL) return ISING_EINVAL;
+  if (wait_budget_ns > 60000000000ull) return ISING_EINVAL;
+  b->fault_kind = kind;
+  b->wait_budget_ns = wait_budget_ns;
   return ISING_OK;
 }
 

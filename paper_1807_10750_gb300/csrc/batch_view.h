@@ -22,6 +22,8 @@ struct BatchUnion {
   const int32_t* vbase = nullptr;    // per position: first position of its instance
   const int32_t* orig = nullptr;     // per position: vertex id within its instance
   uint8_t* spins = nullptr;          // per position: bit r set when replica r's spin is -1
+  const unsigned* error = nullptr;   // not 0: an anneal's wait ran out, and the spins are not its result
+  int* status = nullptr;             // the batch's latched status
   // storage the network fills on first use; freed with the batch
   int32_t** hchunk = nullptr;
   int32_t** chunk_row = nullptr;

@@ -104,6 +104,7 @@ struct GView {
   int shift;
   const int32_t* hchunk;     // per row: first chunk of a heavy row, else -1 (null: no heavy row)
   const int32_t* chunk_row;  // row of every chunk
+  const unsigned* error;     // not 0: the spins are no result (null: never)
   int num_chunks;
 };
 
@@ -148,8 +149,10 @@ __global__ void chunk_sums_kernel(GView v, int4* sums) {
 // lanes sum a light row's entries (integers, so in any order); a heavy row's
 // sums come from chunk_sums_kernel. One pass over the entries without
 // atomics, fused with the features: on 3.5M entries 38 -> 19 us.
+// It also tells the rest of the pass, in *bad, whether the spins are a result.
 template <int L>
-__global__ void features_kernel(GView v, const int4* sums, uint4* x, float* cvec) {
+__global__ void features_kernel(GView v, const int4* sums, uint4* x, float* cvec, int* bad) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *bad = v.error != nullptr && *v.error != 0u;
   const int q = threadIdx.x % L;
   const int subs = (gridDim.x * blockDim.x) / L;
   for (int p0 = (blockIdx.x * blockDim.x + threadIdx.x) / L; p0 - (threadIdx.x / L) % (32 / L) < v.n; p0 += subs) {
@@ -1114,8 +1117,10 @@ __global__ void cast_weights_kernel(const float* p, bf16* w0, bf16* w1, bf16* w2
 
 // Adam (Kingma and Ba) on the fp32 master weights; bc1 = 1 - beta1^t and
 // bc2 = 1 - beta2^t come from the host.
+// A step from spins that are no result leaves everything as it is.
 __global__ void adam_kernel(float* p, float* m, float* v, const float* g, float lr, float b1,
-                            float b2, float bc1, float bc2, float eps) {
+                            float b2, float bc1, float bc2, float eps, const int* bad) {
+  if (*bad != 0) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kNumParams; i += gridDim.x * blockDim.x) {
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.0f - b1) * gi;
@@ -1220,7 +1225,7 @@ struct ising_gnn {
   int64_t chunk_cap = 0;
   float* d_partial = nullptr;  // per heavy-row chunk: its partial sum (width 64)
   int dense_path = ISING_GNN_DENSE_MMA_SYNC;  // forward layers' product
-  int* d_err = nullptr;                      // a tensor-core product that timed out
+  int* d_err = nullptr;                      // a tensor-core product that timed out; the pass's spins are no result
   int tc_blocks[2] = {0, 0};                 // resident tcgen05 layer blocks per SM (D = 8, 64)
 };
 
@@ -1317,6 +1322,7 @@ struct Ctx {
   int sms;
   const int32_t* orig;   // position -> vertex id (within the instance)
   const int32_t* vbase;  // per position: the instance's first position (null: none)
+  int* batch_status;     // the status of the batch (null: a graph)
 };
 
 // Heavy-row chunks of a row table, built once per graph and kept by its owner:
@@ -1376,6 +1382,8 @@ int graph_ctx(ising_gnn* net, ising_graph* g, Ctx* ctx) {
   v.num_chunks = g->gnn_num_chunks;
   v.hchunk = v.num_chunks > 0 ? g->d_gnn_hchunk : nullptr;
   v.chunk_row = g->d_gnn_chunk_row;
+  v.error = nullptr;
+  ctx->batch_status = nullptr;
   ctx->st = g->stream;
   ctx->sms = g->num_sms;
   ctx->orig = g->d_orig;
@@ -1404,6 +1412,8 @@ int batch_ctx(ising_gnn* net, ising_batch* b, uint32_t replica, Ctx* ctx, isingx
   v.num_chunks = *u->num_chunks;
   v.hchunk = v.num_chunks > 0 ? *u->hchunk : nullptr;
   v.chunk_row = *u->chunk_row;
+  v.error = u->error;
+  ctx->batch_status = u->status;
   ctx->st = u->stream;
   ctx->sms = u->num_sms;
   ctx->orig = u->orig;
@@ -1455,12 +1465,18 @@ int run_layer(ising_gnn* net, const Ctx& x, const bf16* h, const bf16* W, const 
   return ISING_OK;
 }
 
-// A tensor-core product that timed out (read after the stream has synchronised).
-int check_err(ising_gnn* net) {
-  int e = 0;
-  GNN_CUDA(net, cudaMemcpy(&e, net->d_err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (e != 0) {
+// A tensor-core product that timed out (latched in the network), or a pass on the
+// spins of an anneal that did (latched in its batch). Read after the stream has
+// synchronised.
+int check_err(ising_gnn* net, const Ctx& x) {
+  int e[2] = {0, 0};
+  GNN_CUDA(net, cudaMemcpy(e, net->d_err, sizeof(e), cudaMemcpyDeviceToHost));
+  if (e[0] != 0) {
     net->status = ISING_ETIMEOUT;
+    return ISING_ETIMEOUT;
+  }
+  if (e[1] != 0) {
+    if (x.batch_status != nullptr) *x.batch_status = ISING_ETIMEOUT;
     return ISING_ETIMEOUT;
   }
   return ISING_OK;
@@ -1488,7 +1504,7 @@ int run_forward(ising_gnn* net, const Ctx& x, bool with_labels) {
   const int lanes = few_rows ? 16 : 4;
   (few_rows ? features_kernel<16> : features_kernel<4>)<<<grid_of(static_cast<long long>(n) * lanes, 128, sms * 16),
                                                          128, 0, st>>>(
-      x.v, net->d_sums, reinterpret_cast<uint4*>(net->d_x), net->d_c);
+      x.v, net->d_sums, reinterpret_cast<uint4*>(net->d_x), net->d_c, net->d_err + 1);
   net->launches++;
   GNN_CUDA(net, cudaGetLastError());
   int rc = run_chunks<kF>(net, x, net->d_x);
@@ -1598,7 +1614,7 @@ int forward_out(ising_gnn* net, const Ctx& x, float* out_logits, int on_device) 
     GNN_CUDA(net, cudaMemcpyAsync(out_logits, net->d_out, sizeof(float) * static_cast<size_t>(x.v.n),
                                   cudaMemcpyDeviceToHost, x.st));
     GNN_CUDA(net, cudaStreamSynchronize(x.st));
-    return check_err(net);
+    return check_err(net, x);
   }
   return ISING_OK;
 }
@@ -1608,7 +1624,7 @@ int read_loss(ising_gnn* net, const Ctx& x, float* out_loss) {
   GNN_CUDA(net, cudaMemcpyAsync(&l, net->d_loss, sizeof(double), cudaMemcpyDeviceToHost, x.st));
   GNN_CUDA(net, cudaStreamSynchronize(x.st));
   *out_loss = static_cast<float>(l / static_cast<double>(x.v.n));
-  return check_err(net);
+  return check_err(net, x);
 }
 
 // The gradient's public tail: copy it and the loss out when asked.
@@ -1616,7 +1632,7 @@ int gradients_out(ising_gnn* net, const Ctx& x, float* out_loss, float* out_grad
   if (out_grad != nullptr) {
     GNN_CUDA(net, cudaMemcpyAsync(out_grad, net->d_grad, sizeof(float) * kNumParams, cudaMemcpyDeviceToHost, x.st));
     GNN_CUDA(net, cudaStreamSynchronize(x.st));
-    const int rc = check_err(net);
+    const int rc = check_err(net, x);
     if (rc != ISING_OK) return rc;
   }
   if (out_loss != nullptr) return read_loss(net, x, out_loss);
@@ -1631,7 +1647,7 @@ int adam_step(ising_gnn* net, const Ctx& x, float lr) {
   const float bc2 = static_cast<float>(1.0 - std::pow(b2, static_cast<double>(net->step)));
   adam_kernel<<<grid_of(kNumParams, 256, 128), 256, 0, x.st>>>(net->d_params, net->d_m, net->d_v, net->d_grad, lr,
                                                                static_cast<float>(b1), static_cast<float>(b2), bc1,
-                                                               bc2, 1e-8f);
+                                                               bc2, 1e-8f, net->d_err + 1);
   cast_weights_kernel<<<32, 256, 0, x.st>>>(net->d_params, net->d_w0, net->d_w1, net->d_w2);
   net->launches += 2;
   GNN_CUDA(net, cudaGetLastError());
@@ -1673,8 +1689,8 @@ int ising_gnn_create(const float* params, ising_gnn** out) {
     if ((e = dalloc(&net->d_w1, 2 * kH * kH)) != cudaSuccess) break;
     if ((e = dalloc(&net->d_w2, 2 * kH * kH)) != cudaSuccess) break;
     if ((e = dalloc(&net->d_loss, 1)) != cudaSuccess) break;
-    if ((e = dalloc(&net->d_err, 1)) != cudaSuccess) break;
-    if ((e = cudaMemset(net->d_err, 0, sizeof(int))) != cudaSuccess) break;
+    if ((e = dalloc(&net->d_err, 2)) != cudaSuccess) break;
+    if ((e = cudaMemset(net->d_err, 0, 2 * sizeof(int))) != cudaSuccess) break;
     if ((e = cudaMemset(net->d_m, 0, sizeof(float) * kNumParams)) != cudaSuccess) break;
     if ((e = cudaMemset(net->d_v, 0, sizeof(float) * kNumParams)) != cudaSuccess) break;
   } while (0);
