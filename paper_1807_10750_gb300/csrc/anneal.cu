@@ -507,10 +507,7 @@ void free_device(ising_graph* g) {
                   g->d_halo_imports, g->d_halo_nbrs, g->d_halo_exports, g->d_halo_quads, g->d_halo_flags,
                   g->d_spins2, g->d_hub_split, g->d_hub_end, g->d_hub_sums, g->d_hub_acc,
                   g->d_hub_flips, g->d_hub_bits, g->d_hub_pflips, g->d_hub_blk,
-                  g->d_gnn_hchunk, g->d_gnn_chunk_row, g->d_map_blocks, g->d_map_task,
-                  g->d_map_words, g->d_map_weights, g->d_map_row_pos, g->d_map_row_orig,
-                  g->d_map_class, g->d_map_steps, g->d_map_msg, g->d_map_index, g->d_map_late, g->d_map_mail,
-                  g->d_pick_count, g->d_picks};
+                  g->d_gnn_hchunk, g->d_gnn_chunk_row, g->d_map};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (g->h_result) cudaFreeHost(g->h_result);
@@ -1060,41 +1057,62 @@ void choose_map_plan(const HostGraph& hg, int num_sms, int device, bool wide, bo
 constexpr size_t kPickInts = size_t(1) << 18;
 constexpr size_t kPickSweeps = size_t(1) << 14;
 
-cudaError_t upload_map_plan(ising_graph* g, const isingx::MapPlan& mp) {
-  cudaError_t e;
-  if ((e = alloc_copy(&g->d_map_blocks, mp.blocks.data(), mp.blocks.size(), g->stream)) != cudaSuccess) return e;
-  if ((e = alloc_copy(&g->d_map_task, mp.tasks.data(), mp.tasks.size(), g->stream)) != cudaSuccess) return e;
-  const size_t entry_bytes = std::max<size_t>(16, static_cast<size_t>(mp.total_groups) * 512);
-  if ((e = cudaMalloc(reinterpret_cast<void**>(&g->d_map_words), entry_bytes)) != cudaSuccess) return e;
-  if (!g->packed && (e = cudaMalloc(reinterpret_cast<void**>(&g->d_map_weights), entry_bytes)) != cudaSuccess) return e;
-  if ((e = alloc_copy(&g->d_map_row_pos, mp.row_pos.data(), mp.row_pos.size(), g->stream)) != cudaSuccess) return e;
-  if ((e = alloc_copy(&g->d_map_row_orig, mp.row_orig.data(), mp.row_orig.size(), g->stream)) != cudaSuccess) return e;
-  const size_t KC = mp.class_row.size(), C1 = mp.class_bytes.size();
-  if ((e = alloc_copy<int32_t>(&g->d_map_class, nullptr, 3 * KC, g->stream)) != cudaSuccess) return e;
-  const std::vector<int32_t>* tables[3] = {&mp.class_row, &mp.class_seg, &mp.block_msg};
-  for (int i = 0; i < 3; ++i)
-    if ((e = cudaMemcpyAsync(g->d_map_class + i * KC, tables[i]->data(), KC * sizeof(int32_t),
-                             cudaMemcpyHostToDevice, g->stream)) != cudaSuccess)
-      return e;
-  if ((e = alloc_copy<int32_t>(&g->d_map_steps, nullptr, 2 * C1, g->stream)) != cudaSuccess) return e;
-  if ((e = cudaMemcpyAsync(g->d_map_steps, mp.class_bytes.data(), C1 * sizeof(int32_t), cudaMemcpyHostToDevice,
-                           g->stream)) != cudaSuccess)
-    return e;
-  if ((e = cudaMemcpyAsync(g->d_map_steps + C1, mp.class_msg.data(), C1 * sizeof(int32_t), cudaMemcpyHostToDevice,
-                           g->stream)) != cudaSuccess)
-    return e;
-  if ((e = alloc_copy(&g->d_map_msg, mp.msg.data(), mp.msg.size(), g->stream)) != cudaSuccess) return e;
-  if ((e = alloc_copy(&g->d_map_index, mp.map_index.data(), mp.map_index.size(), g->stream)) != cudaSuccess) return e;
-  if ((e = alloc_copy<unsigned long long>(&g->d_map_mail, nullptr,
-                                           2 * static_cast<size_t>(mp.K) * static_cast<size_t>(mp.mail_stride), g->stream)) != cudaSuccess)
-    return e;
-  if ((e = alloc_copy(&g->d_map_late, mp.late.data(), mp.late.size(), g->stream)) != cudaSuccess) return e;
-  if (mp.hubs == 0) {
-    g->pick_cap = kPickInts + 8 * static_cast<size_t>(g->n);
-    if ((e = cudaMalloc(reinterpret_cast<void**>(&g->d_pick_count), kPickSweeps * sizeof(uint32_t))) != cudaSuccess) return e;
-    if ((e = cudaMalloc(reinterpret_cast<void**>(&g->d_picks), g->pick_cap * sizeof(int32_t))) != cudaSuccess) return e;
+// The plan on the device: one allocation, its tables in one copy (`staging`
+// holds them until the caller has synchronised the stream). The plan is optional: where there
+// is no room for it the handle goes without.
+cudaError_t upload_map_plan(ising_graph* g, const isingx::MapPlan& mp, std::vector<unsigned char>* staging) {
+  size_t tables = 0, bytes = 0;
+  auto place = [&](size_t size) {
+    const size_t at = bytes;
+    bytes += (std::max<size_t>(size, 16) + 255) & ~size_t(255);
+    return at;
+  };
+  auto size_of = [](const auto& v) { return v.size() * sizeof(v[0]); };
+  const size_t at[] = {place(size_of(mp.blocks)),    place(size_of(mp.tasks)),     place(size_of(mp.row_pos)),
+                       place(size_of(mp.row_orig)),  place(size_of(mp.class_row)), place(size_of(mp.class_seg)),
+                       place(size_of(mp.block_msg)), place(size_of(mp.class_bytes)), place(size_of(mp.class_msg)),
+                       place(size_of(mp.msg)),       place(size_of(mp.map_index)), place(size_of(mp.late))};
+  tables = bytes;
+  const size_t entry_bytes = static_cast<size_t>(mp.total_groups) * 512;
+  const size_t words = place(entry_bytes), weights = g->packed ? 0 : place(entry_bytes);
+  const size_t mail = place(2 * sizeof(unsigned long long) * static_cast<size_t>(mp.K) * static_cast<size_t>(mp.mail_stride));
+  const size_t pick_cap = mp.hubs == 0 ? kPickInts + 8 * static_cast<size_t>(g->n) : 0;
+  const size_t counts = place(mp.hubs == 0 ? kPickSweeps * sizeof(uint32_t) : 0), picks = place(pick_cap * sizeof(int32_t));
+  staging->resize(tables);
+  auto stage = [&](size_t to, const auto& v) {
+    if (!v.empty()) std::memcpy(staging->data() + to, v.data(), size_of(v));
+  };
+  stage(at[0], mp.blocks), stage(at[1], mp.tasks), stage(at[2], mp.row_pos), stage(at[3], mp.row_orig);
+  stage(at[4], mp.class_row), stage(at[5], mp.class_seg), stage(at[6], mp.block_msg), stage(at[7], mp.class_bytes);
+  stage(at[8], mp.class_msg), stage(at[9], mp.msg), stage(at[10], mp.map_index), stage(at[11], mp.late);
+  unsigned char* base = nullptr;
+  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&base), bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    return cudaSuccess;
   }
-  const int2* late = reinterpret_cast<const int2*>(g->d_map_late);
+  if (e != cudaSuccess) return e;
+  g->d_map = base;
+  if ((e = cudaMemcpyAsync(base, staging->data(), tables, cudaMemcpyHostToDevice, g->stream)) != cudaSuccess) return e;
+  auto ints = [&](size_t from) { return reinterpret_cast<int32_t*>(base + from); };
+  g->d_map_blocks = reinterpret_cast<isingx::MapBlock*>(base + at[0]);
+  g->d_map_task = reinterpret_cast<isingx::MapTask*>(base + at[1]);
+  g->d_map_row_pos = ints(at[2]);
+  g->d_map_row_orig = ints(at[3]);
+  g->d_map_class_row = ints(at[4]);
+  g->d_map_class_seg = ints(at[5]);
+  g->d_map_block_msg = ints(at[6]);
+  g->d_map_class_bytes = ints(at[7]);
+  g->d_map_class_msg = ints(at[8]);
+  g->d_map_msg = ints(at[9]);
+  g->d_map_index = ints(at[10]);
+  g->d_map_words = ints(words);
+  g->d_map_weights = g->packed ? nullptr : ints(weights);
+  g->d_map_mail = reinterpret_cast<unsigned long long*>(base + mail);
+  g->d_pick_count = reinterpret_cast<uint32_t*>(base + counts);
+  g->d_picks = ints(picks);
+  g->pick_cap = pick_cap;
+  const int2* late = reinterpret_cast<const int2*>(base + at[11]);
   const dim3 grid(static_cast<unsigned>(mp.K), mp.mode == isingx::kMapGrid ? 4u : 32u);
   if (g->packed)
     isingx::map_fill_kernel<true><<<grid, 256, 0, g->stream>>>(
@@ -1131,7 +1149,6 @@ cudaError_t launch_map(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint64
   if (g->map_mode == isingx::kMapCluster &&
       (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
     return e;
-  const size_t KC = static_cast<size_t>(g->map_K) * (static_cast<size_t>(g->num_colours) + 1);
   isingx::MapArgs a{};
   a.blocks = g->d_map_blocks;
   a.tasks = reinterpret_cast<const int4*>(g->d_map_task);
@@ -1139,11 +1156,11 @@ cudaError_t launch_map(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint64
   a.weights = reinterpret_cast<const int4*>(g->d_map_weights);
   a.row_pos = g->d_map_row_pos;
   a.row_orig = g->d_map_row_orig;
-  a.class_row = g->d_map_class;
-  a.class_seg = g->d_map_class + KC;
-  a.block_msg = g->d_map_class + 2 * KC;
-  a.class_bytes = g->d_map_steps;
-  a.class_msg = g->d_map_steps + g->num_colours + 1;
+  a.class_row = g->d_map_class_row;
+  a.class_seg = g->d_map_class_seg;
+  a.block_msg = g->d_map_block_msg;
+  a.class_bytes = g->d_map_class_bytes;
+  a.class_msg = g->d_map_class_msg;
   a.msg = g->d_map_msg;
   a.map_index = g->d_map_index;
   a.mail = g->d_map_mail;
@@ -1381,6 +1398,7 @@ int ising_create(int32_t n, int64_t m, const int32_t* src, const int32_t* dst, c
   }
   isingx::BlockPlan block;
   isingx::MapPlan map_plan;
+  std::vector<unsigned char> map_staging;
   std::vector<int32_t> dep_ptr, deps;  // item dependencies (before the columns are packed)
   bool have_deps = false;
   std::vector<int32_t> packed_words;  // graphs kept for the halo plan pack into a copy
@@ -1392,7 +1410,11 @@ int ising_create(int32_t n, int64_t m, const int32_t* src, const int32_t* dst, c
                 hg.max_degree <= isingx::kHaloMaxWidth && hg.n >= 64 * g->num_sms;
     // the spin-map engine; graphs with hubs keep the engines that AUTO does not pick
     const bool split = !block.ok && !hub_end.empty();
-    choose_map_plan(hg, g->num_sms, g->device, !g->packed, keep_host, split, &map_plan);
+    try {
+      choose_map_plan(hg, g->num_sms, g->device, !g->packed, keep_host, split, &map_plan);
+    } catch (const std::bad_alloc&) {
+      map_plan.ok = false;  // the plan is optional
+    }
     if (!map_plan.ok || split) have_deps = isingx::build_item_deps(hg, plan, &dep_ptr, &deps);
   } catch (const std::bad_alloc&) {
     delete g;
@@ -1479,7 +1501,11 @@ int ising_create(int32_t n, int64_t m, const int32_t* src, const int32_t* dst, c
       g->block_ok = true;
       g->block_num_chunks = static_cast<int32_t>(block.chunk_off.size());
     }
-    if (map_plan.ok && (e = upload_map_plan(g, map_plan)) != cudaSuccess) break;
+    if (map_plan.ok) try {
+        if ((e = upload_map_plan(g, map_plan, &map_staging)) != cudaSuccess) break;
+      } catch (const std::bad_alloc&) {
+        // no room to stage the tables: no plan
+      }
     if (!hub_end.empty()) {
       const size_t X = hub_end.size();
       if ((e = alloc_copy(&g->d_hub_split, hub_split.data(), X, g->stream)) != cudaSuccess) break;

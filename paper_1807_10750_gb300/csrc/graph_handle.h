@@ -114,17 +114,14 @@ struct ising_graph {
   bool map_ok = false, map_resident = false;
   int map_mode = 0, map_K = 0, map_warps = 0, map_smem = 0;
   int32_t map_bytes = 0, map_tasks = 0, map_rows = 0, map_groups = 0, map_stage = 0, map_stride = 0, map_accs = 0;
+  void* d_map = nullptr;               // one allocation, which holds all of the following
   isingx::MapBlock* d_map_blocks = nullptr;
   isingx::MapTask* d_map_task = nullptr;
-  int32_t* d_map_words = nullptr;
-  int32_t* d_map_weights = nullptr;
-  int32_t* d_map_row_pos = nullptr;
-  int32_t* d_map_row_orig = nullptr;
-  int32_t* d_map_class = nullptr;      // class_row, class_seg, block_msg: K x (C + 1) each
-  int32_t* d_map_steps = nullptr;      // class_bytes, class_msg: C + 1 each
-  int32_t* d_map_msg = nullptr;
-  int32_t* d_map_index = nullptr;      // position -> map index
-  int32_t* d_map_late = nullptr;       // per split row: its entries in the class before
+  int32_t *d_map_words = nullptr, *d_map_weights = nullptr;
+  int32_t *d_map_row_pos = nullptr, *d_map_row_orig = nullptr;
+  int32_t *d_map_class_row = nullptr, *d_map_class_seg = nullptr, *d_map_block_msg = nullptr;  // K x (C + 1)
+  int32_t *d_map_class_bytes = nullptr, *d_map_class_msg = nullptr;                            // C + 1
+  int32_t *d_map_msg = nullptr, *d_map_index = nullptr;  // (position -> map index)
   unsigned long long* d_map_mail = nullptr;
   uint32_t* d_pick_count = nullptr;    // Algorithm 1's picks of a launch: how many after each sweep
   int32_t* d_picks = nullptr;
