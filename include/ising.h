@@ -412,6 +412,10 @@ int ising_batch_tuning(ising_batch* b, int32_t* out_block, int32_t* out_row_spli
  * train step on such spins leaves the weights as they are). The one-block
  * kernel has no waits. */
 int ising_batch_debug_fault(ising_batch* b, int kind, uint64_t wait_budget_ns);
+/* ising_batch_debug_form -- a diagnostic, as ising_debug_form: how many instances
+ * the last anneal ran on the one-block kernel (out_instances[0], -1 before the
+ * first anneal) and in the clustered form on 1, 2, 4, 8 and 16 blocks (entries 1 to 5). */
+int ising_batch_debug_form(ising_batch* b, int32_t* out_instances);
 /* ising_batch_info -- instances, total vertices, block size, kernel launches. */
 int ising_batch_info(ising_batch* b, int32_t* out_num_graphs, int64_t* out_vertices,
                      int32_t* out_block, uint64_t* out_launches);
@@ -573,6 +577,19 @@ void ising_gnn_destroy(ising_gnn* net);
  * (PERSISTENT's one-block form); -1 before the first anneal. */
 #define ISING_ENGINE_USED_BLOCK 6
 int ising_engine_used(ising_graph* g, int32_t* out);
+
+/* ising_debug_form -- a diagnostic of tests and benchmarks: the kernel that the last anneal call's last
+ * launch ran, which ising_engine_used does not tell (the spin-map forms stand
+ * in for several engines), and the blocks that share the graph (0 for
+ * ISING_FORM_ENGINE). -1 before the first anneal. Any pointer may be NULL. */
+enum {
+  ISING_FORM_ENGINE = 0,           /* the engine's own kernel */
+  ISING_FORM_MAP_BLOCK = 1,        /* spin map: one block, entries in shared memory */
+  ISING_FORM_MAP_BLOCK_STREAM = 2, /* one block, entries read from L2 */
+  ISING_FORM_MAP_CLUSTER = 3,      /* the blocks of one cluster */
+  ISING_FORM_MAP_GRID = 4          /* one block per SM */
+};
+int ising_debug_form(ising_graph* g, int32_t* out_form, int32_t* out_blocks);
 
 /* Failure-detection test hook. Every device-side wait of the anneal kernels
  * is bounded (2 s by default); a wait that runs out records an error, the

@@ -40,6 +40,11 @@ ISING_ENGINE_PERSISTENT_GRID = 4
 ISING_ENGINE_ITEMFLOW = 5
 ISING_ENGINE_HALO = 7
 ISING_ENGINE_HUB = 8
+ISING_FORM_ENGINE = 0
+ISING_FORM_MAP_BLOCK = 1
+ISING_FORM_MAP_BLOCK_STREAM = 2
+ISING_FORM_MAP_CLUSTER = 3
+ISING_FORM_MAP_GRID = 4
 ISING_CREATE_WEIGHTS_I32 = 1
 ISING_STATIC_MAX_VERTICES = 1 << 24
 
@@ -59,6 +64,7 @@ EXPORTS = (
     "ising_convergence_region", "ising_batch_set_tuning", "ising_batch_tuning",
     "ising_gnn_batch_forward", "ising_gnn_batch_warm_start", "ising_gnn_batch_gradients",
     "ising_gnn_batch_train_step", "ising_gnn_set_dense_path", "ising_batch_debug_fault",
+    "ising_debug_form", "ising_batch_debug_form",
 )
 ISING_ENGINE_USED_BLOCK = 6
 ISING_FAULT_NONE = 0
@@ -155,6 +161,8 @@ def lib():
         L.ising_gnn_destroy.restype = None
         L.ising_debug_fault.argtypes = [vp, ctypes.c_int, ctypes.c_uint64]
         L.ising_batch_debug_fault.argtypes = [vp, ctypes.c_int, ctypes.c_uint64]
+        L.ising_debug_form.argtypes = [vp, i32p, i32p]
+        L.ising_batch_debug_form.argtypes = [vp, vp]
         L.ising_engine_used.argtypes = [vp, ctypes.POINTER(ctypes.c_int32)]
         L.ising_set_halo_sweeps.argtypes = [vp, ctypes.c_uint32]
         L.ising_plan_halo.argtypes = [ctypes.c_int32, ctypes.c_int64, vp, vp, vp, ctypes.c_int32,
@@ -370,6 +378,13 @@ def ising_engine_used(g: IsingGraph) -> int:
     return v.value
 
 
+def ising_debug_form(g: IsingGraph) -> tuple[int, int]:
+    """The kernel form (ISING_FORM_*) and blocks of the last anneal (see include/ising.h)."""
+    form, blocks = ctypes.c_int32(), ctypes.c_int32()
+    _check(lib().ising_debug_form(g.ptr, ctypes.byref(form), ctypes.byref(blocks)), "ising_debug_form")
+    return form.value, blocks.value
+
+
 def ising_debug_fault(g: IsingGraph, kind: int, wait_budget_ns: int = 0) -> None:
     """Failure-detection test hook (see include/ising.h)."""
     _check(lib().ising_debug_fault(g.ptr, kind, wait_budget_ns), "ising_debug_fault")
@@ -558,6 +573,13 @@ def ising_batch_tuning(b: IsingBatch) -> dict:
 def ising_batch_debug_fault(b: IsingBatch, kind: int, wait_budget_ns: int = 0) -> None:
     """Failure-detection test hook (see include/ising.h)."""
     _check(lib().ising_batch_debug_fault(b.ptr, kind, wait_budget_ns), "ising_batch_debug_fault")
+
+
+def ising_batch_debug_form(b: IsingBatch) -> list[int]:
+    """Instances of the last anneal on the one-block kernel, and on 1, 2, 4, 8, 16 blocks."""
+    out = np.zeros(6, dtype=np.int32)
+    _check(lib().ising_batch_debug_form(b.ptr, out.ctypes.data), "ising_batch_debug_form")
+    return out.tolist()
 
 
 def ising_batch_info(b: IsingBatch) -> dict:

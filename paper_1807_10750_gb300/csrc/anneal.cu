@@ -1209,6 +1209,8 @@ cudaError_t launch_map(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint64
     g->launches++;
     if ((e = cudaLaunchKernelExC(&cfg, kernel, args)) != cudaSuccess) return e;
   }
+  g->form_used = ISING_FORM_MAP_BLOCK + g->map_mode;
+  g->form_blocks = g->map_K;
   return cudaSuccess;
 }
 
@@ -1317,6 +1319,11 @@ int compute_energy(ising_graph* g, int64_t* out) {
 }  // namespace
 
 extern "C" {
+
+static_assert(ISING_FORM_MAP_BLOCK + isingx::kMapBlockStream == ISING_FORM_MAP_BLOCK_STREAM &&
+                  ISING_FORM_MAP_BLOCK + isingx::kMapCluster == ISING_FORM_MAP_CLUSTER &&
+                  ISING_FORM_MAP_BLOCK + isingx::kMapGrid == ISING_FORM_MAP_GRID,
+              "ising_debug_form reports MapMode");
 
 const char* ising_strerror(int status) {
   switch (status) {
@@ -1664,6 +1671,8 @@ static int anneal_impl(ising_graph* g, const ising_schedule* sched, uint32_t swe
                        int mode) {
   if (sweeps == 0) return ISING_OK;
   const isingx::PhiloxRounds rk = isingx::philox_rounds(isingx::philox_key(seed, 0u));
+  g->form_used = ISING_FORM_ENGINE;
+  g->form_blocks = 0;
   // AUTO: the persistent engine when the device supports cooperative launches.
   int engine = g->engine;
   const bool unsliced = g->num_slots == 0;
@@ -1953,6 +1962,13 @@ int ising_launch_count(ising_graph* g, uint64_t* out) {
 int ising_engine_used(ising_graph* g, int32_t* out) {
   if (g == nullptr || out == nullptr) return ISING_EINVAL;
   *out = g->engine_used;
+  return ISING_OK;
+}
+
+int ising_debug_form(ising_graph* g, int32_t* out_form, int32_t* out_blocks) {
+  if (g == nullptr) return ISING_EINVAL;
+  if (out_form) *out_form = g->form_used;
+  if (out_blocks) *out_blocks = g->form_blocks;
   return ISING_OK;
 }
 

@@ -494,6 +494,7 @@ struct ising_batch {
   cudaEvent_t fork = nullptr;
   int fault_kind = ISING_FAULT_NONE;  // ising_batch_debug_fault
   uint64_t wait_budget_ns = 0;
+  int32_t form[6] = {-1, 0, 0, 0, 0, 0};  // ising_batch_debug_form
   int8_t* d_out = nullptr;  // ising_batch_get_spins: max_n + 1 bytes, and their pinned copy
   int8_t* h_out = nullptr;
   // the instances as one graph, for the warm-start network (batch_union)
@@ -786,6 +787,8 @@ int groups_launch(ising_batch* b, uint64_t t_begin, uint32_t sweeps, uint64_t T,
     void* args[] = {&a, &t_begin, &sweeps, &T, &T0, &seed_lo, &seed_hi};
     b->launches++;
     BATCH_CUDA(b, cudaLaunchKernelExC(&cfg, kernel, args));
+    for (int k = 0; k < 5; ++k)
+      if (g.K == 1 << k) b->form[1 + k] += g.count;
     if (i > 0) {
       BATCH_CUDA(b, cudaEventRecord(g.join, s));
       BATCH_CUDA(b, cudaStreamWaitEvent(b->stream, g.join, 0));
@@ -799,7 +802,9 @@ int groups_launch(ising_batch* b, uint64_t t_begin, uint32_t sweeps, uint64_t T,
 // size and replayed with this call's parameters.
 int batch_launch(ising_batch* b, uint64_t t_begin, uint32_t sweeps, uint64_t T, uint64_t T0,
                  uint64_t seed) {
+  std::fill(b->form, b->form + 6, 0);
   if (!b->groups.empty() && !b->tuned) return groups_launch(b, t_begin, sweeps, T, T0, seed);
+  b->form[0] = b->num_graphs;
   const size_t smem = static_cast<size_t>(std::max(b->max_n, 1));
   const void* kernel = batch_kernel_for(b->block, b->split);
   BATCH_CUDA(b, isingx::allow_shared(kernel, b->device, smem));
@@ -1224,6 +1229,12 @@ int ising_batch_debug_fault(ising_batch* b, int kind, uint64_t wait_budget_ns) {
   if (wait_budget_ns > 60000000000ull) return ISING_EINVAL;
   b->fault_kind = kind;
   b->wait_budget_ns = wait_budget_ns;
+  return ISING_OK;
+}
+
+int ising_batch_debug_form(ising_batch* b, int32_t* out_instances) {
+  if (b == nullptr || out_instances == nullptr) return ISING_EINVAL;
+  std::copy(b->form, b->form + 6, out_instances);
   return ISING_OK;
 }
 

@@ -110,6 +110,7 @@ struct ising_graph {
   uint32_t* d_hub_pflips = nullptr;  // a sweep's flips by position (n / 32 + 2 words)
   int32_t* d_hub_blk = nullptr;      // non-hub classes' work split over the worker blocks
   int32_t hub_grid = 0;              // blocks the split was made for
+  int form_used = -1, form_blocks = 0;  // ising_debug_form
   // spin-map engine (map.cuh)
   bool map_ok = false, map_resident = false;
   int map_mode = 0, map_K = 0, map_warps = 0, map_smem = 0;
