@@ -118,7 +118,7 @@ enum {
                                   every spin in shared memory. What AUTO runs as PERSISTENT takes
                                   that spin-map form too (on every SM where a class has enough
                                   work) for deterministic anneals of graphs of up to 204,800
-                                  vertices and 4096 neighbours a vertex */
+                                  vertices and 4096 neighbours a vertex, where it is faster */
   ISING_ENGINE_DATAFLOW = 3,   /* one cooperative launch per anneal call without barriers: each
                                   neighbour read waits (bounded) until the neighbour carries the
                                   update the colour order requires; racy mode runs as PERSISTENT */
@@ -129,8 +129,10 @@ enum {
                                   (per-item counters, release/acquire); for graphs whose rows
                                   are not sliced across warps, deterministic linear schedule;
                                   otherwise runs as PERSISTENT_GRID. Such graphs of up to 204,800
-                                  vertices run in the spin-map form instead (a lattice larger
-                                  than 100,000 vertices does not) */
+                                  vertices run in the spin-map form instead where it is faster (not lattices
+                                  larger than 100,000 vertices or 37,500 a colour, nor graphs
+                                  above about 165,000 vertices of fewer than 4.5 neighbours; a call of
+                                  one sweep may run as PERSISTENT_GRID) */
   ISING_ENGINE_HALO = 7,       /* one cooperative launch per anneal call, one block per SM: the
                                   graph is cut into one part per block (recursive breadth-first
                                   bisection); a block keeps every vertex within D = S * K hops of

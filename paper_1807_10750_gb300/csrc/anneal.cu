@@ -1022,32 +1022,41 @@ bool map_fits(const isingx::MapPlan& mp, bool wide, int device) {
   return fits;
 }
 
-// The plan a graph gets, by the work of a class: its entries, and eight for
-// each of its rows (decision, draw, publication). Up to 4,000 one block is
-// fastest: no exchange (a 1000-vertex, 10,000-edge graph takes 4.1 us a sweep
-// on one block and 5.6 on the cluster; 2000 vertices and 20,000 edges, 5,600
-// a class, 5.8 and 5.0). Up to 300,000 a class the 16 blocks of a cluster, whose
-// exchange costs 0.3 us (70,000 vertices and 2.1M edges, 227,000 a class: 39 us
-// against 42 on the grid); beyond that, every SM and its 1.3 us exchange
-// (100,000 vertices and 5M edges, 360,000 a class: 84 against 62 us). Lattices
-// wait for a halo plan: until then the cluster up to 100,000 vertices (9.8
-// against 11.6 us by item dataflow at 90,300, 14.3 against 13.3 at 160,000).
+// The plan a graph gets. Work of a class: its entries, and eight for each of its
+// rows (decision, draw, publication). Up to 4,000 of it one block is fastest: no
+// exchange (a 1000-vertex, 10,000-edge graph takes 4.1 us a sweep on one block
+// and 5.6 on the cluster; 2000 vertices and 20,000 edges, 5,600 a class, 5.8 and
+// 5.0). Up to 270,000 entries a class the 16 blocks of a cluster, whose exchange
+// costs 0.3 us; beyond that, every SM and its 1.45 us exchange. The rows count
+// alike in both (70,000 vertices and 2.1M edges, 210,000 a class: 39 us on the
+// cluster, 42 on the grid; 130,000 of 4 neighbours: 14.5 and 19.1; 150,000 of 20,
+// 273,000: 32.9 and 34.7; 100,000 and 5M edges, 333,000: 84 and 62).
+// Where the cluster has no room for the spins, the grid needs entries to be
+// worth its exchange and its messages: 200,000 vertices of 4 neighbours 22.7 us by
+// item dataflow and 25.0 on the grid, of 6 neighbours 37.9 and 27.0. It needs classes
+// worth an exchange, too: a near-clique of 800 vertices in as many classes takes
+// 611 us by the block engine and 1163 on the grid. Lattices wait for a halo plan:
+// until then the cluster up to 100,000 vertices (four classes: 90,601 vertices
+// 13.2 us by item dataflow and 9.4).
 // Graphs with hubs (split) go to the cluster wherever their spins fit, up to
 // about 115,000 vertices (110,000: 65 us a sweep against 95 by the hub engine).
 void choose_map_plan(const HostGraph& hg, int num_sms, int device, bool wide, bool lattice, bool split,
                      isingx::MapPlan* mp) {
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
-  const int64_t work = hg.nnz + 8 * static_cast<int64_t>(hg.n), classes = std::max(1, hg.num_colours);
+  const int64_t n = hg.n, work = hg.nnz + 8 * n, classes = std::max(1, hg.num_colours);
   auto build = [&](int mode, int K) {
     isingx::build_map_plan(hg, mode, K, wide, optin, mp, split);
     return mp->ok && map_fits(*mp, wide, device);
   };
-  if (!split && work <= 4000 * classes && (build(isingx::kMapBlock, 1) || build(isingx::kMapBlockStream, 1))) return;
-  if ((lattice ? hg.n <= 100000 : work <= 300000 * classes) &&
+  const bool small_classes = work <= 4000 * classes;
+  if (!split && small_classes && (build(isingx::kMapBlock, 1) || build(isingx::kMapBlockStream, 1))) return;
+  if ((lattice ? n <= 100000 : hg.nnz <= 270000 * classes) &&
       (build(isingx::kMapCluster, 16) || build(isingx::kMapCluster, 8)))
     return;
-  if (!split && !lattice && build(isingx::kMapGrid, std::min(num_sms, std::max(1, hg.n / 32)))) return;
+  if (!split && !lattice && !small_classes && 2 * hg.nnz > 9 * n &&
+      build(isingx::kMapGrid, std::min(num_sms, std::max(1, hg.n / 32))))
+    return;
   mp->ok = false;
 }
 
@@ -1422,7 +1431,11 @@ int ising_create(int32_t n, int64_t m, const int32_t* src, const int32_t* dst, c
     } catch (const std::bad_alloc&) {
       map_plan.ok = false;  // the plan is optional
     }
-    if (!map_plan.ok || split) have_deps = isingx::build_item_deps(hg, plan, &dep_ptr, &deps);
+    // A lattice of two large classes anneals by item dataflow all the same, in
+    // linear schedules (70,200 vertices 7.3 us a sweep and 6.7 on the cluster, 90,000
+    // 7.3 and 8.7; Algorithm 1, by the grid barrier's kernel, 11.4 and 8.2).
+    const bool items_first = keep_host && hg.n > 37500 * static_cast<int64_t>(hg.num_colours);
+    if (!map_plan.ok || split || items_first) have_deps = isingx::build_item_deps(hg, plan, &dep_ptr, &deps);
   } catch (const std::bad_alloc&) {
     delete g;
     return ISING_ENOMEM;
@@ -1740,11 +1753,17 @@ static int anneal_impl(ising_graph* g, const ising_schedule* sched, uint32_t swe
     engine = ISING_ENGINE_ITEMFLOW;  // racy, N-flip or no plan
   }
   // the spin-map form of the block engine, of the item-dataflow engine and of
-  // what AUTO runs as PERSISTENT
+  // what AUTO runs as PERSISTENT. One sweep of many short rows does not pay for
+  // filling the maps: the grid barrier's kernel takes 15 us and 4 for each of the few
+  // classes (50,000 vertices in two classes 25 us, 90,601 in four 31, 90,000 in seven 41,
+  // 130,000 in eight 55), the cluster 28, 38, 41 and 58.
+  const bool one_sweep = sweeps == 1 && g->n >= 13000 * static_cast<int64_t>(g->num_colours) &&
+                         g->nnz <= 12 * static_cast<int64_t>(g->n);
   const bool use_map = g->map_ok && g->map_accs == 0 && mode == ISING_MODE_DET && g->fault_kind != ISING_FAULT_SHORT_COPY &&
+                       !one_sweep &&
                        (engine == ISING_ENGINE_ITEMFLOW ||
                         (engine == ISING_ENGINE_PERSISTENT && (g->block_ok || g->engine == ISING_ENGINE_AUTO)));
-  if (use_map && !(engine == ISING_ENGINE_ITEMFLOW && (nflip || !unsliced))) {
+  if (use_map && !(engine == ISING_ENGINE_ITEMFLOW && (nflip || !unsliced || g->itemflow_ok))) {
     g->engine_used = engine == ISING_ENGINE_ITEMFLOW ? ISING_ENGINE_ITEMFLOW
                      : g->block_ok                   ? ISING_ENGINE_USED_BLOCK
                                                      : ISING_ENGINE_PERSISTENT_GRID;
