@@ -430,6 +430,7 @@ uint64_t batch_t0(double p0) {
 }
 
 constexpr int kBlockChoices[3] = {128, 256, 512};
+constexpr int kBlockDefault = 256;
 constexpr int kSplitChoices[3] = {1, 2, 4};
 constexpr int kTailChoices[2] = {0, 32};
 constexpr int kBatchError = 15;  // d_work: work queue heads, then the clustered form's error flag
@@ -439,10 +440,13 @@ constexpr int kTuneConfigs = 18;  // block x split x tail
 }  // namespace
 
 // Instances of the clustered form that share a cluster size; all but the
-// first group run on streams of their own beside the first.
+// first group run on streams of their own beside the first. The group of single
+// blocks may run on the one-block kernel instead.
 struct BatchMapGroup {
   int K = 1, clusters = 1, smem = 0, count = 0;
-  bool unit = false;
+  bool unit = false, one_block = false;
+  int32_t max_n = 0;         // one_block: the largest instance,
+  int32_t* order = nullptr;  // and the instances by decreasing size
   int32_t map_bytes = 0, units_max = 0, classes_max = 0;
   cudaStream_t stream = nullptr;
   cudaEvent_t join = nullptr;
@@ -461,7 +465,7 @@ struct ising_batch {
   int32_t num_graphs = 0;
   int replicas = 1;
   int32_t max_n = 0;
-  int block = 256;  // chosen by ising_batch_autotune (with split and tail below)
+  int block = kBlockDefault;  // chosen by ising_batch_autotune (with split and tail below)
   uint64_t launches = 0;
   std::vector<int32_t> n;                  // per instance
   std::vector<int64_t> total_weight;       // per instance
@@ -524,7 +528,7 @@ namespace {
 void group_free(BatchMapGroup& g) {
   if (g.stream) cudaStreamDestroy(g.stream);
   if (g.join) cudaEventDestroy(g.join);
-  void* ptrs[] = {g.inst, g.units, g.block_unit, g.class_unit, g.class_bytes, g.dst, g.row_sum, g.map_index, g.words};
+  void* ptrs[] = {g.inst, g.units, g.block_unit, g.class_unit, g.class_bytes, g.dst, g.row_sum, g.map_index, g.words, g.order};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   g = BatchMapGroup();
@@ -603,12 +607,12 @@ const void* batch_kernel_for(int block, int split) {
 
 // Blocks of the persistent batch kernel: every co-resident block (shared
 // memory holds the largest instance's spins).
-int batch_grid(ising_batch* b, int block, int split, size_t smem) {
+int batch_grid(ising_batch* b, int block, int split, size_t smem, int count) {
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel_for(block, split), block, smem);
   cudaGetLastError();
   if (per_sm < 1) per_sm = 1;
-  return std::min(per_sm * b->num_sms, std::max(1, b->num_graphs));
+  return std::min(per_sm * b->num_sms, std::max(1, count));
 }
 
 // ---------------------------------------------------------------------------
@@ -671,8 +675,6 @@ cudaError_t group_upload(ising_batch* b, const isingx::BatchMapPlan& p, const in
   cudaError_t e;
   int32_t* d_unit_inst = nullptr;
   do {
-    if ((e = cudaStreamCreateWithFlags(&g->stream, cudaStreamNonBlocking)) != cudaSuccess) break;
-    if ((e = cudaEventCreateWithFlags(&g->join, cudaEventDisableTiming)) != cudaSuccess) break;
     if ((e = upload(&g->inst, p.inst, b->stream)) != cudaSuccess) break;
     if ((e = upload(&g->units, p.units, b->stream)) != cudaSuccess) break;
     if ((e = upload(&g->block_unit, p.block_unit, b->stream)) != cudaSuccess) break;
@@ -693,6 +695,23 @@ cudaError_t group_upload(ising_batch* b, const isingx::BatchMapPlan& p, const in
   } while (false);
   cudaFree(d_unit_inst);
   return e;
+}
+
+// Whether the instances of one block each are better off on the one-block kernel,
+// which holds eight instances an SM where the clustered form holds two.
+// Microseconds for 100 sweeps of n vertices (mean degree 10, +-1 weights, eight
+// replicas), one-block kernel and clustered form as ratios: 300 instances of 250
+// vertices 1.5, 450 0.84, 1000 0.86, 4000 0.67; of 1000 vertices 1.3, 1.05, 1.04
+// (at fewer replicas or with wider weights 0.93, and 1.0 at 2000 vertices). A class of
+// few rows is padded to a unit of 32: where two instances an SM are more than its
+// first-level cache holds, that costs more than the packed planes give (complete
+// graphs of 60 vertices, 460 KB each: 150 of them 1.0, 300 0.51; of 40, 205 KB: 150
+// 1.4, 300 0.92; of 20, 51 KB: 300 1.5).
+bool prefers_one_block(const isingx::BatchMapPlan& p, int64_t vertices, int64_t entries, int replicas, int num_sms) {
+  const int64_t count = static_cast<int64_t>(p.inst.size());
+  const int64_t small = p.unit && replicas > 4 ? 900 : 1500;
+  if (count > 2 * num_sms && vertices < small * count) return true;
+  return count > num_sms && p.groups * 512 > 128 * 1024 * count && p.groups * 128 > 4 * entries;
 }
 
 // The groups of the clustered form, largest cluster first. Without room for
@@ -716,9 +735,33 @@ cudaError_t groups_build(ising_batch* b, const std::vector<isingx::BatchMapRows>
     left = rest;
     if (mine.empty()) continue;
     isingx::BatchMapPlan plan;
-    b->groups.emplace_back();
     fits = isingx::build_batch_map(mine, unit, wmax, K, optin, &plan);
-    if (fits) e = group_upload(b, plan, d_row_base, &b->groups.back(), &fits);
+    if (!fits) break;
+    int64_t vertices = 0, entries = 0;
+    std::vector<int32_t> ids;
+    for (const isingx::BatchMapRows* r : mine) {
+      vertices += static_cast<int64_t>(r->degree.size());
+      entries += std::accumulate(r->degree.begin(), r->degree.end(), int64_t(0));
+      ids.push_back(r->id);
+    }
+    const bool one_block = K == 1 && prefers_one_block(plan, vertices, entries, b->replicas, b->num_sms);
+    if (one_block && b->groups.empty()) break;  // the whole batch
+    b->groups.emplace_back();
+    BatchMapGroup& g = b->groups.back();
+    if (b->groups.size() > 1) {
+      e = cudaStreamCreateWithFlags(&g.stream, cudaStreamNonBlocking);
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g.join, cudaEventDisableTiming);
+      if (e != cudaSuccess) break;
+    }
+    if (one_block) {
+      g.one_block = true;
+      g.count = static_cast<int>(mine.size());
+      for (const isingx::BatchMapRows* r : mine) g.max_n = std::max(g.max_n, static_cast<int32_t>(r->degree.size()));
+      e = upload(&g.order, ids, b->stream);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    } else {
+      e = group_upload(b, plan, d_row_base, &g, &fits);
+    }
   }
   cudaFree(d_row_base);
   if (e == cudaSuccess && fits) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
@@ -748,12 +791,34 @@ int batch_sync(ising_batch* b) {
 }
 
 // One launch per group: the first on the batch's stream, the others beside it
-// on their own, forked from and joined to it.
+// on their own, forked from and joined to it. (The one-block kernel's group is
+// never the first.)
 int groups_launch(ising_batch* b, uint64_t t_begin, uint32_t sweeps, uint64_t T, uint64_t T0, uint64_t seed) {
   BATCH_CUDA(b, cudaMemsetAsync(b->d_work, 0, sizeof(unsigned) * b->groups.size(), b->stream));
   if (b->groups.size() > 1) BATCH_CUDA(b, cudaEventRecord(b->fork, b->stream));
   for (size_t i = 0; i < b->groups.size(); ++i) {
     BatchMapGroup& g = b->groups[i];
+    const cudaStream_t s = i == 0 ? b->stream : g.stream;
+    uint32_t seed_lo = static_cast<uint32_t>(seed), seed_hi = static_cast<uint32_t>(seed >> 32);
+    if (i > 0) BATCH_CUDA(b, cudaStreamWaitEvent(s, b->fork, 0));
+    if (g.one_block) {
+      const size_t smem = static_cast<size_t>(std::max(g.max_n, 1));
+      const void* kernel = batch_kernel_for(kBlockDefault, 1);
+      BATCH_CUDA(b, isingx::allow_shared(kernel, b->device, smem));
+      BatchDev d = b->dev();
+      d.order = g.order;
+      unsigned* work = b->d_work + i;
+      int tail = 0;
+      void* args[] = {&d,       &g.count,     &work, &t_begin, &sweeps, &T, &T0, &seed_lo,
+                      &seed_hi, &b->replicas, &tail};
+      b->launches++;
+      BATCH_CUDA(b, cudaLaunchKernel(kernel, dim3(static_cast<unsigned>(batch_grid(b, kBlockDefault, 1, smem, g.count))),
+                                     dim3(kBlockDefault), args, smem, s));
+      b->form[0] += g.count;
+      BATCH_CUDA(b, cudaEventRecord(g.join, s));
+      BATCH_CUDA(b, cudaStreamWaitEvent(b->stream, g.join, 0));
+      continue;
+    }
     const void* kernel = batch_map_kernel_for(g.K > 1, g.unit);
     BATCH_CUDA(b, isingx::allow_shared(kernel, b->device, static_cast<size_t>(g.smem)));
     if (g.K > 1) BATCH_CUDA(b, cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
@@ -778,9 +843,6 @@ int groups_launch(ising_batch* b, uint64_t t_begin, uint32_t sweeps, uint64_t T,
     a.classes_max = g.classes_max;
     a.budget = b->wait_budget_ns > 0 ? static_cast<long long>(b->wait_budget_ns) : isingx::kBarrierBudgetNs;
     a.silent = b->fault_kind == ISING_FAULT_SKIP_ARRIVAL ? 1 : 0;
-    uint32_t seed_lo = static_cast<uint32_t>(seed), seed_hi = static_cast<uint32_t>(seed >> 32);
-    const cudaStream_t s = i == 0 ? b->stream : g.stream;
-    if (i > 0) BATCH_CUDA(b, cudaStreamWaitEvent(s, b->fork, 0));
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
     batch_map_config(&cfg, &attr, g.K, g.clusters, g.smem, s);
@@ -808,7 +870,7 @@ int batch_launch(ising_batch* b, uint64_t t_begin, uint32_t sweeps, uint64_t T, 
   const size_t smem = static_cast<size_t>(std::max(b->max_n, 1));
   const void* kernel = batch_kernel_for(b->block, b->split);
   BATCH_CUDA(b, isingx::allow_shared(kernel, b->device, smem));
-  const int grid = batch_grid(b, b->block, b->split, smem);
+  const int grid = batch_grid(b, b->block, b->split, smem, b->num_graphs);
   BatchDev d = b->dev();
   int num_graphs = b->num_graphs;
   unsigned* work = b->d_work;
