@@ -23,7 +23,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["anneal.cu", "host_graph.cpp", "halo_plan.cpp", "map_plan.cpp", "batch_map_plan.cpp", "energy_static.cu", "batch.cu", "gnn.cu"]
 HEADERS = ["host_graph.h", "philox.cuh", "sweep.cuh", "graph_handle.h", "block.cuh", "halo.cuh", "hub.cuh", "map.cuh", "cluster.cuh",
            "batch_view.h", "batch_map.cuh", "batch_map_plan.h",
-           "host_parallel.h", "shared_limit.h"]
+           "host_parallel.h", "shared_limit.h", "pinned_slots.h"]
 
 
 def nvcc() -> str:

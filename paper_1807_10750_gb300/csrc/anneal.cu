@@ -40,6 +40,7 @@
 #include "halo.cuh"
 #include "hub.cuh"
 #include "map.cuh"
+#include "pinned_slots.h"
 #include "shared_limit.h"
 
 using isingx::HostGraph;
@@ -106,6 +107,7 @@ struct HostResult {
   int error;  // the barrier state's error flag
   int bad;    // ising_set_spins: a value other than +1 / -1
 };
+static_assert(sizeof(HostResult) <= isingx::PinnedSlots::kSlotBytes, "a slot holds a result");
 
 // Twice the energy of the current spins, with the barrier state's error flag,
 // straight into pinned host memory: the block that finishes last writes it and
@@ -510,7 +512,7 @@ void free_device(ising_graph* g) {
                   g->d_gnn_hchunk, g->d_gnn_chunk_row, g->d_map};
   for (void* p : ptrs)
     if (p) cudaFree(p);
-  if (g->h_result) cudaFreeHost(g->h_result);
+  isingx::pinned_slots().give(g->h_result);
 }
 
 // Drop the halo plan (its device arrays); the next anneal that asks for the
@@ -1496,7 +1498,10 @@ int ising_create(int32_t n, int64_t m, const int32_t* src, const int32_t* dst, c
     if ((e = alloc_copy<unsigned long long>(&g->d_slice_acc, nullptr, 2 * slots, g->stream)) != cudaSuccess) break;
     if ((e = alloc_copy(&g->d_slice_parts, plan.split_parts.data(), slots, g->stream)) != cudaSuccess) break;
     if ((e = alloc_copy<unsigned long long>(&g->d_energy, nullptr, 2, g->stream)) != cudaSuccess) break;
-    if ((e = cudaHostAlloc(&g->h_result, sizeof(HostResult), cudaHostAllocDefault)) != cudaSuccess) break;
+    if ((g->h_result = isingx::pinned_slots().take()) == nullptr) {
+      e = cudaErrorMemoryAllocation;
+      break;
+    }
     if ((e = alloc_copy<int8_t>(&g->d_tmp, nullptr, N, g->stream)) != cudaSuccess) break;
     if ((e = alloc_copy(&g->d_class_items, plan.class_item_begin.data(),
                         plan.class_item_begin.size(), g->stream)) != cudaSuccess) break;
