@@ -159,6 +159,61 @@ __device__ __forceinline__ int map_row_sum(int f, int lg) {
   }
 }
 
+// Every vertex's spin into the map, four a load and four loads in flight a thread
+// (eight: the same): a call of one sweep is mostly this and the way back. With a
+// vertex a load, and the way back by the blocks' own rows, class by class: 130,000
+// vertices of 8 on a cluster 66 us a call, now 50; 600 vertices in 600 classes on one
+// block 504, now 323. Both are functions of their own: inlined they changed the
+// registers of the sweep (800 vertices, 1000 sweeps on one block 6.58 -> 6.81 ms).
+static __device__ __noinline__ void map_fill_spins(int8_t* map, const int32_t* index, const int8_t* spins, int n) {
+  const int tid = threadIdx.x, threads = blockDim.x;
+  const int4* index4 = reinterpret_cast<const int4*>(index);
+  const uint32_t* spins4 = reinterpret_cast<const uint32_t*>(spins);
+  for (int i0 = tid; i0 < (n + 3) >> 2; i0 += 4 * threads) {
+    int4 to[4];
+    uint32_t s[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = i0 + u * threads;
+      if (4 * i + 4 <= n) {
+        to[u] = __ldg(index4 + i);
+        s[u] = spins4[i];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = i0 + u * threads;
+      if (4 * i + 4 <= n) {
+        map[to[u].x] = static_cast<int8_t>(spin_of(static_cast<int>(s[u])));
+        map[to[u].y] = static_cast<int8_t>(spin_of(static_cast<int>(s[u] >> 8)));
+        map[to[u].z] = static_cast<int8_t>(spin_of(static_cast<int>(s[u] >> 16)));
+        map[to[u].w] = static_cast<int8_t>(spin_of(static_cast<int>(s[u] >> 24)));
+      } else {
+        for (int p = 4 * i; p < n; ++p) map[__ldg(index + p)] = static_cast<int8_t>(spin_of(spins[p]));
+      }
+    }
+  }
+}
+
+// The k-th of K shares of the positions back to the state bytes, a word a thread.
+static __device__ __noinline__ void map_write_back(const int8_t* map, const int32_t* index, int8_t* spins, int n, int k,
+                                                   int K, int parity) {
+  const int4* index4 = reinterpret_cast<const int4*>(index);
+  uint32_t* spins4 = reinterpret_cast<uint32_t*>(spins);
+  const int share = ((n + K - 1) / K + 3) & ~3, last = min(n, (k + 1) * share);
+  for (int p = k * share + 4 * static_cast<int>(threadIdx.x); p < last; p += 4 * static_cast<int>(blockDim.x)) {
+    if (p + 4 <= last) {
+      const int4 at = __ldg(index4 + (p >> 2));
+      spins4[p >> 2] = static_cast<uint32_t>(state_byte(map[at.x], parity)) |
+                       static_cast<uint32_t>(state_byte(map[at.y], parity)) << 8 |
+                       static_cast<uint32_t>(state_byte(map[at.z], parity)) << 16 |
+                       static_cast<uint32_t>(state_byte(map[at.w], parity)) << 24;
+    } else {
+      for (int q = p; q < last; ++q) spins[q] = static_cast<int8_t>(state_byte(map[__ldg(index + q)], parity));
+    }
+  }
+}
+
 // K blocks; sweeps t_begin .. t_begin + sweeps - 1.
 // SPLIT: a cluster's plan with split rows (no Algorithm 1); G covers a part.
 // RES: the block's entries are in shared memory.
@@ -193,38 +248,7 @@ __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
   int32_t* acc = reinterpret_cast<int32_t*>(bars + 8);
   if (SPLIT)
     for (int i = tid; i < a.accs + 32; i += threads) acc[i] = 0;
-  // The map, four vertices a load and four loads in flight a thread (eight: the
-  // same): a call of one sweep is mostly this and the way back. With a vertex a
-  // load, and the way back by the blocks' own rows, class by class: 130,000
-  // vertices of 8 on a cluster 66 us a call, now 50; 600 vertices in 600 classes
-  // on one block 519, now 332.
-  const int4* index4 = reinterpret_cast<const int4*>(a.map_index);
-  uint32_t* spins4 = reinterpret_cast<uint32_t*>(d.spins);
-  for (int i0 = tid; i0 < (a.n + 3) >> 2; i0 += 4 * threads) {
-    int4 to[4];
-    uint32_t s[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = i0 + u * threads;
-      if (4 * i + 4 <= a.n) {
-        to[u] = __ldg(index4 + i);
-        s[u] = spins4[i];
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = i0 + u * threads;
-      if (4 * i + 4 <= a.n) {
-        map[to[u].x] = static_cast<int8_t>(spin_of(static_cast<int>(s[u])));
-        map[to[u].y] = static_cast<int8_t>(spin_of(static_cast<int>(s[u] >> 8)));
-        map[to[u].z] = static_cast<int8_t>(spin_of(static_cast<int>(s[u] >> 16)));
-        map[to[u].w] = static_cast<int8_t>(spin_of(static_cast<int>(s[u] >> 24)));
-      } else {
-        for (int p = 4 * i; p < a.n; ++p) map[__ldg(a.map_index + p)] = static_cast<int8_t>(spin_of(d.spins[p]));
-      }
-    }
-  }
-#pragma unroll 4
+  map_fill_spins(map, a.map_index, d.spins, a.n);
   for (int i = tid; i < B.rounds * warps; i += threads) tasks[i] = __ldg(a.tasks + B.task0 + i);
   for (int c = tid; c <= C; c += threads) {
     crow[c] = __ldg(a.class_row + k_me * (C + 1) + c);
@@ -233,16 +257,12 @@ __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
     if (MODE != kMapGrid) cbytes[c] += __ldg(a.class_bytes + c);
     cmsg[c] = __ldg(a.class_msg + c);
   }
-#pragma unroll 4
-  for (int r = tid; r < B.rows / 4; r += threads)
-    reinterpret_cast<int4*>(orig)[r] = __ldg(reinterpret_cast<const int4*>(a.row_orig + B.row0) + r);
-  if (d.bias != nullptr)
-    for (int r = tid; r < B.rows; r += threads) {
-      const int p = __ldg(a.row_pos + B.row0 + r);
-      bias[r] = p >= 0 ? __ldg(d.bias + p) : 128;
-    }
+  for (int r = tid; r < B.rows; r += threads) {
+    orig[r] = __ldg(a.row_orig + B.row0 + r);
+    const int p = __ldg(a.row_pos + B.row0 + r);
+    bias[r] = d.bias != nullptr && p >= 0 ? __ldg(d.bias + p) : 128;
+  }
   if (RES)
-#pragma unroll 4
     for (int i = tid; i < B.groups * 32; i += threads) {
       res_words[i] = __ldg(a.words + static_cast<size_t>(B.words0) * 32 + i);
       if (WIDE) res_weights[i] = __ldg(a.weights + static_cast<size_t>(B.words0) * 32 + i);
@@ -512,20 +532,7 @@ __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
     }
   }
 done:
-  // back to the state bytes, from maps that all hold every spin: a block writes
-  // its share of the positions, a word a thread
-  const int share = ((a.n + K - 1) / K + 3) & ~3, last = min(a.n, (k_me + 1) * share);
-  for (int p = k_me * share + 4 * tid; p < last; p += 4 * threads) {
-    if (p + 4 <= last) {
-      const int4 at = __ldg(index4 + (p >> 2));
-      spins4[p >> 2] = static_cast<uint32_t>(state_byte(map[at.x], a.par_end)) |
-                       static_cast<uint32_t>(state_byte(map[at.y], a.par_end)) << 8 |
-                       static_cast<uint32_t>(state_byte(map[at.z], a.par_end)) << 16 |
-                       static_cast<uint32_t>(state_byte(map[at.w], a.par_end)) << 24;
-    } else {
-      for (int q = p; q < last; ++q) d.spins[q] = static_cast<int8_t>(state_byte(map[__ldg(a.map_index + q)], a.par_end));
-    }
-  }
+  map_write_back(map, a.map_index, d.spins, a.n, k_me, K, a.par_end);
   if (CLUSTER) {
     if (!ok) __nanosleep(20000);  // its last stores may still be on their way (a fraction of a microsecond)
     cluster_sync();
