@@ -431,7 +431,7 @@ uint64_t batch_t0(double p0) {
 
 constexpr int kBlockChoices[3] = {128, 256, 512};
 constexpr int kBlockDefault = 256;
-constexpr int kPackedSpins = 6144;  // ising_batch_get_spins: instances up to this size by their packed bytes
+constexpr int kPackedSpins = 1024;  // ising_batch_get_spins: instances up to this size by their packed bytes
 constexpr int kSplitChoices[3] = {1, 2, 4};
 constexpr int kTailChoices[2] = {0, 32};
 constexpr int kBatchError = 15;  // d_work: work queue heads, then the clustered form's error flag
@@ -1182,8 +1182,9 @@ int ising_batch_get_spins(ising_batch* b, int32_t graph, uint32_t replica, int8_
   const int32_t nn = b->n[(size_t)graph];
   // Through pinned memory, in one copy: the packed bytes, decoded here, of a small
   // instance (no kernel to wait for), the spins decoded on the device of a large
-  // one. Microseconds a call, packed / decoded: 100 vertices 15.5 / 21, 5,000 20 / 22,
-  // 10,000 39 / 23, 60,000 252 / 27.
+  // one. Microseconds a call, packed / decoded, one read of each of 320 instances (so
+  // that the host's tables are in no cache): up to 1024 vertices 15.6 / 17.9, 1024 to 6144
+  // 23.5 / 17.1; one instance again and again: 100 vertices 15.5 / 21, 5,000 20 / 22.
   const bool packed = nn <= kPackedSpins;
   if (b->h_out == nullptr || (b->d_out == nullptr && !packed)) {
     const size_t bytes = static_cast<size_t>(b->max_n) + 1;
