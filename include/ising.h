@@ -406,8 +406,8 @@ int ising_batch_set_tuning(ising_batch* b, int32_t block, int32_t row_split, int
 int ising_batch_tuning(ising_batch* b, int32_t* out_block, int32_t* out_row_split, int32_t* out_tail,
                        float* out_probe_ms);
 /* ising_batch_debug_fault -- failure-detection test hook, as ising_debug_fault:
- * ISING_FAULT_SKIP_ARRIVAL keeps the first block of every cluster from sending
- * its spins, so that the clustered form's waits run out; wait_budget_ns bounds
+ * ISING_FAULT_SKIP_ARRIVAL lets every block of a cluster wait for four bytes
+ * that nobody sends, so that the clustered form's waits run out; wait_budget_ns bounds
  * every wait of later anneals (0: the default, 2 s; at most 60 s). The next call
  * that synchronises reports ISING_ETIMEOUT and latches it in the batch: cuts,
  * get / set spins, autotune, and the warm-start network's calls on the batch (a

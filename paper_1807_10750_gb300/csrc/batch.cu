@@ -454,6 +454,8 @@ struct BatchMapGroup {
   isingx::BatchMapInst* inst = nullptr;
   isingx::BatchMapUnit* units = nullptr;
   int32_t *block_unit = nullptr, *class_unit = nullptr, *class_bytes = nullptr;
+  int32_t num_class_bytes = 0;
+  int32_t* missing_bytes = nullptr;  // ising_batch_debug_fault: class_bytes, and four that nobody sends
   int32_t *dst = nullptr, *row_sum = nullptr, *map_index = nullptr;
   int4* words = nullptr;
 };
@@ -531,7 +533,8 @@ namespace {
 void group_free(BatchMapGroup& g) {
   if (g.stream) cudaStreamDestroy(g.stream);
   if (g.join) cudaEventDestroy(g.join);
-  void* ptrs[] = {g.inst, g.units, g.block_unit, g.class_unit, g.class_bytes, g.dst, g.row_sum, g.map_index, g.words, g.order};
+  void* ptrs[] = {g.inst, g.units, g.block_unit, g.class_unit, g.class_bytes, g.dst, g.row_sum, g.map_index, g.words, g.order,
+                  g.missing_bytes};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   g = BatchMapGroup();
@@ -675,6 +678,7 @@ cudaError_t group_upload(ising_batch* b, const isingx::BatchMapPlan& p, const in
   g->map_bytes = p.map_bytes;
   g->units_max = p.units_max;
   g->classes_max = p.classes_max;
+  g->num_class_bytes = static_cast<int32_t>(p.class_bytes.size());
   cudaError_t e;
   int32_t* d_unit_inst = nullptr;
   do {
@@ -833,7 +837,7 @@ int groups_launch(ising_batch* b, uint64_t t_begin, uint32_t sweeps, uint64_t T,
     a.block_unit = g.block_unit;
     a.units = reinterpret_cast<const int4*>(g.units);
     a.class_unit = g.class_unit;
-    a.class_bytes = g.class_bytes;
+    a.class_bytes = b->fault_kind == ISING_FAULT_SKIP_ARRIVAL ? g.missing_bytes : g.class_bytes;
     a.dst = g.dst;
     a.row_sum = g.row_sum;
     a.map_index = g.map_index;
@@ -848,7 +852,6 @@ int groups_launch(ising_batch* b, uint64_t t_begin, uint32_t sweeps, uint64_t T,
     a.units_max = g.units_max;
     a.classes_max = g.classes_max;
     a.budget = b->wait_budget_ns > 0 ? static_cast<long long>(b->wait_budget_ns) : isingx::kBarrierBudgetNs;
-    a.silent = b->fault_kind == ISING_FAULT_SKIP_ARRIVAL ? 1 : 0;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
     batch_map_config(&cfg, &attr, g.K, g.clusters, g.smem, s);
@@ -1307,6 +1310,24 @@ int ising_batch_debug_fault(ising_batch* b, int kind, uint64_t wait_budget_ns) {
   if (b == nullptr) return ISING_EINVAL;
   if (kind != ISING_FAULT_NONE && kind != ISING_FAULT_SKIP_ARRIVAL) return ISING_EINVAL;
   if (wait_budget_ns > 60000000000ull) return ISING_EINVAL;
+  const int rc = batch_enter(b);
+  if (rc != ISING_OK) return rc;
+  // a table for the tests: the kernel has no switch for them (one add where it
+  // reads the table cost 2 % of a sweep)
+  for (BatchMapGroup& g : b->groups) {
+    if (kind == ISING_FAULT_NONE || g.one_block || g.missing_bytes != nullptr) continue;
+    try {
+      std::vector<int32_t> bytes(static_cast<size_t>(g.num_class_bytes));
+      BATCH_CUDA(b, cudaMemcpyAsync(bytes.data(), g.class_bytes, bytes.size() * sizeof(int32_t), cudaMemcpyDeviceToHost,
+                                    b->stream));
+      BATCH_CUDA(b, cudaStreamSynchronize(b->stream));
+      for (int32_t& x : bytes) x += 4;
+      BATCH_CUDA(b, upload(&g.missing_bytes, bytes, b->stream));
+      BATCH_CUDA(b, cudaStreamSynchronize(b->stream));
+    } catch (const std::bad_alloc&) {
+      return ISING_ENOMEM;
+    }
+  }
   b->fault_kind = kind;
   b->wait_budget_ns = wait_budget_ns;
   return ISING_OK;

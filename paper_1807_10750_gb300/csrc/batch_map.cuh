@@ -56,7 +56,6 @@ struct BatchMapArgs {
   int32_t num_graphs, K, replicas;
   int32_t map_bytes, units_max, classes_max;  // of the largest instance
   long long budget;
-  int silent;  // failure-detection tests: the clusters' first blocks send nothing
 };
 
 // All ones if the low byte of x is negative, else 0.
@@ -218,7 +217,6 @@ __global__ void __launch_bounds__(kBatchMapThreads, 2)
   int* slot_now = reinterpret_cast<int*>(drawn + 1);
   const uint32_t bar = smem_u32(bars);
   const uint32_t dst_lane = lane & 3;
-  const uint32_t receivers = a.silent != 0 && k_me == 0 ? 0u : static_cast<uint32_t>(K);
   if (CLUSTER) {
     if (tid == 0) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(U) : "memory");
@@ -414,7 +412,7 @@ __global__ void __launch_bounds__(kBatchMapThreads, 2)
             word |= __shfl_xor_sync(kFullMask, word, 1);
             word |= __shfl_xor_sync(kFullMask, word, 2);
             const uint32_t to = smem_u32(map + u.y) + (lane & 28), on = bar + 8 * (step & 1u);
-            for (uint32_t b = dst_lane; b < receivers && ok; b += 4)
+            for (uint32_t b = dst_lane; b < static_cast<uint32_t>(K) && ok; b += 4)
               asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(
                                cluster_addr(to, b)),
                            "r"(word), "r"(cluster_addr(on, b))

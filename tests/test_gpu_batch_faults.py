@@ -1,5 +1,5 @@
-"""A clustered batch anneal whose waits run out (the first block of every cluster
-sends nothing) is reported by whichever call synchronises next, the network's
+"""A clustered batch anneal whose waits run out (every block of a cluster waits for
+bytes that nobody sends) is reported by whichever call synchronises next, the network's
 included, and latched in the batch; a train step on such spins leaves the weights."""
 
 import numpy as np
