@@ -1155,11 +1155,7 @@ cudaError_t launch_map(ising_graph* g, uint64_t t_begin, uint32_t sweeps, uint64
                        uint32_t replica, const isingx::PhiloxRounds& rk, uint32_t n0, int par0) {
   const bool wide = !g->packed;
   const void* kernel = map_kernel_for(g->map_mode, wide, g->map_stage, g->map_accs > 0, g->map_resident);
-  cudaError_t e = isingx::allow_shared(kernel, g->device, static_cast<size_t>(g->map_smem));
-  if (e != cudaSuccess) return e;
-  if (g->map_mode == isingx::kMapCluster &&
-      (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
-    return e;
+  cudaError_t e = cudaSuccess;  // (map_fits has allowed the kernel its shared memory and its cluster)
   isingx::MapArgs a{};
   a.blocks = g->d_map_blocks;
   a.tasks = reinterpret_cast<const int4*>(g->d_map_task);

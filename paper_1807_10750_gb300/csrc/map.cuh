@@ -169,13 +169,14 @@ static __device__ __noinline__ void map_fill_spins(int8_t* map, const int32_t* i
   const int tid = threadIdx.x, threads = blockDim.x;
   const int4* index4 = reinterpret_cast<const int4*>(index);
   const uint32_t* spins4 = reinterpret_cast<const uint32_t*>(spins);
-  for (int i0 = tid; i0 < (n + 3) >> 2; i0 += 4 * threads) {
+  if (tid < (n & 3)) map[__ldg(index + (n & ~3) + tid)] = static_cast<int8_t>(spin_of(spins[(n & ~3) + tid]));
+  for (int i0 = tid; i0 < n >> 2; i0 += 4 * threads) {
     int4 to[4];
     uint32_t s[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int i = i0 + u * threads;
-      if (4 * i + 4 <= n) {
+      if (i < n >> 2) {
         to[u] = __ldg(index4 + i);
         s[u] = spins4[i];
       }
@@ -183,13 +184,11 @@ static __device__ __noinline__ void map_fill_spins(int8_t* map, const int32_t* i
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int i = i0 + u * threads;
-      if (4 * i + 4 <= n) {
+      if (i < n >> 2) {
         map[to[u].x] = static_cast<int8_t>(spin_of(static_cast<int>(s[u])));
         map[to[u].y] = static_cast<int8_t>(spin_of(static_cast<int>(s[u] >> 8)));
         map[to[u].z] = static_cast<int8_t>(spin_of(static_cast<int>(s[u] >> 16)));
         map[to[u].w] = static_cast<int8_t>(spin_of(static_cast<int>(s[u] >> 24)));
-      } else {
-        for (int p = 4 * i; p < n; ++p) map[__ldg(index + p)] = static_cast<int8_t>(spin_of(spins[p]));
       }
     }
   }
@@ -200,17 +199,15 @@ static __device__ __noinline__ void map_write_back(const int8_t* map, const int3
                                                    int K, int parity) {
   const int4* index4 = reinterpret_cast<const int4*>(index);
   uint32_t* spins4 = reinterpret_cast<uint32_t*>(spins);
-  const int share = ((n + K - 1) / K + 3) & ~3, last = min(n, (k + 1) * share);
-  for (int p = k * share + 4 * static_cast<int>(threadIdx.x); p < last; p += 4 * static_cast<int>(blockDim.x)) {
-    if (p + 4 <= last) {
-      const int4 at = __ldg(index4 + (p >> 2));
-      spins4[p >> 2] = static_cast<uint32_t>(state_byte(map[at.x], parity)) |
-                       static_cast<uint32_t>(state_byte(map[at.y], parity)) << 8 |
-                       static_cast<uint32_t>(state_byte(map[at.z], parity)) << 16 |
-                       static_cast<uint32_t>(state_byte(map[at.w], parity)) << 24;
-    } else {
-      for (int q = p; q < last; ++q) spins[q] = static_cast<int8_t>(state_byte(map[__ldg(index + q)], parity));
-    }
+  const int tid = threadIdx.x, words = n >> 2, share = (words + K - 1) / K, last = min(words, (k + 1) * share);
+  const int rest = (n & ~3) + tid;
+  if (k == K - 1 && rest < n) spins[rest] = static_cast<int8_t>(state_byte(map[__ldg(index + rest)], parity));
+  for (int i = k * share + tid; i < last; i += static_cast<int>(blockDim.x)) {
+    const int4 at = __ldg(index4 + i);
+    spins4[i] = static_cast<uint32_t>(state_byte(map[at.x], parity)) |
+                static_cast<uint32_t>(state_byte(map[at.y], parity)) << 8 |
+                static_cast<uint32_t>(state_byte(map[at.z], parity)) << 16 |
+                static_cast<uint32_t>(state_byte(map[at.w], parity)) << 24;
   }
 }
 
@@ -248,7 +245,11 @@ __global__ void __launch_bounds__(32 * kMapMaxWarps, 1)
   int32_t* acc = reinterpret_cast<int32_t*>(bars + 8);
   if (SPLIT)
     for (int i = tid; i < a.accs + 32; i += threads) acc[i] = 0;
-  map_fill_spins(map, a.map_index, d.spins, a.n);
+  if (MODE <= kMapBlockStream) {  // few vertices: a call would wait for its loads before the next ones start
+    for (int p = tid; p < a.n; p += threads) map[__ldg(a.map_index + p)] = static_cast<int8_t>(spin_of(d.spins[p]));
+  } else {
+    map_fill_spins(map, a.map_index, d.spins, a.n);
+  }
   for (int i = tid; i < B.rounds * warps; i += threads) tasks[i] = __ldg(a.tasks + B.task0 + i);
   for (int c = tid; c <= C; c += threads) {
     crow[c] = __ldg(a.class_row + k_me * (C + 1) + c);

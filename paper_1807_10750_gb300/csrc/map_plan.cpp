@@ -31,8 +31,11 @@ void build_map_plan(const HostGraph& g, int32_t mode, int32_t K, bool wide, int6
       K > kMapMaxBlocks || (mode <= kMapBlockStream && K != 1) || (mode == kMapCluster && (K > 16 || (K & (K - 1)) != 0)) ||
       (split && mode != kMapCluster))
     return;
-  // a block holds the map, and an id and a bias byte for its share of the rows
-  if (g.n + g.n / K * int64_t(5) > smem_limit) return;
+  // At the least a block holds the map, an id and a bias byte for its share of the
+  // rows, and for every class a round of eight tasks and its tables; but for the
+  // grid it has a unit in every class, padded to 32 rows of 5.25 bytes.
+  const int64_t rows_bytes = std::max<int64_t>(g.n / K * int64_t(5), mode != kMapGrid ? int64_t(168) * C : 0);
+  if (g.n + rows_bytes + int64_t(128 + 16) * C > smem_limit) return;
   const bool cluster = mode == kMapCluster;
   const size_t stride = static_cast<size_t>(C) + 1;
   // a unit's rows in the block's row order: whole aligned words of the map
