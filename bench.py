@@ -99,10 +99,10 @@ def algorithmic_bytes_per_sweep(n: int, nnz: int, entry_bytes: int) -> int:
 # the sweeps. The entry holds only while the kernel sources hash to `sources`:
 # once they change the counters are stale and traffic is reported as null.
 NCU_TRAFFIC = {
-    "zipf1m": {"fixed": 97.6e6, "per_sweep": 12.38e6, "kernel": "hub_kernel", "engine": "hub",
+    "zipf1m": {"fixed": 98.5e6, "per_sweep": 12.30e6, "kernel": "hub_kernel", "engine": "hub",
                "files": ('hub.cuh', 'sweep.cuh', 'philox.cuh', 'anneal.cu'),
-               "sources": "3984244a39941fb0",
-               "how": "ncu 4- and 12-sweep captures: 147.13 MB and 246.21 MB (read + write); the "
+               "sources": "7704eef2e728c014",
+               "how": "ncu 4- and 12-sweep captures: 147.69 MB and 246.09 MB (read + write); the "
                       "CSR is read from DRAM once and then mostly served from L2"},
     "torus1024": {"fixed": 31.80e6, "per_sweep": 3.32e3, "kernel": "halo_kernel",
                   "engine": "halo",
@@ -110,10 +110,12 @@ NCU_TRAFFIC = {
                   "sources": "aa10d359c3f8355f",
                   "how": "ncu 20- and 40-sweep captures: 31.869 MB and 31.936 MB, so the "
                          "working set is read once and then stays in shared memory and L2"},
-    "batched": {"fixed": 0.2490e9, "per_sweep": 0.1997e9, "kernel": "batch_map_kernel",
-                "files": ('batch.cu', 'batch_map.cuh', 'cluster.cuh', 'philox.cuh'),
-                "sources": "0a8224281505d3a7",
-                "how": "ncu 20- and 60-sweep captures: 4.243 GB and 12.231 GB"},
+    "batched": {"fixed": 0.1937e9, "per_sweep": 0.2003e9, "kernel": "batch_map_kernel",
+                "engine": "clustered",
+                "files": ('batch.cu', 'batch_map.cuh', 'batch_map_plan.cpp', 'batch_map_plan.h', 'cluster.cuh', 'host_graph.cpp',
+                          'philox.cuh'),
+                "sources": "0c9fabebb62a1690",
+                "how": "ncu 20- and 60-sweep captures: 4.199 GB and 12.210 GB"},
 }
 
 
@@ -354,6 +356,8 @@ def run_batched(args, world, rank, P, torch, dist):
             anneal_ms.append(ev[0].elapsed_time(ev[1]))
             best.append(float(cuts.max(axis=1).sum()))
     launches = P.ising_batch_info(b)["launches"] - launches0
+    on_blocks = P.ising_batch_debug_form(b)  # instances on the one-block kernel, on clusters of 1, 2, 4, 8, 16 blocks
+    form = "one_block" if on_blocks[0] == len(gs) else "clustered" if on_blocks[0] == 0 else "mixed"
     total_ms = sum(s_.elapsed_time(e_) for s_, e_ in zip(starts, ends))
     total_ms = max_over_ranks(total_ms, world, dist, "cuda")
     value = job_throughput(nvert * R * T * args.steps, world, total_ms / 1e3)
@@ -369,7 +373,8 @@ def run_batched(args, world, rank, P, torch, dist):
         for k in range(args.e2e_steps + 1):
             t0 = time.perf_counter()
             with P.ising_batch_create(arrays, replicas=R, stream=stream) as b2:
-                P.ising_batch_set_tuning(b2, tuning["block"], tuning["row_split"], tuning["tail"])
+                if form == "one_block":  # else the tuner kept what a batch does without a tuning
+                    P.ising_batch_set_tuning(b2, tuning["block"], tuning["row_split"], tuning["tail"])
                 P.ising_batch_init_random(b2, seed + k)
                 P.ising_batch_anneal(b2, p0=p0, t_total=T, seed=seed + k, stream=stream)
                 P.ising_batch_cuts(b2)
@@ -391,7 +396,7 @@ def run_batched(args, world, rank, P, torch, dist):
         "config": {"workload": "batched", "instances": len(gs), "vertices": nvert,
                    "edges": nnz // 2, "replicas": R, "sweeps": T, "p0": p0, "block": block,
                    "tuning": {"block": tuning["block"], "row_split": tuning["row_split"],
-                              "tail": tuning["tail"],
+                              "tail": tuning["tail"], "form": form, "instances_on_blocks": on_blocks,
                               "probe_ms_20_sweeps": [round(x, 3) for x in tuning["probe_ms"]],
                               "probe_order": "6 * block(128,256,512) + 2 * row_split(1,2,4) + tail(0,32)"},
                    "parallelism": f"replicas{world}",
@@ -399,9 +404,10 @@ def run_batched(args, world, rank, P, torch, dist):
         "sweeps_per_s": T * args.steps * world / (total_ms / 1e3),
         "best_cut_sum_mean": float(np.mean(best)),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                     "frac": achieved / peak, "traffic": kernel_traffic("batched", T),
+                     "frac": achieved / peak, "traffic": kernel_traffic("batched", T, form),
                      "peak_kind": peak_kind, "bytes_per_sweep": B, "bytes_per_launch": B * T,
-                     "kernel": "batch_map_kernel (clusters by instance size) or, where tuned so, batch_anneal_kernel"},
+                     "kernel": {"one_block": "batch_anneal_kernel", "clustered": "batch_map_kernel",
+                                "mixed": "batch_map_kernel and batch_anneal_kernel"}[form]},
         "cpu_baseline": None, "e2e": e2e, "gpu_launches": int(launches), "clocks": clocks.summary(),
     }
     print(json.dumps(line), flush=True)
@@ -594,19 +600,17 @@ def run_warmstart(args, world, rank, P, torch, dist):
 
 def gnn_forward_bytes(n: int, nnz: int) -> int:
     """Algorithmic bytes of one forward pass of the warm-start network: row
-    sums (CSR word, row id, neighbour spin per entry; an int4 per row out, as
-    the form this figure began with; the current one needs neither id nor
-    int4), features (sums, spin in; 8 bf16 features and c out), three layers (per
+    sums and features (CSR word and neighbour spin per entry; per row its bounds
+    and spin in, 8 bf16 features and c out), three layers (per
     entry the CSR word, c_j and the neighbour's bf16 feature row; per row its
     row bounds, c, its own row in and its 64-wide bf16 output) and the head
     (h3 in, z out). The aggregate a never leaves the layer kernel, so it
     moves no bytes."""
-    rowsum = nnz * 9 + n * 16
-    feats = n * (16 + 1 + 16 + 4)
+    feats = nnz * (4 + 1) + n * (4 + 1 + 16 + 4)
     layer8 = nnz * (8 + 16) + n * (12 + 16 + 128)
     layer64 = nnz * (8 + 128) + n * (12 + 128 + 128)
     head = n * (128 + 4)
-    return rowsum + feats + layer8 + 2 * layer64 + head
+    return feats + layer8 + 2 * layer64 + head
 
 
 def run_gnn(args, world, rank, P, torch, dist):
