@@ -129,10 +129,11 @@ enum {
                                   (per-item counters, release/acquire); for graphs whose rows
                                   are not sliced across warps, deterministic linear schedule;
                                   otherwise runs as PERSISTENT_GRID. Such graphs of up to 204,800
-                                  vertices run in the spin-map form instead where it is faster (not lattices
-                                  larger than 100,000 vertices or 37,500 a colour, nor graphs
-                                  above about 165,000 vertices of fewer than 4.5 neighbours; a call of
-                                  one sweep may run as PERSISTENT_GRID) */
+                                  vertices run in the spin-map form instead where it is
+                                  faster (not lattices larger than 100,000 vertices or
+                                  37,500 a colour, nor graphs above about 165,000 vertices
+                                  of fewer than 4.5 neighbours; a call of one sweep may run
+                                  as PERSISTENT_GRID) */
   ISING_ENGINE_HALO = 7,       /* one cooperative launch per anneal call, one block per SM: the
                                   graph is cut into one part per block (recursive breadth-first
                                   bisection); a block keeps every vertex within D = S * K hops of
@@ -351,8 +352,9 @@ int ising_plan_halo(int32_t n, int64_t m, const int32_t* src, const int32_t* dst
  *
  * Batches whose rows have at most 63 entries and whose weights are at most 31
  * in magnitude run with each instance on one block or on the blocks of a
- * cluster, by its size, unless a tuning is set; others, and batches with a
- * tuning set, run one block per instance.
+ * cluster, by its size, unless a tuning is set; others, batches with a tuning
+ * set, and more small instances than the SMs hold at once in that form, run on
+ * a kernel of one block per instance.
  * ------------------------------------------------------------------------ */
 typedef struct ising_batch ising_batch; /* opaque */
 
@@ -416,7 +418,8 @@ int ising_batch_tuning(ising_batch* b, int32_t* out_block, int32_t* out_row_spli
 int ising_batch_debug_fault(ising_batch* b, int kind, uint64_t wait_budget_ns);
 /* ising_batch_debug_form -- a diagnostic, as ising_debug_form: how many instances
  * the last anneal ran on the one-block kernel (out_instances[0], -1 before the
- * first anneal) and in the clustered form on 1, 2, 4, 8 and 16 blocks (entries 1 to 5). */
+ * first anneal) and in the clustered form on 1, 2, 4, 8 and 16 blocks (entries
+ * 1 to 5). */
 int ising_batch_debug_form(ising_batch* b, int32_t* out_instances);
 /* ising_batch_info -- instances, total vertices, block size, kernel launches. */
 int ising_batch_info(ising_batch* b, int32_t* out_num_graphs, int64_t* out_vertices,
@@ -580,10 +583,10 @@ void ising_gnn_destroy(ising_gnn* net);
 #define ISING_ENGINE_USED_BLOCK 6
 int ising_engine_used(ising_graph* g, int32_t* out);
 
-/* ising_debug_form -- a diagnostic of tests and benchmarks: the kernel that the last anneal call's last
- * launch ran, which ising_engine_used does not tell (the spin-map forms stand
- * in for several engines), and the blocks that share the graph (0 for
- * ISING_FORM_ENGINE). -1 before the first anneal. Any pointer may be NULL. */
+/* ising_debug_form -- a diagnostic of tests and benchmarks: the form of the last
+ * anneal call's last launch, which ising_engine_used does not tell (the spin-map
+ * forms stand in for several engines), and the blocks that share the graph (0
+ * for ISING_FORM_ENGINE). -1 before the first anneal. Any pointer may be NULL. */
 enum {
   ISING_FORM_ENGINE = 0,           /* the engine's own kernel */
   ISING_FORM_MAP_BLOCK = 1,        /* spin map: one block, entries in shared memory */
